@@ -595,19 +595,6 @@ __device__ void coarse_passes(int nv, const TT* cbox, TT* tile, TT* scr, const P
   g.sync();
 }
 
-// Value of a ghost node predicted from the coarse box after coarse_passes: the
-// last axis (z in 3D, y in 2D) from the scratch.
-template <int D, int B, int W, typename TT>
-__device__ __forceinline__ TT coarse_predicted(const TT* scr_v, int i, int j, int k) {
-  using Bx = Box<D, B, W>;
-  const TT* c = scr_v + (i + W) + (D == 3 ? (j + W) * Bx::S : 0);
-  constexpr int st = D == 3 ? Bx::S * Bx::S : Bx::S;
-  const int e = D == 3 ? k : j, fl = e >> 1;
-  return (e & 1) ? dd4(c[(fl - 1 - Bx::CLO) * st], c[(fl - Bx::CLO) * st], c[(fl + 1 - Bx::CLO) * st],
-                       c[(fl + 2 - Bx::CLO) * st])
-                 : c[(fl - Bx::CLO) * st];
-}
-
 // Fills the synchronised tile (nvar x T^d, type TT) of block b from field F.
 // Block-edge nodes owned by another block (a finer one, Sec. 2.2 rule 2, or an
 // equal-level one that holds the node at its lower edge, which keeps redundant
@@ -832,234 +819,6 @@ __device__ void fill_tile(const PoolView& pv, const BlockInfo& b, const TF* F, T
   }
 }
 
-// Column form of the 3D tile fill for one CTA: each thread fills whole z-columns
-// (fixed x, y) of the tile, with the z loop unrolled, so every quantity that
-// depends on z alone (neighbour index, local offset, class box, inside or
-// ghost) is a compile-time constant and the per-node work is a table lookup,
-// an address and the copy.  Up to KC loads of a column are in flight together.
-// nbase (nullable): pool offsets (slot * nvar * vs) of the 27 equal-level
-// neighbours of a block with a uniform neighbourhood (x fastest, the block
-// itself in the centre); null: the owners come from the ring's class boxes
-// (build_ring must have run).  Same values, stores and commits as fill_tile.
-template <int B, typename TF, typename TT, int W>
-__device__ void fill_cols(const PoolView& pv, const BlockInfo& b, const int64_t* nbase, const TF* F, TF* Fw,
-                          TT* tile, bool commit, RingD<3>& R, TT* cbox, TT* scr, bool have_regions = false) {
-  using Gm = Geo<3, B>;
-  using Bx = Box<3, B, W>;
-  constexpr int S = Bx::S, S2 = S * S, BB = B * B;
-  // same field and tile types: asynchronous copies, all in flight at once
-  constexpr bool ASYNC = std::is_same<TF, TT>::value;
-  constexpr int KC = ASYNC ? 11 : 7;  // nodes per chunk (register loads in flight)
-  const int nv = pv.nvar;
-  const int64_t own = (int64_t)b.slot * nv * pv.vs;
-  const int l1 = b.lvl + 1;
-  const bool uni = nbase != nullptr;
-  auto load_store = [&](auto kcc, const int64_t* at, const int* kind, int col, int i, int j, int kbase) {
-    constexpr int KN = decltype(kcc)::value;
-    if constexpr (ASYNC) {
-      // copies now; block-edge nodes of other owners are committed after the wait
-      for (int v = 0; v < nv; ++v) {
-#pragma unroll
-        for (int u = 0; u < KN; ++u) {
-          const int k = kbase + u;
-          TT* t = tile + v * Bx::TILE + col + (k + W) * S2;
-          if (kind[u] <= 2) cp_async(t, F + at[u] + (int64_t)v * pv.vs);
-          else if (kind[u] == 3) *t = coarse_predicted<3, B, W, TT>(scr + v * Bx::SCR, i, j, k);
-          else *t = TT(0);
-        }
-      }
-      return;
-    }
-    for (int v = 0; v < nv; ++v) {
-      TF val[KN];
-#pragma unroll
-      for (int u = 0; u < KN; ++u) val[u] = kind[u] <= 2 ? F[at[u] + (int64_t)v * pv.vs] : TF(0);
-#pragma unroll
-      for (int u = 0; u < KN; ++u) {
-        const int k = kbase + u;
-        TT* t = tile + v * Bx::TILE + col + (k + W) * S2;
-        if (kind[u] == 3) {
-          *t = coarse_predicted<3, B, W, TT>(scr + v * Bx::SCR, i, j, k);
-        } else if (kind[u] == 4) {
-          *t = TT(0);
-        } else {
-          *t = (TT)val[u];
-          if (kind[u] == 1 && commit) {
-            const int64_t me = own + (int64_t)v * pv.vs + Gm::lin(i, j, k);
-            if (F[me] != val[u]) Fw[me] = val[u];
-          }
-        }
-      }
-    }
-  };
-  if (!uni) {
-    if (!have_regions) {
-      build_regions<3, B, CtaGroup>(b, R);
-      __syncthreads();
-    }
-    if (R.coarser && R.cmask) {
-      // coarse box: columns of CB coarse nodes (coarse node n at level-l node
-      // 2n), where the prediction of the nodes of pb reads them
-      const PredBox<B, W> pb(R.cmask, 3);
-      constexpr int CB = Bx::CB;
-      for (int c = threadIdx.x; c < CB * CB; c += blockDim.x) {
-        const int nx = c % CB + Bx::CLO, ny = c / CB + Bx::CLO;
-        if (nx < pb.nlo[0] || nx > pb.nhi[0] || ny < pb.nlo[1] || ny > pb.nhi[1]) continue;
-        const int rb = reg_class<B>(2 * nx) + 7 * reg_class<B>(2 * ny);
-        // per chunk of the column: addresses first, then the loads, then the stores
-        bool bad = false;
-        auto cchunk = [&](auto knc, auto z0c) {
-          constexpr int KN = decltype(knc)::value, Z0 = decltype(z0c)::value;
-          int64_t at[KN];
-          int good[KN];  // 1 load, 0 not needed, -1 no owner (error)
-#pragma unroll
-          for (int u = 0; u < KN; ++u) {
-            const int nz = Z0 + u + Bx::CLO;
-            at[u] = 0;
-            good[u] = 0;
-            if (nz < pb.nlo[2] || nz > pb.nhi[2]) continue;
-            const int4 e = R.reg[rb + 49 * reg_class<B>(2 * nz)];
-            if (e.x < 0 || e.y < b.lvl - 1) {
-              good[u] = -1;
-              continue;
-            }
-            const int sh = l1 - e.y;
-            const int ox = 4 * nx - (int)(int16_t)(e.z & 0xffff), oy = 4 * ny - (e.z >> 16), oz = 4 * nz - e.w;
-            at[u] = ((int64_t)e.x * nv) * pv.vs + Gm::lin(ox >> sh, oy >> sh, oz >> sh);
-            good[u] = 1;
-          }
-          for (int v = 0; v < nv; ++v) {
-            if constexpr (ASYNC) {
-#pragma unroll
-              for (int u = 0; u < KN; ++u) {
-                TT* t = cbox + v * Bx::CBOX + (Z0 + u) * CB * CB + c;
-                if (good[u] > 0) cp_async(t, F + at[u] + (int64_t)v * pv.vs);
-                else if (good[u] < 0) *t = TT(0);
-                bad |= good[u] < 0;
-              }
-            } else {
-              TF val[KN];
-#pragma unroll
-              for (int u = 0; u < KN; ++u) val[u] = good[u] > 0 ? F[at[u] + (int64_t)v * pv.vs] : TF(0);
-#pragma unroll
-              for (int u = 0; u < KN; ++u) {
-                if (good[u] != 0) cbox[v * Bx::CBOX + (Z0 + u) * CB * CB + c] = good[u] > 0 ? (TT)val[u] : TT(0);
-                bad |= good[u] < 0;
-              }
-            }
-          }
-        };
-        constexpr int ZC = 7;
-        static_for<0, (CB + ZC - 1) / ZC>([&](auto cc) {
-          constexpr int C = decltype(cc)::value;
-          constexpr int KN = (CB - C * ZC) < ZC ? (CB - C * ZC) : ZC;
-          cchunk(std::integral_constant<int, KN>{}, std::integral_constant<int, C * ZC>{});
-        });
-        if (bad) set_err(pv, kErrGraded);
-      }
-      if constexpr (ASYNC) cp_async_wait_all();
-      __syncthreads();
-      if (scr) coarse_passes<3, B, W, TT, CtaGroup>(nv, cbox, tile, scr, pb);
-    }
-  }
-  for (int col = threadIdx.x; col < S2; col += blockDim.x) {
-    const int i = col % S - W, j = col / S - W;
-    const bool inxy = i >= 0 && i <= B - 1 && j >= 0 && j <= B - 1;
-    // strictly inside the block in x and y: with 1 <= k <= Bs - 2 the node is
-    // the block's own (no other leaf contains it), whatever the ring holds
-    const bool core = i >= 1 && i <= B - 2 && j >= 1 && j <= B - 2;
-    // uniform form: neighbour row and local offset of the column
-    const int sx = i < 0 ? 0 : (i <= B - 2 ? 1 : 2), sy = j < 0 ? 0 : (j <= B - 2 ? 1 : 2);
-    const int lxy = (i - (sx - 1) * (B - 1)) + B * (j - (sy - 1) * (B - 1));
-    const int64_t* nrow = uni ? nbase + sx + 3 * sy : nullptr;
-    // ring form: class box row of the column
-    const int rb = reg_class<B>(i) + 7 * reg_class<B>(j);
-    auto chunk = [&](auto kcc, auto k0c) {
-      constexpr int KN = decltype(kcc)::value, K0 = decltype(k0c)::value;
-      int64_t at[KN];
-      int kind[KN];
-#pragma unroll
-      for (int u = 0; u < KN; ++u) {
-        const int k = K0 + u;
-        const int sk = k < 0 ? 0 : (k <= B - 2 ? 1 : 2);  // compile-time per u
-        const bool ink = k >= 0 && k <= B - 1;
-        const bool inner = inxy && ink;
-        if (uni) {
-          const int64_t nb = nrow[9 * sk];
-          at[u] = nb + lxy + BB * (k - (sk - 1) * (B - 1));
-          kind[u] = inner ? (nb != own ? 1 : 0) : 2;
-          continue;
-        }
-        if (k >= 1 && k <= B - 2 && core) {
-          kind[u] = 0;
-          at[u] = own + Gm::lin(i, j, k);
-          continue;
-        }
-        const int4 e = R.reg[rb + 49 * reg_class<B>(k)];
-        if (e.x < 0) {
-          set_err(pv, kErrGraded);
-          kind[u] = 4;
-          at[u] = 0;
-          continue;
-        }
-        const int m = e.y, sh = l1 - m;
-        const int ox = 2 * i - (int)(int16_t)(e.z & 0xffff), oy = 2 * j - (e.z >> 16), oz = 2 * k - e.w;
-        const int64_t src = ((int64_t)e.x * nv) * pv.vs + Gm::lin(ox >> sh, oy >> sh, oz >> sh);
-        if (inner) {
-          kind[u] = e.x == b.slot ? 0 : 1;
-          at[u] = e.x == b.slot ? own + Gm::lin(i, j, k) : src;
-          continue;
-        }
-        const bool node = ((ox | oy | oz) & ((1 << sh) - 1)) == 0;
-        if (m >= b.lvl || node) {
-          kind[u] = 2;
-          at[u] = src;
-        } else {
-          if (m != b.lvl - 1) set_err(pv, kErrGraded);
-          kind[u] = 3;
-          at[u] = 0;
-        }
-      }
-      load_store(kcc, at, kind, col, i, j, K0);
-    };
-    // k = -W .. B-1+W in chunks of KC (compile-time k)
-    static_for<0, (S + KC - 1) / KC>([&](auto cc) {
-      constexpr int C = decltype(cc)::value;
-      constexpr int K0 = -W + C * KC;
-      constexpr int KN = (S - C * KC) < KC ? (S - C * KC) : KC;
-      chunk(std::integral_constant<int, KN>{}, std::integral_constant<int, K0>{});
-    });
-  }
-  if constexpr (ASYNC) {
-    cp_async_wait_all();
-    if (commit) {
-      // block-edge nodes owned by another block: store the owner's value (now
-      // in the tile) where the block's own copy differs
-      __syncthreads();
-      for (int col = threadIdx.x; col < BB; col += blockDim.x) {
-        const int i = col % B, j = col / B;
-        const bool side = i == 0 || i == B - 1 || j == 0 || j == B - 1;
-        const int sx = i <= B - 2 ? 1 : 2, sy = j <= B - 2 ? 1 : 2;
-        const int rb = reg_class<B>(i) + 7 * reg_class<B>(j);
-        for (int k = 0; k < B; k += (side || k == B - 1) ? 1 : B - 1) {
-          bool other;
-          if (uni) {
-            other = nbase[sx + 3 * sy + 9 * (k <= B - 2 ? 1 : 2)] != own;
-          } else {
-            other = R.reg[rb + 49 * reg_class<B>(k)].x != b.slot;
-          }
-          if (!other) continue;
-          for (int v = 0; v < nv; ++v) {
-            const TT val = tile[v * Bx::TILE + Bx::tix(i, j, k)];
-            const int64_t me = own + (int64_t)v * pv.vs + Gm::lin(i, j, k);
-            if (F[me] != val) Fw[me] = val;
-          }
-        }
-      }
-    }
-  }
-}
-
 // Stage plan of one active block, valid while the tree is fixed (the four RK
 // stages of a step): INTS int32 per active position,
 //   [0] slot, [1] level | tree << 8 | uniform << 30, [2 .. 2+D) block coordinates,
@@ -1225,38 +984,6 @@ __device__ __forceinline__ void gather_table(const PoolView& pv, int64_t own, co
   } else {
     for (int q0 = g.rank(); q0 < Bx::NPTS; q0 += U * g.size()) chunk(std::integral_constant<int, U>{}, q0, g.size());
   }
-}
-
-// Tensor-product prediction at half-coarse position o (per axis, odd = between
-// coarse nodes) from a tile whose coarse node n sits at tile index n*stride.
-// x first, then y, then z.  Used by refinement (stride 1: the mother's tile) and
-// by the details (stride 2: even nodes of the block's own tile).
-template <int D, int B, int W, typename TT, typename TA = TT>
-__device__ __forceinline__ TA predict_tile(const TT* tile, const int o[3], int stride) {
-  using Gm = Box<D, B, W>;
-  int base[3] = {0, 0, 0}, ns[3] = {1, 1, 1};
-#pragma unroll
-  for (int a = 0; a < D; ++a) {
-    const int fl = o[a] >> 1;  // floor(o / 2)
-    if (o[a] & 1) { ns[a] = 4; base[a] = fl - 1; }
-    else base[a] = fl;
-  }
-  TA vx[4][4];
-  for (int sz = 0; sz < ns[2]; ++sz)
-    for (int sy = 0; sy < ns[1]; ++sy) {
-      const int y = stride * (base[1] + sy), z = D == 3 ? stride * (base[2] + sz) : 0;
-      if (ns[0] == 4) {
-        const int x0 = stride * base[0];
-        vx[sz][sy] = dd4((TA)tile[Gm::tix(x0, y, z)], (TA)tile[Gm::tix(x0 + stride, y, z)],
-                         (TA)tile[Gm::tix(x0 + 2 * stride, y, z)], (TA)tile[Gm::tix(x0 + 3 * stride, y, z)]);
-      } else {
-        vx[sz][sy] = (TA)tile[Gm::tix(stride * base[0], y, z)];
-      }
-    }
-  TA vy[4];
-  for (int sz = 0; sz < ns[2]; ++sz)
-    vy[sz] = ns[1] == 4 ? dd4(vx[sz][0], vx[sz][1], vx[sz][2], vx[sz][3]) : vx[sz][0];
-  return ns[2] == 4 ? dd4(vy[0], vy[1], vy[2], vy[3]) : vy[0];
 }
 
 template <typename T>

@@ -38,19 +38,20 @@ template <typename T> __device__ __forceinline__ const T* lattice(const PoolView
 //   k = N(Y_s) on the synchronised tile, then the 3-register update
 //   s0: acc = y + dt/6 k, Y1 = y + dt/2 k      s1: acc += dt/3 k, Y2 = y + dt/2 k
 //   s2: acc += dt/3 k,    Y3 = y + dt k        s3: y = acc + dt/6 k
-// Advection RHS: -(u Dx phi + v Dy phi [+ w Dz phi]),
+// Advection RHS: -(u Dx phi + v Dy phi),
 //   D1 f = ((f[-2] - f[2]) + 8 (f[1] - f[-1])) / (12 dx).
+// 2D blocks; the 3D stage is k_stage3 (mr_adv3.cuh).
 //
 // The block's plan (k_plan) is read from shared memory, the next block's plan
 // is fetched while this one is processed; blocks with a uniform neighbourhood
 // take the direct gather, the others the general one through their ring.
-template <int D, int B, int RHS, typename TS, typename TY, typename TSRC, int NT, int ST>
-__global__ void __launch_bounds__(NT, NT <= 128 ? 8 : (D == 3 ? 3 : 4)) k_stage_adv(PoolView pv, const TSRC* __restrict__ src, TS* __restrict__ y,
+template <int B, int RHS, typename TS, typename TY, typename TSRC, int NT, int ST>
+__global__ void __launch_bounds__(NT, NT <= 128 ? 8 : 4) k_stage_adv(PoolView pv, const TSRC* __restrict__ src, TS* __restrict__ y,
                             TS* __restrict__ acc, TY* __restrict__ ynext, int stage_arg, StageArgs sa) {
   pdl_enter();
   constexpr int stage = ST;  // the RK stage, fixed at compile time
   static_assert(ST >= 0 && ST <= 3, "RK4 stage");
-  using Gm = Geo<D, B>;
+  constexpr int D = 2;
   using Bx = Box<D, B, 2>;  // the stencils reach two nodes
   using PL = Plan<D>;
   using TC = TY;  // stencil arithmetic type
@@ -59,12 +60,12 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 8 : (D == 3 ? 3 : 4)) k_stage_
   TC* tile = smem_as<TC>(kRingBytesD<D>);  // nvar == 1
   TC* cbox = tile + Bx::TILE;
   TC* scr = cbox + Bx::CBOX;
-  int32_t* gtab = reinterpret_cast<int32_t*>(scr + Bx::SCR);  // 2D: gather table
+  int32_t* gtab = reinterpret_cast<int32_t*>(scr + Bx::SCR);  // gather table
   __shared__ int32_t splan[2][PL::INTS];
   __shared__ int64_t snb[2][PL::NB];  // pool offsets of the plan's neighbours
   const int nact = pv.cnt->n_act;
   if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&pv.cnt->stage_blocks, (unsigned long long)nact);
-  if (D == 2) build_gtab<D, B, 2>(gtab);
+  build_gtab<D, B, 2>(gtab);
   if (blockIdx.x < nact && threadIdx.x < PL::INTS) {
     const int32_t v = pv.plan[(int64_t)blockIdx.x * PL::INTS + threadIdx.x];
     splan[0][threadIdx.x] = v;
@@ -80,18 +81,12 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 8 : (D == 3 ? 3 : 4)) k_stage_
     const BlockInfo b = plan_block<D>(pl);
     const TreeDev& td = pv.trees[b.tree];
     if ((pl[1] >> 30) & 1) {
-      if constexpr (D == 2)
-        gather_table<D, B, 2, 1, TSRC, TC>(pv, (int64_t)b.slot * pv.vs, snb[buf], gtab, src, (TSRC*)src, tile,
-                                           stage == 0);
-      else
-        fill_cols<B, TSRC, TC, 2>(pv, b, snb[buf], src, (TSRC*)src, tile, stage == 0, R, cbox, scr);
+      gather_table<D, B, 2, 1, TSRC, TC>(pv, (int64_t)b.slot * pv.vs, snb[buf], gtab, src, (TSRC*)src, tile,
+                                         stage == 0);
     } else {
       load_regions<D, CtaGroup>(pv, p, R);
       __syncthreads();
-      if constexpr (D == 2)
-        fill_tile<D, B, TSRC, TC, 2>(pv, b, src, (TSRC*)src, tile, stage == 0, R, cbox, scr, true);
-      else
-        fill_cols<B, TSRC, TC, 2>(pv, b, nullptr, src, (TSRC*)src, tile, stage == 0, R, cbox, scr, true);
+      fill_tile<D, B, TSRC, TC, 2>(pv, b, src, (TSRC*)src, tile, stage == 0, R, cbox, scr, true);
     }
     __syncthreads();
     const TC c = tree_cD<TC>(td, b.lvl);
@@ -100,7 +95,7 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 8 : (D == 3 ? 3 : 4)) k_stage_
     const int64_t base = (int64_t)b.slot * pv.vs;  // nvar == 1
     const int sh = td.Jmax - b.lvl;
     const TS cas = cs.ca, cys = cs.cy;
-    if constexpr (D == 2) {
+    {
       // thread = (column i, rows j0, j0 + G, ...): the column's velocity
       // factors are loaded once; the rows' loads are issued together
       constexpr int G = NT / B, RU = (B + G - 1) / G;
@@ -153,59 +148,6 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 8 : (D == 3 ? 3 : 4)) k_stage_
           } else {
             y[at] = av[r] + cas * kk;
           }
-        }
-      }
-    }
-    // 3D: UC points per thread at a time: their state, accumulator and
-    // velocity loads are issued together, then the stencils and the updates
-    constexpr int UC = D == 3 ? 4 : 1;
-    const TC uc2 = tree_rhs<TC>(td, 2);
-    for (int q0 = threadIdx.x; D == 3 && q0 < Gm::NI; q0 += UC * NT) {
-      TS yv[UC], av[UC];
-      TC u0[UC], u1[UC];
-#pragma unroll
-      for (int u = 0; u < UC; ++u) {
-        const int q = q0 + u * NT;
-        yv[u] = av[u] = TS(0);
-        u0[u] = tree_rhs<TC>(td, 0);
-        u1[u] = tree_rhs<TC>(td, 1);
-        if (q >= Gm::NI) continue;
-        if (stage <= 2) yv[u] = y[base + q];  // stage 0: committed (synchronised) y_n
-        if (stage >= 1) av[u] = acc[base + q];
-        if (RHS == MR_RHS_SWIRL) {
-          const int i = q % B, j = (q / B) % B;
-          const int64_t Ux = pmod64((b.c[0] * (B - 1) + i) << sh, td.N);
-          const int64_t Uy = pmod64((b.c[1] * (B - 1) + j) << sh, td.N);
-          const TC* A = lattice<TC>(pv) + td.lat_off + (int64_t)kLatSwA * td.N;
-          const TC* Bt = lattice<TC>(pv) + td.lat_off + (int64_t)kLatSwB * td.N;
-          u0[u] = ct * (A[Ux] * Bt[Uy]);
-          u1[u] = -(ct * (A[Uy] * Bt[Ux]));
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < UC; ++u) {
-        const int q = q0 + u * NT;
-        if (q >= Gm::NI) continue;
-        const int i = q % B, j = (q / B) % B, k = D == 3 ? q / (B * B) : 0;
-        const TC* t0 = tile + Bx::tix(i, j, k);
-        const TC dxv = ((t0[-2] - t0[2]) + TC(8) * (t0[1] - t0[-1])) * c;
-        const TC dyv = ((t0[-2 * Bx::S] - t0[2 * Bx::S]) + TC(8) * (t0[Bx::S] - t0[-Bx::S])) * c;
-        TC s = u0[u] * dxv + u1[u] * dyv;
-        if (D == 3) {
-          constexpr int P = Bx::S * Bx::S;
-          const TC dzv = ((t0[-2 * P] - t0[2 * P]) + TC(8) * (t0[P] - t0[-P])) * c;
-          s = s + uc2 * dzv;
-        }
-        const TS kk = (TS)(-s);
-        const int64_t at = base + q;
-        if (stage == 0) {
-          acc[at] = yv[u] + cas * kk;
-          ynext[at] = (TY)(yv[u] + cys * kk);
-        } else if (stage == 1 || stage == 2) {
-          acc[at] = av[u] + cas * kk;
-          ynext[at] = (TY)(yv[u] + cys * kk);
-        } else {
-          y[at] = av[u] + cas * kk;
         }
       }
     }
@@ -664,23 +606,25 @@ __global__ void __launch_bounds__(256) k_stage_ns(PoolView pv, const TSRC* __res
 }
 
 // ----------------------------------------------------------------- refine ----
-// x pass of the upsampling: fine x in [0, 2(B-1)] on mother rows y, z in [-1, B]
-template <int D, int B>
+// x pass of the upsampling: fine x in [0, 2(B-1)] on mother rows y in [-1, B]
+template <int B>
 struct RefGeo {
   static constexpr int NF = 2 * B - 1;
   static constexpr int NR = B + 2;
-  static constexpr int NX = NF * NR * (D == 3 ? NR : 1);
+  static constexpr int NX = NF * NR;
 };
 
 // Sec. 2.3: the synchronised mother tile is upsampled by the 4th-order
 // interpolating prediction and split into 2^d children (one treecode digit
 // appended); children are placed in the new active list in Hilbert order.
-template <int D, int B, typename TS, int NT>
-__global__ void __launch_bounds__(NT, NT <= 128 ? 8 : (D == 3 ? 3 : 4)) k_refine(PoolView pv, TS* __restrict__ y) {
+// 2D blocks; 3D ones are refined by k_refine3 (mr_adv3.cuh).
+template <int B, typename TS, int NT>
+__global__ void __launch_bounds__(NT, NT <= 128 ? 8 : 4) k_refine(PoolView pv, TS* __restrict__ y) {
   pdl_enter();
+  constexpr int D = 2;
   using Gm = Geo<D, B>;
   using Bx = Box<D, B, 1>;  // prediction of the children reaches one node
-  using RG = RefGeo<D, B>;
+  using RG = RefGeo<B>;
   RingD<D>& R = *smem_as<RingD<D>>(0);
   __shared__ int cslot[8];
   TS* tile = smem_as<TS>(kRingBytesD<D>);
@@ -706,10 +650,7 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 8 : (D == 3 ? 3 : 4)) k_refine
     const TreeDev& td = pv.trees[b.tree];
     build_ring<D, B>(pv, td, b, R);
     __syncthreads();
-    if constexpr (D == 2)
-      fill_tile<D, B, TS, TS, 1>(pv, b, y, y, tile, false, R, cbox, scr);
-    else
-      fill_cols<B, TS, TS, 1>(pv, b, nullptr, y, y, tile, false, R, cbox, scr);
+    fill_tile<D, B, TS, TS, 1>(pv, b, y, y, tile, false, R, cbox, scr);
     if (threadIdx.x == 0) {
       uint64_t key[8];
       int32_t cc[8][3];
@@ -733,37 +674,25 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 8 : (D == 3 ? 3 : 4)) k_refine
     }
     __syncthreads();
     // Separable upsampling, per variable: X = prediction along x on the
-    // mother's rows (y, z in [-1, B]), then y (and z) per child node -- the
-    // operations of the tensor product in the same order.
+    // mother's rows (y in [-1, B]), then y per child node -- the operations of
+    // the tensor product in the same order.
     for (int v = 0; v < nv; ++v) {
       const TS* tv = tile + v * Bx::TILE;
       for (int idx = threadIdx.x; idx < RG::NX; idx += blockDim.x) {
-        const int ox = idx % RG::NF, jy = (idx / RG::NF) % RG::NR - 1;
-        const int kz = D == 3 ? idx / (RG::NF * RG::NR) - 1 : 0;
+        const int ox = idx % RG::NF, jy = idx / RG::NF - 1;
         const int fl = ox >> 1;
-        X[idx] = (ox & 1) ? dd4(tv[Bx::tix(fl - 1, jy, kz)], tv[Bx::tix(fl, jy, kz)], tv[Bx::tix(fl + 1, jy, kz)],
-                                tv[Bx::tix(fl + 2, jy, kz)])
-                          : tv[Bx::tix(fl, jy, kz)];
+        X[idx] = (ox & 1) ? dd4(tv[Bx::tix(fl - 1, jy, 0)], tv[Bx::tix(fl, jy, 0)], tv[Bx::tix(fl + 1, jy, 0)],
+                                tv[Bx::tix(fl + 2, jy, 0)])
+                          : tv[Bx::tix(fl, jy, 0)];
       }
       __syncthreads();
-      auto xr = [&](int ox, int jy, int kz) { return X[((D == 3 ? kz + 1 : 0) * RG::NR + (jy + 1)) * RG::NF + ox]; };
+      auto xr = [&](int ox, int jy) { return X[(jy + 1) * RG::NF + ox]; };
       for (int idx = threadIdx.x; idx < Gm::NCH * Gm::NI; idx += blockDim.x) {
         const int ch = idx / Gm::NI, q = idx % Gm::NI;
-        const int i = q % B, j = (q / B) % B, k = D == 3 ? q / (B * B) : 0;
-        const int ox = ((ch >> 0) & 1) * (B - 1) + i, oy = ((ch >> 1) & 1) * (B - 1) + j;
-        const int oz = D == 3 ? ((ch >> 2) & 1) * (B - 1) + k : 0;
-        auto ypass = [&](int kz) -> TS {
-          const int fl = oy >> 1;
-          return (oy & 1) ? dd4(xr(ox, fl - 1, kz), xr(ox, fl, kz), xr(ox, fl + 1, kz), xr(ox, fl + 2, kz))
-                          : xr(ox, fl, kz);
-        };
-        TS val;
-        if (D == 2) {
-          val = ypass(0);
-        } else {
-          const int fl = oz >> 1;
-          val = (oz & 1) ? dd4(ypass(fl - 1), ypass(fl), ypass(fl + 1), ypass(fl + 2)) : ypass(fl);
-        }
+        const int i = q % B, j = q / B;
+        const int ox = (ch & 1) * (B - 1) + i, oy = (ch >> 1) * (B - 1) + j;
+        const int fl = oy >> 1;
+        const TS val = (oy & 1) ? dd4(xr(ox, fl - 1), xr(ox, fl), xr(ox, fl + 1), xr(ox, fl + 2)) : xr(ox, fl);
         y[((int64_t)cslot[ch] * nv + v) * pv.vs + q] = val;
       }
       __syncthreads();
@@ -787,11 +716,10 @@ __device__ __forceinline__ bool certain_vs_eps(float m32, float E, const TreeDev
   return __fadd_ru(m32, E) < td.epsf[0] || __fsub_rd(m32, E) >= td.epsf[1];
 }
 
-template <int D, int B>
+template <int B>
 struct DetGeo {
   static constexpr int NC = (B + 1) / 2 + 2;  // coarse rows -1 .. (B+1)/2
-  static constexpr int NX = NC * B * (D == 3 ? NC : 1);
-  static constexpr int NY = D == 3 ? B * B * NC : 0;  // 3D: after the y pass, coarse z rows
+  static constexpr int NX = NC * B;
 };
 
 // Maximum of v over the CTA (warp shuffles, then one value per warp in red);
@@ -805,26 +733,6 @@ __device__ __forceinline__ T block_max(T v, T* red) {
   __syncthreads();
   for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v = fmax(v, red[w]);
   return v;
-}
-
-// Maxima of a and b over the CTA in one reduction (warp shuffles, then one
-// value per warp in ra / rb); every thread gets the results.
-template <typename A, typename Bt>
-__device__ __forceinline__ void block_max2(A& a, Bt& b, A* ra, Bt* rb) {
-  for (int s = 16; s > 0; s >>= 1) {
-    a = fmax(a, (A)__shfl_xor_sync(0xffffffffu, a, s));
-    b = fmax(b, (Bt)__shfl_xor_sync(0xffffffffu, b, s));
-  }
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) {
-    ra[threadIdx.x >> 5] = a;
-    rb[threadIdx.x >> 5] = b;
-  }
-  __syncthreads();
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-    a = fmax(a, ra[w]);
-    b = fmax(b, rb[w]);
-  }
 }
 
 // Maxima of a, b and c over the CTA in one reduction (one value per warp in
@@ -857,7 +765,7 @@ __device__ __forceinline__ void block_max3(A& a, Bt& b, Ct& c, A* ra, Bt* rb, Ct
 template <int B>
 struct DetTab {
   using Bx = Box<2, B, 2>;
-  using DG = DetGeo<2, B>;
+  using DG = DetGeo<B>;
   static constexpr int NODD = B * B - ((B + 1) / 2) * ((B + 1) / 2);
   static constexpr int INTS = DG::NX + NODD;
   static_assert(Bx::NPTS < (1 << 12) && DG::NX < (1 << 12), "table entries fit their fields");
@@ -941,39 +849,32 @@ struct DetTab {
   }
 };
 
-// Shared-memory layout of k_details after the ring and the tile: the coarse
-// box and prediction scratch of the gather, reused once the tile is complete
-// for the passes of the prediction (X, and in 3D the y pass Y).  A pass in
-// type A keeps Y when it fits in that region, else (3D FP64 over an FP32 tile)
-// evaluates the y pass again per point: the same operations in the same order.
-template <int D, int B, typename TT, typename TD>
+// Shared memory of k_details after the ring and the tile: the coarse box and
+// prediction scratch of the gather, reused once the tile is complete for the x
+// pass of the prediction.
+template <int B, typename TT, typename TD>
 struct DetSmem {
-  using Bx = Box<D, B, 2>;
-  using DG = DetGeo<D, B>;
+  using Bx = Box<2, B, 2>;
   static constexpr size_t FILL = sizeof(TT) * (Bx::CBOX + Bx::SCR);  // per variable
-  template <typename A>
-  __host__ __device__ static constexpr bool ystore() { return D == 2 || sizeof(A) * (DG::NX + DG::NY) <= FILL; }
-  template <typename A>
-  __host__ __device__ static constexpr size_t pass_bytes() {
-    return sizeof(A) * (ystore<A>() ? DG::NX + DG::NY : DG::NX);
-  }
-  static constexpr size_t PASS = pass_bytes<TD>() > pass_bytes<float>() ? pass_bytes<TD>() : pass_bytes<float>();
+  static constexpr size_t PASS = (sizeof(TD) > 4 ? sizeof(TD) : 4) * DetGeo<B>::NX;
   __host__ __device__ static size_t region(int nv) { return FILL * nv > PASS ? FILL * nv : PASS; }
 };
 
-template <int D, int B, typename TS, typename TD, int NT, typename TT = TS>
-__global__ void __launch_bounds__(NT, NT <= 128 ? 8 : (D == 3 ? 3 : 4)) k_details(PoolView pv, TS* __restrict__ y) {
+// 2D blocks; the 3D details are k_details3 (mr_adv3.cuh).
+template <int B, typename TS, typename TD, int NT, typename TT = TS>
+__global__ void __launch_bounds__(NT, NT <= 128 ? 8 : 4) k_details(PoolView pv, TS* __restrict__ y) {
   pdl_enter();
+  constexpr int D = 2;
   using Gm = Geo<D, B>;
   using Bx = Box<D, B, 2>;  // prediction from even nodes reaches two nodes
-  using DG = DetGeo<D, B>;
+  using DG = DetGeo<B>;
   RingD<D>& R = *smem_as<RingD<D>>(0);
   __shared__ double red[2][32];
   TT* tile = smem_as<TT>(kRingBytesD<D>);  // tile type (TS or FP32); TD is the decision type
   TT* cbox = tile + pv.nvar * Bx::TILE;
   // gather scratch, reused for the passes once the tile is complete
   TT* scr = cbox + pv.nvar * Bx::CBOX;
-  using DS = DetSmem<D, B, TT, TD>;
+  using DS = DetSmem<B, TT, TD>;
   TD* X = reinterpret_cast<TD*>((reinterpret_cast<uintptr_t>(cbox) + 15) & ~(uintptr_t)15);
   const int nact = pv.cnt->n_round;
   const int nv = pv.nvar;
@@ -990,12 +891,10 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 8 : (D == 3 ? 3 : 4)) k_detail
   const bool plan_ok = pv.cnt->plan_topo == pv.cnt->topo;
   const size_t xbytes = DS::region(nv);
   int32_t* gtab = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(X) + ((xbytes + 15) & ~(size_t)15));
-  int32_t* xtab = gtab + Bx::NPTS;  // 2D detail tables
+  int32_t* xtab = gtab + Bx::NPTS;  // detail tables
   int32_t* otab = xtab + DG::NX;
-  if constexpr (D == 2) {
-    build_gtab<D, B, 2>(gtab);
-    DetTab<B>::build(xtab, otab);
-  }
+  build_gtab<D, B, 2>(gtab);
+  DetTab<B>::build(xtab, otab);
   // CTA-local work count and threshold scales (one atomic per CTA, not per block)
   unsigned long long ndet = 0;
   __shared__ double csv[kMaxVar];
@@ -1025,10 +924,10 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 8 : (D == 3 ? 3 : 4)) k_detail
       q = b.slot;
       if (threadIdx.x < PL::NB) {
         const int n = threadIdx.x;
-        const int o[3] = {n % 3 - 1, (n / 3) % 3 - 1, D == 3 ? n / 9 - 1 : 0};
-        if (o[0] != 0 || o[1] != 0 || o[2] != 0) {
+        const int o[2] = {n % 3 - 1, n / 3 - 1};
+        if (o[0] != 0 || o[1] != 0) {
           const TreeDev& tdl = pv.trees[b.tree];
-          const int64_t cn[3] = {b.c[0] + o[0], b.c[1] + o[1], b.c[2] + o[2]};
+          const int64_t cn[3] = {b.c[0] + o[0], b.c[1] + o[1], 0};
           q = tab_get<D>(pv, tdl, b.lvl, cn);
         }
       }
@@ -1072,127 +971,48 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 8 : (D == 3 ? 3 : 4)) k_detail
     }
     ndet += 1;
     const int64_t own = (int64_t)b.slot * nv * pv.vs;
-    if (uni && nv == 1 && D == 2)
+    if (uni && nv == 1) {
       gather_table<D, B, 2, 1, TS, TT>(pv, own, snbo, gtab, y, y, tile, true);
-    else if (uni && nv == 4 && D == 2)
+    } else if (uni && nv == 4) {
       gather_table<D, B, 2, 4, TS, TT>(pv, own, snbo, gtab, y, y, tile, true);
-    else if (D == 3 && uni) {
-      if constexpr (D == 3) fill_cols<B, TS, TT, 2>(pv, b, snbo, y, y, tile, true, R, cbox, scr);
     } else {
       if (uni) {
         build_ring<D, B>(pv, td, b, R);
         __syncthreads();
       }
       const bool ready = !uni && plan_ok && all_blocks;
-      if constexpr (D == 2)
-        fill_tile<D, B, TS, TT, 2>(pv, b, y, y, tile, true, R, cbox, scr, ready);
-      else
-        fill_cols<B, TS, TT, 2>(pv, b, nullptr, y, y, tile, true, R, cbox, scr, ready);
+      fill_tile<D, B, TS, TT, 2>(pv, b, y, y, tile, true, R, cbox, scr, ready);
     }
     __syncthreads();
     // Block maximum of |d| over the interior with arithmetic type A: x pass on
-    // coarse rows (yc, zc) in [-1, NC-2] into X, then y (and z) per odd node.
-    // 3D with EX: the same sweeps also give the interior's largest |value| and
-    // non-finite test (ex_mq, bad; the z sweep reads every interior node) and
-    // the coarse lattice's largest |value| (ex_mt; the x sweep reads every
-    // coarse node of the tile), reduced with the detail maximum in one step.
+    // the coarse rows into X, then y per odd node.  With EX the same sweeps also
+    // give the interior's largest |value| and non-finite test (ex_mq, bad) and
+    // the coarse lattice's largest |value| (ex_mt), reduced with the detail
+    // maximum in one step.
     TT ex_mq = TT(0);
     float ex_mt = 0.f;
     bool bad = false;
     auto pass = [&](auto tag, const TT* tv, auto exc) -> decltype(tag) {
       using A = decltype(tag);
-      constexpr bool EX = decltype(exc)::value;
       A* XA = reinterpret_cast<A*>(X);
-      if constexpr (D == 2) {
-        if constexpr (EX) {
-          TT mq = TT(0);
-          float mt = 0.f;
-          A md = DetTab<B>::template max_detail_ex<A>(xtab, otab, tv, XA, CtaGroup{}, mq, mt, bad);
-          block_max3<A, TT, float>(md, mq, mt, reinterpret_cast<A*>(red[0]), reinterpret_cast<TT*>(red[1]),
-                                   reinterpret_cast<float*>(red[1]) + 32);
-          ex_mq = mq;
-          ex_mt = mt;
-          return md;
-        } else {
-          const A md = DetTab<B>::template max_detail<A>(xtab, otab, tv, XA, CtaGroup{});
-          return block_max<A>(md, reinterpret_cast<A*>(red[0]));
-        }
-      }
-      float mt = 0.f;
-      for (int idx = threadIdx.x; idx < DG::NX; idx += blockDim.x) {
-        const int x = idx % B, yc = (idx / B) % DG::NC - 1, zc = D == 3 ? idx / (B * DG::NC) - 1 : 0;
-        const int yy = 2 * yc, zz = 2 * zc;
-        A val;
-        if ((x & 1) == 0) {
-          const TT t = tv[Bx::tix(x, yy, zz)];
-          if constexpr (EX) mt = fmaxf(mt, fabsf((float)t));
-          val = (A)t;
-        } else {
-          const int n0 = (x - 1) / 2;
-          const TT t0 = tv[Bx::tix(2 * n0 - 2, yy, zz)], t1 = tv[Bx::tix(2 * n0, yy, zz)],
-                   t2 = tv[Bx::tix(2 * n0 + 2, yy, zz)], t3 = tv[Bx::tix(2 * n0 + 4, yy, zz)];
-          if constexpr (EX)
-            mt = fmaxf(fmaxf(mt, fmaxf(fabsf((float)t0), fabsf((float)t1))), fmaxf(fabsf((float)t2), fabsf((float)t3)));
-          val = dd4((A)t0, (A)t1, (A)t2, (A)t3);
-        }
-        XA[idx] = val;
-      }
-      __syncthreads();
-      auto xat = [&](int x, int yc, int zc) { return XA[((D == 3 ? (zc + 1) * DG::NC : 0) + (yc + 1)) * B + x]; };
-      auto ypass = [&](int i, int j, int zc) -> A {
-        if ((j & 1) == 0) return xat(i, j / 2, zc);
-        const int m0 = (j - 1) / 2;
-        return dd4(xat(i, m0 - 1, zc), xat(i, m0, zc), xat(i, m0 + 1, zc), xat(i, m0 + 2, zc));
-      };
-      // 3D: the y pass once per (x, y, coarse z row), kept for the z pass
-      // where it fits (else evaluated again for each use)
-      constexpr bool ys = DS::template ystore<A>();
-      A* YA = XA + DG::NX;
-      if (D == 3 && ys) {
-        for (int idx = threadIdx.x; idx < DG::NY; idx += blockDim.x)
-          YA[idx] = ypass(idx % B, (idx / B) % B, idx / (B * B) - 1);
-        __syncthreads();
-      }
-      auto yat = [&](int i, int j, int zc) -> A {
-        if constexpr (ys) return YA[((zc + 1) * B + j) * B + i];
-        else return ypass(i, j, zc);
-      };
-      A md = A(0);  // a maximum of A values: exact in A
-      TT mq = TT(0);
-      for (int q = threadIdx.x; q < Gm::NI; q += blockDim.x) {
-        const int i = q % B, j = (q / B) % B, k = D == 3 ? q / (B * B) : 0;
-        const TT tq = tv[Bx::tix(i, j, k)];
-        if constexpr (EX) {
-          mq = fmax(mq, (TT)fabs(tq));
-          bad |= !isfinite(tq);
-        }
-        if (((i | j | k) & 1) == 0) continue;
-        const A val = (A)tq;
-        A pr;
-        if (D == 2) {
-          pr = ypass(i, j, 0);
-        } else if ((k & 1) == 0) {
-          pr = yat(i, j, k / 2);
-        } else {
-          const int k0 = (k - 1) / 2;
-          pr = dd4(yat(i, j, k0 - 1), yat(i, j, k0), yat(i, j, k0 + 1), yat(i, j, k0 + 2));
-        }
-        const A d = val - pr;
-        md = fmax(md, (A)fabs(d));
-      }
-      if constexpr (EX) {
+      if constexpr (decltype(exc)::value) {
+        TT mq = TT(0);
+        float mt = 0.f;
+        A md = DetTab<B>::template max_detail_ex<A>(xtab, otab, tv, XA, CtaGroup{}, mq, mt, bad);
         block_max3<A, TT, float>(md, mq, mt, reinterpret_cast<A*>(red[0]), reinterpret_cast<TT*>(red[1]),
                                  reinterpret_cast<float*>(red[1]) + 32);
         ex_mq = mq;
         ex_mt = mt;
         return md;
+      } else {
+        const A md = DetTab<B>::template max_detail<A>(xtab, otab, tv, XA, CtaGroup{});
+        return block_max<A>(md, reinterpret_cast<A*>(red[0]));
       }
-      return block_max<A>(md, reinterpret_cast<A*>(red[0]));
     };
     for (int v = 0; v < nv; ++v) {
       const TT* tv = tile + v * Bx::TILE;
       constexpr bool cert = sizeof(TT) == 4 && sizeof(TD) == 8;
-      // the first pass's sweeps (x and z in 3D, x and odd points in 2D) give the
+      // the first pass's sweeps (x pass and odd points) give the
       // detail maximum, the interior's largest |value| (exact in its type), the
       // non-finite test (any non-finite value makes the block norm NaN) and,
       // for the certified FP32 decision, the largest |value| the evaluation
@@ -1240,7 +1060,7 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 8 : (D == 3 ? 3 : 4)) k_detail
 template <int B, typename TS, typename TD, int NT>
 struct DetW {
   using Bx = Box<2, B, 2>;
-  using DG = DetGeo<2, B>;
+  using DG = DetGeo<B>;
   static constexpr int NW = NT / 32;
   static constexpr size_t GTAB = (4 * Bx::NPTS + 15) / 16 * 16;
   static constexpr size_t TABS = (4 * DetTab<B>::INTS + 15) / 16 * 16;  // detail index tables
@@ -1261,7 +1081,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_details_w(PoolView pv, TS* __
   pdl_enter();
   using Gm = Geo<2, B>;
   using Bx = Box<2, B, 2>;
-  using DG = DetGeo<2, B>;
+  using DG = DetGeo<B>;
   using PL = Plan<2>;
   using DW = DetW<B, TS, TD, NT>;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;

@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cstdio>
 
+#include "mr_adv3.cuh"
 #include "mr_kernels.cuh"
 
 namespace mr {
@@ -35,21 +36,20 @@ constexpr int64_t kFusedScanMax = 8192;
 
 // ---------------------------------------------------------------- stage ------
 // 2D blocks of 17^2 nodes: 128-thread CTAs, so small grids run in one wave.
-template <int D, int B>
-struct Threads { static constexpr int value = (D == 2 && B == 17) ? 128 : 256; };
+template <int B>
+struct Threads { static constexpr int value = B == 17 ? 128 : 256; };
 
-template <int D, int B, int RHS, typename TS, typename TY>
+template <int B, int RHS, typename TS, typename TY>
 static void stage_impl(const PoolView& pv, const Fields& f, int stage, const StageArgs& sa,
                        const LaunchCfg& lc, cudaStream_t st) {
-  constexpr int threads = Threads<D, B>::value;
-  const int nv = 1;
-  using Bx = Box<D, B, 2>;
-  const size_t smem = kRingBytesD<D> + sizeof(TY) * nv * (Bx::TILE + Bx::CBOX + Bx::SCR) + (D == 2 ? 4 * Bx::NPTS : 0);
+  constexpr int threads = Threads<B>::value;
+  using Bx = Box<2, B, 2>;
+  const size_t smem = kRingBytesD<2> + sizeof(TY) * (Bx::TILE + Bx::CBOX + Bx::SCR) + 4 * Bx::NPTS;
   TY* ynext = (TY*)(stage == 1 ? f.Yb : f.Ya);
-  // 2D: one warp per block when the grid holds enough blocks to fill the GPU
+  // one warp per block when the grid holds enough blocks to fill the GPU
   // several times over (or as tuned), else one CTA per block (shorter latency)
   const bool warp_form = lc.stage_form == 1 || (lc.stage_form < 0 && lc.n_hint >= 8 * lc.num_sms);
-  if constexpr (D == 2 && B == 17) {  // 17^2 blocks: 289 points per warp
+  if constexpr (B == 17) {  // 17^2 blocks: 289 points per warp
     if (warp_form) {
       // one instantiation per stage: stage 0 reads the committed state, the
       // others the previous stage value
@@ -85,7 +85,7 @@ static void stage_impl(const PoolView& pv, const Fields& f, int stage, const Sta
     constexpr int S = decltype(stc)::value;
     using TSRC = std::conditional_t<S == 0, TS, TY>;
     const TSRC* src = S == 0 ? (const TSRC*)f.y : (const TSRC*)(S == 2 ? f.Yb : f.Ya);
-    auto k = k_stage_adv<D, B, RHS, TS, TY, TSRC, threads, S>;
+    auto k = k_stage_adv<B, RHS, TS, TY, TSRC, threads, S>;
     prep_smem(k, smem);
     const int grid = persistent_grid(k, threads, smem, lc, lc.grid_mult);
     launch_k(lc.pdl, k, grid, threads, smem, st, pv, src, (TS*)f.y, (TS*)f.acc, ynext, stage, sa);
@@ -99,13 +99,37 @@ static void stage_impl(const PoolView& pv, const Fields& f, int stage, const Sta
   count_launch();
 }
 
-template <int D, int B, int RHS>
+// 3D advection stage (17^3 blocks).
+template <typename TS, typename TY>
+static void stage3_impl(const PoolView& pv, const Fields& f, int stage, const StageArgs& sa, const LaunchCfg& lc,
+                        cudaStream_t st) {
+  TY* ynext = (TY*)(stage == 1 ? f.Yb : f.Ya);
+  auto go = [&](auto stc) {
+    constexpr int S = decltype(stc)::value;
+    using TSRC = std::conditional_t<S == 0, TS, TY>;
+    const TSRC* src = S == 0 ? (const TSRC*)f.y : (const TSRC*)(S == 2 ? f.Yb : f.Ya);
+    auto k = k_stage3<TS, TY, TSRC, S>;
+    using SM = Stage3Smem<TY, TS>;
+    prep_smem(k, SM::BYTES);
+    launch_k(lc.pdl, k, persistent_grid(k, SM::NT, SM::BYTES, lc, lc.grid_mult), SM::NT, SM::BYTES, st, pv, src,
+             (TS*)f.y, (TS*)f.acc, ynext, sa);
+  };
+  switch (stage) {
+    case 0: go(std::integral_constant<int, 0>{}); break;
+    case 1: go(std::integral_constant<int, 1>{}); break;
+    case 2: go(std::integral_constant<int, 2>{}); break;
+    default: go(std::integral_constant<int, 3>{}); break;
+  }
+  count_launch();
+}
+
+template <int B, int RHS>
 static void stage_prec(const PoolView& pv, const Fields& f, int stage, const StageArgs& sa,
                        const LaunchCfg& lc, cudaStream_t st) {
   switch (pv.prec) {
-    case MR_PREC_FP64: stage_impl<D, B, RHS, double, double>(pv, f, stage, sa, lc, st); break;
-    case MR_PREC_FP32: stage_impl<D, B, RHS, float, float>(pv, f, stage, sa, lc, st); break;
-    default: stage_impl<D, B, RHS, double, float>(pv, f, stage, sa, lc, st); break;
+    case MR_PREC_FP64: stage_impl<B, RHS, double, double>(pv, f, stage, sa, lc, st); break;
+    case MR_PREC_FP32: stage_impl<B, RHS, float, float>(pv, f, stage, sa, lc, st); break;
+    default: stage_impl<B, RHS, double, float>(pv, f, stage, sa, lc, st); break;
   }
 }
 
@@ -158,10 +182,14 @@ void launch_stage_bs(const PoolView& pv, const Fields& f, int stage, const Stage
   if constexpr (D == 2) {
     if (pv.rhs_kind == MR_RHS_NS) stage_ns<B>(pv, f, stage, sa, lc, st);
     else if (pv.rhs_kind == MR_RHS_NS_SKEW) launch_stage_nss<B>(pv, f, stage, sa, lc, st);
-    else if (pv.rhs_kind == MR_RHS_SWIRL) stage_prec<D, B, MR_RHS_SWIRL>(pv, f, stage, sa, lc, st);
-    else stage_prec<D, B, MR_RHS_ADV>(pv, f, stage, sa, lc, st);
+    else if (pv.rhs_kind == MR_RHS_SWIRL) stage_prec<B, MR_RHS_SWIRL>(pv, f, stage, sa, lc, st);
+    else stage_prec<B, MR_RHS_ADV>(pv, f, stage, sa, lc, st);
   } else {
-    stage_prec<D, B, MR_RHS_ADV>(pv, f, stage, sa, lc, st);
+    switch (pv.prec) {
+      case MR_PREC_FP64: stage3_impl<double, double>(pv, f, stage, sa, lc, st); break;
+      case MR_PREC_FP32: stage3_impl<float, float>(pv, f, stage, sa, lc, st); break;
+      default: stage3_impl<double, float>(pv, f, stage, sa, lc, st); break;
+    }
   }
 }
 
@@ -194,18 +222,21 @@ static void dispatch_bs(const PoolView& pv, A&&... args) {
 template <int D, int B, typename TS>
 struct RefineRun {
   static void run(const PoolView& pv, const Fields& f, const LaunchCfg& lc, cudaStream_t st) {
-    constexpr int threads = Threads<D, B>::value;
-    using Bx = Box<D, B, 1>;
-    const size_t scr = (size_t)std::max<int64_t>((int64_t)pv.nvar * Bx::SCR, RefGeo<D, B>::NX);
-    const size_t smem = kRingBytesD<D> + sizeof(TS) * (pv.nvar * (Bx::TILE + Bx::CBOX) + scr);
-    auto k = k_refine<D, B, TS, threads>;
-    prep_smem(k, smem);
-    const int grid = persistent_grid(k, threads, smem, lc, lc.grid_mult);
-    launch_k(lc.pdl, k, grid, threads, smem, st, pv, (TS*)f.y);
-    count_launch();
+    auto go = [&](auto k, int threads, size_t smem) {
+      prep_smem(k, smem);
+      launch_k(lc.pdl, k, persistent_grid(k, threads, smem, lc, lc.grid_mult), threads, smem, st, pv, (TS*)f.y);
+      count_launch();
+    };
+    if constexpr (D == 3) {
+      go(k_refine3<TS>, Col3::NT, Refine3Smem<TS>::BYTES);
+    } else {
+      constexpr int threads = Threads<B>::value;
+      using Bx = Box<2, B, 1>;
+      const size_t scr = (size_t)std::max<int64_t>((int64_t)pv.nvar * Bx::SCR, RefGeo<B>::NX);
+      go(k_refine<B, TS, threads>, threads, kRingBytesD<2> + sizeof(TS) * (pv.nvar * (Bx::TILE + Bx::CBOX) + scr));
+    }
   }
 };
-
 
 template <int D>
 void launch_refine(const PoolView& pv, const Fields& f, int mode, const int8_t* mask,
@@ -246,42 +277,33 @@ template <int D, int B, typename TS>
 struct DetailsRun {
   static void run(const PoolView& pv, const Fields& f, bool fp64, const LaunchCfg& lc,
                   cudaStream_t st) {
-    constexpr int threads = Threads<D, B>::value;
+    auto go = [&](auto k, int threads, size_t smem) {
+      prep_smem(k, smem);
+      launch_k(lc.pdl, k, persistent_grid(k, threads, smem, lc, lc.grid_mult), threads, smem, st, pv, (TS*)f.y);
+      count_launch();
+    };
     // FP64 details for the plain FP64 form or when asked for (thresholds below
     // FP32 resolution); otherwise FP32, also for FP64 state
     const bool d64 = fp64 || pv.prec == MR_PREC_FP64;
-    const bool warp_form = pv.nvar == 1 && pv.norm_kind == 0 && sizeof(TS) == 4 &&
-                           (lc.stage_form == 1 || (lc.stage_form < 0 && lc.n_hint >= 8 * lc.num_sms));
-    if (D == 2 && warp_form) {  // one warp per block
-      if (d64) {
-        auto k = k_details_w<B, TS, double, threads>;
-        using DW = DetW<B, TS, double, threads>;
-        prep_smem(k, DW::SMEM);
-        launch_k(lc.pdl, k, persistent_grid(k, threads, DW::SMEM, lc, lc.grid_mult), threads, DW::SMEM, st, pv, (TS*)f.y);
-      } else {
-        auto k = k_details_w<B, TS, TS, threads>;
-        using DW = DetW<B, TS, TS, threads>;
-        prep_smem(k, DW::SMEM);
-        launch_k(lc.pdl, k, persistent_grid(k, threads, DW::SMEM, lc, lc.grid_mult), threads, DW::SMEM, st, pv, (TS*)f.y);
-      }
-      count_launch();
-      return;
-    }
-    using Bx = Box<D, B, 2>;
-    const size_t tt = d64 ? sizeof(TS) : 4;  // tile type: the state type, FP32 for FP32 details
-    const size_t region = d64 ? DetSmem<D, B, TS, double>::region(pv.nvar) : DetSmem<D, B, float, float>::region(pv.nvar);
-    const size_t smem = kRingBytesD<D> + tt * pv.nvar * Bx::TILE + 16 + region + 16 +
-                        (D == 2 ? 4 * (Bx::NPTS + DetTab<B>::INTS) : 0);
-    if (d64) {
-      auto k = k_details<D, B, TS, double, threads>;
-      prep_smem(k, smem);
-      launch_k(lc.pdl, k, persistent_grid(k, threads, smem, lc, lc.grid_mult), threads, smem, st, pv, (TS*)f.y);
+    if constexpr (D == 3) {
+      if (d64) go(k_details3<TS, double, TS>, Col3::NT, Det3Smem<TS, double>::BYTES);
+      else go(k_details3<TS, float, float>, Col3::NT, Det3Smem<float, float>::BYTES);
     } else {
-      auto k = k_details<D, B, TS, float, threads, float>;
-      prep_smem(k, smem);
-      launch_k(lc.pdl, k, persistent_grid(k, threads, smem, lc, lc.grid_mult), threads, smem, st, pv, (TS*)f.y);
+      constexpr int threads = Threads<B>::value;
+      const bool warp_form = pv.nvar == 1 && pv.norm_kind == 0 && sizeof(TS) == 4 &&
+                             (lc.stage_form == 1 || (lc.stage_form < 0 && lc.n_hint >= 8 * lc.num_sms));
+      if (warp_form) {  // one warp per block
+        if (d64) go(k_details_w<B, TS, double, threads>, threads, DetW<B, TS, double, threads>::SMEM);
+        else go(k_details_w<B, TS, TS, threads>, threads, DetW<B, TS, TS, threads>::SMEM);
+        return;
+      }
+      using Bx = Box<2, B, 2>;
+      const size_t tt = d64 ? sizeof(TS) : 4;  // tile type: the state type, FP32 for FP32 details
+      const size_t region = d64 ? DetSmem<B, TS, double>::region(pv.nvar) : DetSmem<B, float, float>::region(pv.nvar);
+      const size_t smem = kRingBytesD<2> + tt * pv.nvar * Bx::TILE + 16 + region + 16 + 4 * (Bx::NPTS + DetTab<B>::INTS);
+      if (d64) go(k_details<B, TS, double, threads>, threads, smem);
+      else go(k_details<B, TS, float, threads, float>, threads, smem);
     }
-    count_launch();
   }
 };
 template <int D, int B, typename TS>
