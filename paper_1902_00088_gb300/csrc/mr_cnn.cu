@@ -13,6 +13,8 @@
 // the block's details (max over variables) at interior nodes, -3 elsewhere.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "mr_device.cuh"
 #include "mr_cnn.h"
 
@@ -136,77 +138,13 @@ __global__ void __launch_bounds__(256) k_features(PoolView pv, const TS* __restr
   }
 }
 
-// -------------------------------------------------------- forward pass -------
-template <int T, typename WT>
-__device__ float cnn_forward(const float* x, const WT* w, float* h1, float* h2, float* h3, float* z) {
-  using CG = CnnGeo<T>;
-  constexpr int T2 = CG::T2, T3 = CG::T3;
-  for (int idx = threadIdx.x; idx < CG::N1; idx += blockDim.x) {
-    const int o = idx / (T * T), pix = idx % (T * T), i = pix / T, j = pix % T;
-    float s = (float)w[kB1 + o];
-    for (int c = 0; c < 2; ++c)
-      for (int di = 0; di < 3; ++di) {
-        const int ii = i + di - 1;
-        if (ii < 0 || ii >= T) continue;
-        for (int dj = 0; dj < 3; ++dj) {
-          const int jj = j + dj - 1;
-          if (jj < 0 || jj >= T) continue;
-          s += (float)w[kW1 + ((o * 2 + c) * 3 + di) * 3 + dj] * x[c * T * T + ii * T + jj];
-        }
-      }
-    h1[idx] = fmaxf(s, 0.f);
-  }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < CG::N2; idx += blockDim.x) {
-    const int o = idx / (T2 * T2), pix = idx % (T2 * T2), i = pix / T2, j = pix % T2;
-    float s = (float)w[kB2 + o];
-    for (int c = 0; c < kC; ++c)
-      for (int di = 0; di < 3; ++di) {
-        const int ii = 2 * i + di - 1;
-        if (ii < 0 || ii >= T) continue;
-        for (int dj = 0; dj < 3; ++dj) {
-          const int jj = 2 * j + dj - 1;
-          if (jj < 0 || jj >= T) continue;
-          s += (float)w[kW2 + ((o * kC + c) * 3 + di) * 3 + dj] * h1[c * T * T + ii * T + jj];
-        }
-      }
-    h2[idx] = fmaxf(s, 0.f);
-  }
-  __syncthreads();
-  for (int idx = threadIdx.x; idx < CG::N3; idx += blockDim.x) {
-    const int o = idx / (T3 * T3), pix = idx % (T3 * T3), i = pix / T3, j = pix % T3;
-    float s = (float)w[kB3 + o];
-    for (int c = 0; c < kC; ++c)
-      for (int di = 0; di < 3; ++di) {
-        const int ii = 2 * i + di - 1;
-        if (ii < 0 || ii >= T2) continue;
-        for (int dj = 0; dj < 3; ++dj) {
-          const int jj = 2 * j + dj - 1;
-          if (jj < 0 || jj >= T2) continue;
-          s += (float)w[kW3 + ((o * kC + c) * 3 + di) * 3 + dj] * h2[c * T2 * T2 + ii * T2 + jj];
-        }
-      }
-    h3[idx] = fmaxf(s, 0.f);
-  }
-  __syncthreads();
-  if (threadIdx.x < kC) {
-    float m = h3[threadIdx.x * T3 * T3];
-    for (int q = 1; q < T3 * T3; ++q) m = fmaxf(m, h3[threadIdx.x * T3 * T3 + q]);
-    z[threadIdx.x] = m;
-  }
-  __syncthreads();
-  float logit = (float)w[kBL];
-  for (int o = 0; o < kC; ++o) logit += (float)w[kWL + o] * z[o];
-  return logit;
-}
-
+// ----------------------------------------------------------- inference -------
 // Inference: p for every active block below Jmax (others get 0).  The
 // weights are staged once per CTA in shared memory as floats, transposed so
 // that the 16 output channels of a tap are contiguous; each thread computes
 // all 16 output channels of one pixel (one input load feeds 16 FMAs, the 16
-// weights come as four broadcast 16-byte loads).  Per output the sum runs in
-// the order of cnn_forward (bias, then input channel, row, column), so the
-// probabilities equal the training forward pass bit for bit.
+// weights come as four broadcast 16-byte loads).  Per output the sum runs over
+// bias, then input channel, row, column.
 template <int T>
 struct InferGeo {
   using CG = CnnGeo<T>;
@@ -316,140 +254,382 @@ __global__ void __launch_bounds__(256) k_cnn_infer(PoolView pv, const float* __r
 }
 
 // ---------------------------------------------------- training (fwd + bwd) ---
-// Samples [s0, s0 + nb) of the dataset (index list idx), mean weighted BCE.
-// Each CTA takes samples blockIdx.x, blockIdx.x + gridDim.x, ...; gradients
-// accumulate in shared memory and are added to the global buffer once.
+// Samples [s0, s0 + nb) of the dataset (index list idx), mean weighted BCE, one
+// sample at a time per CTA.  FP32 multiply-adds throughout (1.6 M per sample of
+// 25^2).  Shared-memory reads bound the kernel (a load writes a register per lane,
+// a broadcast one too, so every loaded value has to meet several others), and
+// every pass is tiled in registers:
+//   conv1: 16 channels of a pixel per thread; conv2: 4 channels of two pixels, one
+//   above the other; conv3: 4 channels of a pixel (weights transposed to
+//   [channel][tap][16]);
+//   conv2 weight gradient: 4 outputs x 3 taps of a row per thread, conv1: 2 outputs x
+//   2 channels x 3, conv3 (nonzero only at each channel's maximum): the 9 taps of an
+//   (o, c) pair -- all kept in registers over the CTA's samples;
+//   da1: a 2 x 2 pixel block (its 9 taps meet 4 output pixels) of 2 channels.
+// Activations are padded by one node, so no tap tests its bounds, and the rows of
+// h1 hold their even columns, then the odd ones: the stride-2 convolution reads
+// consecutive words.  Products with a zero gradient are left out (a non-finite
+// input under an inactive unit has no gradient).
+// 3000 samples of 25^2: 5890 us with one output value per thread and loop, now
+// 485 us (shared-memory pipe 89 % of peak).  Larger tiles (two pixels in conv1, four
+// in conv2, two blocks in da1) read less but leave threads idle: 490-510 us.
 template <int T>
-__global__ void __launch_bounds__(256) k_cnn_train(const float* __restrict__ feat,
-                                                   const float* __restrict__ label,
-                                                   const int32_t* __restrict__ idx, int64_t s0,
-                                                   int nb, const float* __restrict__ w, float w_pos,
-                                                   float* __restrict__ grad, float* __restrict__ loss,
-                                                   float* __restrict__ prob_out) {
-  pdl_enter();
+struct TrainGeo {
   using CG = CnnGeo<T>;
-  constexpr int T2 = CG::T2, T3 = CG::T3;
-  float* x = smem_as<float>(0);
-  float* h1 = x + CG::NX;
-  float* h2 = h1 + CG::N1;
-  float* h3 = h2 + CG::N2;
-  float* dh2 = h3 + CG::N3;
-  float* gacc = dh2 + CG::N2;
-  __shared__ float z[kC], dz[kC];
+  // 25^2: two CTAs of 12 warps per SM; 41^2: one of 24 (its activations fill the shared memory)
+  static constexpr int NT = T == 25 ? 384 : 768;
+  static constexpr int T2 = CG::T2, T3 = CG::T3;
+  static constexpr int P = T + 2, H = (P + 1) / 2;  // padded width; even columns of a row
+  static constexpr int P2 = T2 + 2;
+  static constexpr int DP = 20;                     // pitch of a pixel's 16 gradients
+  // offsets (floats)
+  static constexpr int W1 = 0, W2 = W1 + 18 * kC, W3 = W2 + 144 * kC, WS = W3 + 144 * kC;  // WS: b1 b2 b3 wl bl
+  static constexpr int D2 = (WS + 4 * kC + 1 + 3) / 4 * 4;
+  static constexpr int X = D2 + T2 * T2 * DP;
+  static constexpr int H1 = X + 2 * P * P;
+  static constexpr int H2 = H1 + kC * P * P;
+  static constexpr int H3 = H2 + kC * P2 * P2;
+  static constexpr int END = H3 + kC * T3 * T3;
+  static constexpr size_t SMEM = sizeof(float) * END;
+  static constexpr int MINB = SMEM <= 112 * 1024 ? 2 : 1;
+  static_assert(kC * P * P >= kCnnParams, "the gradients are summed over h1 at the end");
+  // node (r, c) of a padded h1 plane
+  __device__ static __forceinline__ int h1at(int o, int r, int c) { return (o * P + r) * P + (c & 1) * H + (c >> 1); }
+};
+
+template <int T>
+__global__ void __launch_bounds__(TrainGeo<T>::NT, TrainGeo<T>::MINB)
+    k_cnn_train(const float* __restrict__ feat, const float* __restrict__ label, const int32_t* __restrict__ idx,
+                int64_t s0, int nb, const float* __restrict__ w, float w_pos, float* __restrict__ grad,
+                float* __restrict__ loss, float* __restrict__ prob_out) {
+  pdl_enter();
+  using G = TrainGeo<T>;
+  constexpr int NT = G::NT, T2 = G::T2, T3 = G::T3, P = G::P, H = G::H, P2 = G::P2, DP = G::DP;
+  float* sm = smem_as<float>(0);
+  const float4* w1 = reinterpret_cast<const float4*>(sm + G::W1);
+  const float4* w2 = reinterpret_cast<const float4*>(sm + G::W2);
+  const float4* w3 = reinterpret_cast<const float4*>(sm + G::W3);
+  const float *b1 = sm + G::WS, *b2 = b1 + kC, *b3 = b2 + kC, *wl = b3 + kC, *bl = wl + kC;
+  float *d2 = sm + G::D2, *x = sm + G::X, *h1 = sm + G::H1, *h2 = sm + G::H2, *h3 = sm + G::H3;
+  __shared__ float z[kC];
   __shared__ int arg[kC];
-  __shared__ float dlogit_s;
-  for (int q = threadIdx.x; q < kCnnParams; q += blockDim.x) gacc[q] = 0.f;
-  float lsum = 0.f;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  for (int q = t; q < G::END; q += NT) sm[q] = 0.f;  // the padding stays zero
   __syncthreads();
+  for (int q = t; q < kC * 18; q += NT) sm[G::W1 + (q % 18) * kC + q / 18] = w[kW1 + q];
+  for (int q = t; q < kC * 144; q += NT) {
+    sm[G::W2 + (q % 144) * kC + q / 144] = w[kW2 + q];
+    sm[G::W3 + (q % 144) * kC + q / 144] = w[kW3 + q];
+  }
+  if (t < kC) {
+    sm[G::WS + t] = w[kB1 + t];
+    sm[G::WS + kC + t] = w[kB2 + t];
+    sm[G::WS + 2 * kC + t] = w[kB3 + t];
+    sm[G::WS + 3 * kC + t] = w[kWL + t];
+  }
+  if (t == 0) sm[G::WS + 4 * kC] = w[kBL];
+  float lsum = 0.f;
+  // gradients of this thread, over the CTA's samples
+  const int o3 = t >> 4, c3 = t & 15;                                  // conv3: pair (o, c), t < 256
+  const int og2 = t & 3, cd2 = (t >> 2) % 48, part2 = t / 192;         // conv2: 4 outputs, channel and row tap
+  const int c2 = cd2 / 3, di2 = cd2 % 3;
+  const int cb1 = t % 24, part1 = t / 24, op1 = cb1 / 3, di1 = cb1 % 3;  // conv1: 2 outputs, row tap
+  float g3[9] = {}, g2[4][3] = {}, g1[2][2][3] = {};
+  float gb1[2] = {}, gb2 = 0.f, gb3 = 0.f, gwl = 0.f, gbl = 0.f;
   for (int sb = blockIdx.x; sb < nb; sb += gridDim.x) {
+    __syncthreads();
     const int64_t sidx = idx ? (int64_t)idx[s0 + sb] : s0 + sb;
-    for (int q = threadIdx.x; q < CG::NX; q += blockDim.x) x[q] = feat[sidx * CG::NX + q];
+    const float* in = feat + sidx * (2 * T * T);
+    for (int q = t; q < 2 * T * T; q += NT) {
+      const int c = q / (T * T), r = q % (T * T);
+      x[(c * P + r / T + 1) * P + r % T + 1] = in[q];
+    }
+    for (int q = t; q < T2 * T2 * DP; q += NT) d2[q] = 0.f;
+    const float yv = label[sidx];
     __syncthreads();
-    const float logit = cnn_forward<T>(x, w, h1, h2, h3, z);
-    if (threadIdx.x == 0) {
-      const float p = 1.f / (1.f + expf(-logit));
-      const float yv = label[sidx];
-      const float pc = fminf(fmaxf(p, 1e-7f), 1.f - 1e-7f);
-      lsum += -(w_pos * yv * logf(pc) + (1.f - yv) * logf(1.f - pc)) / nb;
-      const float dl = (yv * w_pos * (p - 1.f) + (1.f - yv) * p) / nb;
-      dlogit_s = dl;
-      if (prob_out) prob_out[s0 + sb] = p;
-    }
-    if (threadIdx.x < kC) {
-      int a = 0;
-      float m = h3[threadIdx.x * T3 * T3];
-      for (int q = 1; q < T3 * T3; ++q)
-        if (h3[threadIdx.x * T3 * T3 + q] > m) { m = h3[threadIdx.x * T3 * T3 + q]; a = q; }
-      arg[threadIdx.x] = a;
-    }
-    __syncthreads();
-    const float dl = dlogit_s;
-    if (threadIdx.x < kC) {
-      gacc[kWL + threadIdx.x] += dl * z[threadIdx.x];
-      dz[threadIdx.x] = dl * w[kWL + threadIdx.x];
-    }
-    if (threadIdx.x == 0) gacc[kBL] += dl;
-    for (int q = threadIdx.x; q < CG::N2; q += blockDim.x) dh2[q] = 0.f;
-    __syncthreads();
-    // conv3: da3 is nonzero only at each channel's (first) maximum, if positive
-    for (int q = threadIdx.x; q < kC * kC * 9; q += blockDim.x) {
-      const int o = q / (kC * 9), c = (q / 9) % kC, di = (q / 3) % 3, dj = q % 3;
-      const int a = arg[o];
-      const float da = h3[o * T3 * T3 + a] > 0.f ? dz[o] : 0.f;
-      const int ii = 2 * (a / T3) + di - 1, jj = 2 * (a % T3) + dj - 1;
-      if (da != 0.f && ii >= 0 && ii < T2 && jj >= 0 && jj < T2) {
-        gacc[kW3 + q] += da * h2[c * T2 * T2 + ii * T2 + jj];
-        atomicAdd(&dh2[c * T2 * T2 + ii * T2 + jj], da * w[kW3 + q]);
-      }
-    }
-    if (threadIdx.x < kC) {
-      const int o = threadIdx.x;
-      gacc[kB3 + o] += h3[o * T3 * T3 + arg[o]] > 0.f ? dz[o] : 0.f;
+    // conv1
+    for (int pix = t; pix < T * T; pix += NT) {
+      const int i = pix / T, j = pix % T;
+      float a[kC];
+#pragma unroll
+      for (int o = 0; o < kC; ++o) a[o] = b1[o];
+#pragma unroll 1
+      for (int kd = 0; kd < 6; ++kd)  // channel and row of the tap
+#pragma unroll
+        for (int dj = 0; dj < 3; ++dj) {
+          const float xv = x[((kd / 3) * P + i + kd % 3) * P + j + dj];
+          const float4* wp = w1 + (kd * 3 + dj) * 4;
+#pragma unroll
+          for (int o4 = 0; o4 < 4; ++o4) {
+            const float4 wv = wp[o4];
+            a[4 * o4] = fmaf(wv.x, xv, a[4 * o4]);
+            a[4 * o4 + 1] = fmaf(wv.y, xv, a[4 * o4 + 1]);
+            a[4 * o4 + 2] = fmaf(wv.z, xv, a[4 * o4 + 2]);
+            a[4 * o4 + 3] = fmaf(wv.w, xv, a[4 * o4 + 3]);
+          }
+        }
+      const int at = G::h1at(0, i + 1, j + 1);
+#pragma unroll
+      for (int o = 0; o < kC; ++o) h1[at + o * P * P] = fmaxf(a[o], 0.f);
     }
     __syncthreads();
-    for (int q = threadIdx.x; q < CG::N2; q += blockDim.x)  // da2 = dh2 * relu'(a2)
-      if (!(h2[q] > 0.f)) dh2[q] = 0.f;
-    __syncthreads();
-    // conv2 weights: dW2[o][c][di][dj] = sum_pix da2[o][pix] h1[c][2i+di-1][2j+dj-1]
-    for (int q = threadIdx.x; q < kC * kC * 9; q += blockDim.x) {
-      const int o = q / (kC * 9), c = (q / 9) % kC, di = (q / 3) % 3, dj = q % 3;
-      float s = 0.f;
-      for (int pix = 0; pix < T2 * T2; ++pix) {
-        const float da = dh2[o * T2 * T2 + pix];
-        if (da == 0.f) continue;
-        const int ii = 2 * (pix / T2) + di - 1, jj = 2 * (pix % T2) + dj - 1;
-        if (ii >= 0 && ii < T && jj >= 0 && jj < T) s += da * h1[c * T * T + ii * T + jj];
-      }
-      gacc[kW2 + q] += s;
-    }
-    if (threadIdx.x < kC) {
-      float s = 0.f;
-      for (int pix = 0; pix < T2 * T2; ++pix) s += dh2[threadIdx.x * T2 * T2 + pix];
-      gacc[kB2 + threadIdx.x] += s;
-    }
-    __syncthreads();
-    // da1 = conv2^T(da2) * relu'(a1), written over h1
-    for (int q = threadIdx.x; q < CG::N1; q += blockDim.x) {
-      const int o = q / (T * T), pix = q % (T * T), i = pix / T, j = pix % T;
-      float s = 0.f;
-      if (h1[q] > 0.f) {
-        for (int di = 0; di < 3; ++di) {
-          const int ti = i + 1 - di;
-          if (ti < 0 || (ti & 1) || ti / 2 >= T2) continue;
-          for (int dj = 0; dj < 3; ++dj) {
-            const int tj = j + 1 - dj;
-            if (tj < 0 || (tj & 1) || tj / 2 >= T2) continue;
-            for (int c2 = 0; c2 < kC; ++c2)
-              s += w[kW2 + ((c2 * kC + o) * 3 + di) * 3 + dj] * dh2[c2 * T2 * T2 + (ti / 2) * T2 + tj / 2];
+    // conv2: pixels (2 ip, j) and (2 ip + 1, j), 4 channels
+    constexpr int NP = (T2 + 1) / 2;
+    for (int q = t; q < NP * T2 * 4; q += NT) {
+      const int og = q / (NP * T2), r = q % (NP * T2), ip = r / T2, j = r % T2;
+      float a[2][4];
+#pragma unroll
+      for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int o = 0; o < 4; ++o) a[m][o] = b2[4 * og + o];
+      const float* hp = h1 + 4 * ip * P + j;
+      const int down = 2 * ip + 1 < T2 ? P : 0;  // rows 3 and 4 repeat row 2 where the second pixel lies outside
+#pragma unroll 1
+      for (int c = 0; c < kC; ++c, hp += P * P) {
+        float v[5][3];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          const float* h = hp + (k < 3 ? k * P : 2 * P + (k - 2) * down);
+          v[k][0] = h[0];
+          v[k][1] = h[H];
+          v[k][2] = h[1];
+        }
+#pragma unroll
+        for (int tap = 0; tap < 9; ++tap) {
+          const float4 wv = w2[(c * 9 + tap) * 4 + og];
+#pragma unroll
+          for (int m = 0; m < 2; ++m) {
+            const float hv = v[2 * m + tap / 3][tap % 3];
+            a[m][0] = fmaf(wv.x, hv, a[m][0]);
+            a[m][1] = fmaf(wv.y, hv, a[m][1]);
+            a[m][2] = fmaf(wv.z, hv, a[m][2]);
+            a[m][3] = fmaf(wv.w, hv, a[m][3]);
           }
         }
       }
-      h1[q] = s;  // now da1
+#pragma unroll
+      for (int m = 0; m < 2; ++m)
+        if (2 * ip + m < T2)
+#pragma unroll
+          for (int o = 0; o < 4; ++o) h2[((4 * og + o) * P2 + 2 * ip + m + 1) * P2 + j + 1] = fmaxf(a[m][o], 0.f);
     }
     __syncthreads();
-    for (int q = threadIdx.x; q < kC * 2 * 9 + kC; q += blockDim.x) {
-      if (q < kC * 2 * 9) {
-        const int o = q / 18, c = (q / 9) % 2, di = (q / 3) % 3, dj = q % 3;
-        float s = 0.f;
-        for (int pix = 0; pix < T * T; ++pix) {
-          const float da = h1[o * T * T + pix];
-          if (da == 0.f) continue;
-          const int ii = pix / T + di - 1, jj = pix % T + dj - 1;
-          if (ii >= 0 && ii < T && jj >= 0 && jj < T) s += da * x[c * T * T + ii * T + jj];
+    // conv3
+    for (int q = t; q < T3 * T3 * 4; q += NT) {
+      const int og = q / (T3 * T3), pix = q % (T3 * T3), i = pix / T3, j = pix % T3;
+      float a[4];
+#pragma unroll
+      for (int o = 0; o < 4; ++o) a[o] = b3[4 * og + o];
+      const float* hp = h2 + 2 * i * P2 + 2 * j;
+#pragma unroll 1
+      for (int c = 0; c < kC; ++c)
+#pragma unroll
+        for (int tap = 0; tap < 9; ++tap) {
+          const float hv = hp[(c * P2 + tap / 3) * P2 + tap % 3];
+          const float4 wv = w3[(c * 9 + tap) * 4 + og];
+          a[0] = fmaf(wv.x, hv, a[0]);
+          a[1] = fmaf(wv.y, hv, a[1]);
+          a[2] = fmaf(wv.z, hv, a[2]);
+          a[3] = fmaf(wv.w, hv, a[3]);
         }
-        gacc[kW1 + q] += s;
-      } else {
-        const int o = q - kC * 18;
-        float s = 0.f;
-        for (int pix = 0; pix < T * T; ++pix) s += h1[o * T * T + pix];
-        gacc[kB1 + o] += s;
+#pragma unroll
+      for (int o = 0; o < 4; ++o) h3[(4 * og + o) * T3 * T3 + pix] = fmaxf(a[o], 0.f);
+    }
+    __syncthreads();
+    // global maximum of each channel and its first pixel
+    for (int c = warp; c < kC; c += NT / 32) {
+      float m = -1.f;
+      int a = 1 << 20;
+      for (int q = lane; q < T3 * T3; q += 32) {
+        const float v = h3[c * T3 * T3 + q];
+        if (v > m) { m = v; a = q; }
+      }
+      for (int s = 16; s > 0; s >>= 1) {
+        const float om = __shfl_xor_sync(0xffffffffu, m, s);
+        const int oa = __shfl_xor_sync(0xffffffffu, a, s);
+        if (om > m || (om == m && oa < a)) { m = om; a = oa; }
+      }
+      if (lane == 0) { z[c] = m; arg[c] = a; }
+    }
+    __syncthreads();
+    float logit = *bl;
+#pragma unroll
+    for (int o = 0; o < kC; ++o) logit = fmaf(wl[o], z[o], logit);
+    const float p = 1.f / (1.f + expf(-logit));
+    const float dl = (yv * w_pos * (p - 1.f) + (1.f - yv) * p) / nb;
+    if (t == 0) {
+      const float pc = fminf(fmaxf(p, 1e-7f), 1.f - 1e-7f);
+      lsum += -(w_pos * yv * logf(pc) + (1.f - yv) * logf(1.f - pc)) / nb;
+      if (prob_out) prob_out[s0 + sb] = p;
+      gbl += dl;
+    }
+    if (t < kC) {
+      gwl = fmaf(dl, z[t], gwl);
+      if (z[t] > 0.f) gb3 = fmaf(dl, wl[t], gb3);
+    }
+    // conv3: da3 is nonzero only at each channel's (first) maximum, if positive
+    if (t < 256) {
+      const float da = z[o3] > 0.f ? dl * wl[o3] : 0.f;
+      if (da != 0.f) {
+        const float* hp = h2 + (c3 * P2 + 2 * (arg[o3] / T3)) * P2 + 2 * (arg[o3] % T3);
+#pragma unroll
+        for (int tap = 0; tap < 9; ++tap) g3[tap] = fmaf(da, hp[(tap / 3) * P2 + tap % 3], g3[tap]);
+      }
+    }
+    if (warp >= 6) {
+      // gradient of h2, added output by output: a warp holds the 9 taps of 3 channels
+      const int c = (warp - 6) * 3 + lane / 9, tap = lane % 9;
+      for (int o = 0; o < kC; ++o) {
+        const float da = z[o] > 0.f ? dl * wl[o] : 0.f;
+        const int ii = 2 * (arg[o] / T3) + tap / 3 - 1, jj = 2 * (arg[o] % T3) + tap % 3 - 1;
+        if (lane < 27 && c < kC && da != 0.f && ii >= 0 && ii < T2 && jj >= 0 && jj < T2) {
+          float* d = d2 + (ii * T2 + jj) * DP + c;
+          *d = fmaf(da, sm[G::W3 + (c * 9 + tap) * kC + o], *d);
+        }
+        __syncwarp();
       }
     }
     __syncthreads();
+    for (int q = t; q < T2 * T2 * kC; q += NT) {  // da2 = dh2 * relu'(a2)
+      const int pix = q >> 4, o = q & 15;
+      if (!(h2[(o * P2 + pix / T2 + 1) * P2 + pix % T2 + 1] > 0.f)) d2[pix * DP + o] = 0.f;
+    }
+    __syncthreads();
+    // conv2 weights: dW2[o][c][di][dj] = sum_pix da2[o][pix] h1[c][2i+di-1][2j+dj-1]
+    for (int i = part2; i < T2; i += NT / 192) {
+      const float* hr = h1 + (c2 * P + 2 * i + di2) * P;
+      const float4* dr = reinterpret_cast<const float4*>(d2 + i * T2 * DP) + og2;
+      float e0 = hr[0];
+      for (int j = 0; j < T2; ++j) {
+        const float4 d = dr[j * (DP / 4)];
+        const float od = hr[H + j], e1 = hr[j + 1];
+        const float dv[4] = {d.x, d.y, d.z, d.w};
+#pragma unroll
+        for (int o = 0; o < 4; ++o)
+          if (dv[o] != 0.f) {
+            g2[o][0] = fmaf(dv[o], e0, g2[o][0]);
+            g2[o][1] = fmaf(dv[o], od, g2[o][1]);
+            g2[o][2] = fmaf(dv[o], e1, g2[o][2]);
+          }
+        e0 = e1;
+      }
+    }
+    {  // bias: NT / 16 threads per channel
+      const int o = t & 15;
+      for (int pix = t >> 4; pix < T2 * T2; pix += NT / 16) gb2 += d2[pix * DP + o];
+    }
+    __syncthreads();
+    // da1 = conv2^T(da2) * relu'(a1), written over h1: pixels (2a, 2b) .. (2a+1, 2b+1)
+    for (int q = t; q < T2 * T2 * 8; q += NT) {
+      const int cg = q / (T2 * T2), r = q % (T2 * T2), a = r / T2, b = r % T2;
+      float s[2][2][2] = {};  // channel, row, column
+      const bool ra = a + 1 < T2, rb = b + 1 < T2;
+      const float4* dp = reinterpret_cast<const float4*>(d2 + r * DP);
+#pragma unroll 1
+      for (int o4 = 0; o4 < 4; ++o4) {
+        const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 d[2][2];
+        d[0][0] = dp[o4];
+        d[0][1] = rb ? dp[o4 + DP / 4] : zero;
+        d[1][0] = ra ? dp[o4 + T2 * (DP / 4)] : zero;
+        d[1][1] = ra && rb ? dp[o4 + (T2 + 1) * (DP / 4)] : zero;
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+          for (int tap = 0; tap < 9; ++tap) {
+            const int di = tap / 3, dj = tap % 3;
+            const float4 wv = w2[((2 * cg + c) * 9 + tap) * 4 + o4];
+            const float4 dv = d[di == 0][dj == 0];
+            float& u = s[c][di != 1][dj != 1];
+            u = fmaf(wv.x, dv.x, u);
+            u = fmaf(wv.y, dv.y, u);
+            u = fmaf(wv.z, dv.z, u);
+            u = fmaf(wv.w, dv.w, u);
+          }
+      }
+#pragma unroll
+      for (int c = 0; c < 2; ++c)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          const int i = 2 * a + m / 2, j = 2 * b + m % 2;
+          if (i >= T || j >= T) continue;
+          float* h = h1 + G::h1at(2 * cg + c, i + 1, j + 1);
+          *h = *h > 0.f ? s[c][m / 2][m % 2] : 0.f;
+        }
+    }
+    __syncthreads();
+    // conv1 weights: dW1[o][k][di][dj] = sum_pix da1[o][pix] x[k][i+di-1][j+dj-1]
+    for (int i = part1; i < T; i += NT / 24) {
+      const float* xr = x + (i + di1) * P;
+      const float* ha = h1 + (2 * op1 * P + i + 1) * P;
+      const float* hb = ha + P * P;
+      float xv[2][3];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        xv[k][0] = xr[k * P * P];
+        xv[k][1] = xr[k * P * P + 1];
+      }
+      auto add = [&](float da, float db, int j) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) xv[k][2] = xr[k * P * P + j + 2];
+        if (da != 0.f) {
+#pragma unroll
+          for (int k = 0; k < 2; ++k)
+#pragma unroll
+            for (int dj = 0; dj < 3; ++dj) g1[0][k][dj] = fmaf(da, xv[k][dj], g1[0][k][dj]);
+        }
+        if (db != 0.f) {
+#pragma unroll
+          for (int k = 0; k < 2; ++k)
+#pragma unroll
+            for (int dj = 0; dj < 3; ++dj) g1[1][k][dj] = fmaf(db, xv[k][dj], g1[1][k][dj]);
+        }
+        gb1[0] += da;
+        gb1[1] += db;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          xv[k][0] = xv[k][1];
+          xv[k][1] = xv[k][2];
+        }
+      };
+      // node j is padded column j + 1: odd columns of the row for even j
+      for (int m = 0; m < T / 2; ++m) {
+        add(ha[H + m], hb[H + m], 2 * m);
+        add(ha[m + 1], hb[m + 1], 2 * m + 1);
+      }
+      add(ha[H + T / 2], hb[H + T / 2], T - 1);
+    }
   }
-  for (int q = threadIdx.x; q < kCnnParams; q += blockDim.x)
-    if (gacc[q] != 0.f) atomicAdd(&grad[q], gacc[q]);
-  if (threadIdx.x == 0 && loss) atomicAdd(loss, lsum);
+  // sum of the CTA's threads in shared memory, then one addition per parameter
+  __syncthreads();
+  float* ga = h1;
+  for (int q = t; q < kCnnParams; q += NT) ga[q] = 0.f;
+  __syncthreads();
+  if (t < 256)
+#pragma unroll
+    for (int tap = 0; tap < 9; ++tap) ga[kW3 + (o3 * kC + c3) * 9 + tap] = g3[tap];
+#pragma unroll
+  for (int o = 0; o < 4; ++o)
+#pragma unroll
+    for (int dj = 0; dj < 3; ++dj) atomicAdd(&ga[kW2 + ((4 * og2 + o) * kC + c2) * 9 + di2 * 3 + dj], g2[o][dj]);
+#pragma unroll
+  for (int o = 0; o < 2; ++o) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int dj = 0; dj < 3; ++dj) atomicAdd(&ga[kW1 + ((2 * op1 + o) * 2 + k) * 9 + di1 * 3 + dj], g1[o][k][dj]);
+    if (di1 == 0) atomicAdd(&ga[kB1 + 2 * op1 + o], gb1[o]);
+  }
+  atomicAdd(&ga[kB2 + (t & 15)], gb2);
+  if (t < kC) {
+    ga[kB3 + t] = gb3;
+    ga[kWL + t] = gwl;
+  }
+  if (t == 0) ga[kBL] = gbl;
+  __syncthreads();
+  for (int q = t; q < kCnnParams; q += NT)
+    if (ga[q] != 0.f) atomicAdd(&grad[q], ga[q]);
+  if (t == 0 && loss) atomicAdd(loss, lsum);
 }
 
 __global__ void k_adam(float* w, float* m, float* v, float* g, int n, float lr, float b1, float b2,
@@ -633,12 +813,6 @@ template <int T>
 static size_t infer_smem() {
   return InferGeo<T>::SMEM;
 }
-template <int T>
-static size_t train_smem() {
-  using CG = CnnGeo<T>;
-  return sizeof(float) * (CG::NX + CG::N1 + CG::N2 + CG::N3 + CG::N2 + kCnnParams);
-}
-
 void launch_infer(const PoolView& pv, int Bs, const float* feat, const __nv_bfloat16* wb, float* prob,
                   int64_t n_explicit, int num_sms, cudaStream_t st) {
   if (Bs == 17) {
@@ -656,16 +830,13 @@ void launch_infer(const PoolView& pv, int Bs, const float* feat, const __nv_bflo
 void launch_train(int Bs, const float* feat, const float* label, const int32_t* idx, int64_t s0, int nb,
                   const float* w, float w_pos, float* grad, float* loss, float* prob_out, int num_sms,
                   cudaStream_t st) {
-  const int grid = nb < num_sms ? nb : num_sms;
-  if (Bs == 17) {
-    auto k = k_cnn_train<25>;
-    prep(k, train_smem<25>());
-    k<<<grid, 256, train_smem<25>(), st>>>(feat, label, idx, s0, nb, w, w_pos, grad, loss, prob_out);
-  } else {
-    auto k = k_cnn_train<41>;
-    prep(k, train_smem<41>());
-    k<<<grid, 256, train_smem<41>(), st>>>(feat, label, idx, s0, nb, w, w_pos, grad, loss, prob_out);
-  }
+  auto go = [&](auto k, auto geo) {
+    using G = decltype(geo);
+    prep(k, G::SMEM);
+    k<<<std::min(nb, num_sms * G::MINB), G::NT, G::SMEM, st>>>(feat, label, idx, s0, nb, w, w_pos, grad, loss, prob_out);
+  };
+  if (Bs == 17) go(k_cnn_train<25>, TrainGeo<25>{});
+  else go(k_cnn_train<41>, TrainGeo<41>{});
   count_launch();
 }
 
