@@ -1600,23 +1600,22 @@ mr_status mr_cnn_eval(mr_ctx ctx, const float* params, const float* x, const flo
   mr_status s = ensure_cnn(ctx);
   if (s) return s;
   const int64_t fl = feat_len(ctx);
-  TmpBuf<float> dx, dy, dw, dg, dl, dp;
-  CK(dx.alloc(n * fl * 4));
-  CK(dy.alloc(n * 4));
-  CK(dw.alloc(kCnnParams * 4));
-  CK(dg.alloc(kCnnParams * 4));
-  CK(dl.alloc(4));
-  CK(dp.alloc(n * 4));
-  CK(cudaMemcpy(dx.p, x, n * fl * 4, cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(dy.p, y, n * 4, cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(dw.p, params, kCnnParams * 4, cudaMemcpyHostToDevice));
-  CK(cudaMemset(dg.p, 0, kCnnParams * 4));
-  CK(cudaMemset(dl.p, 0, 4));
-  launch_train(ctx->p.Bs, dx.p, dy.p, nullptr, 0, (int)n, dw.p, w_pos, dg.p, dl.p, dp.p, ctx->lc.num_sms, ctx->st);
+  // one stream-ordered buffer for the call (cudaMalloc and cudaFree synchronise
+  // the device): samples, labels, parameters; gradient, loss, probabilities
+  const int64_t nin = n * fl + n + kCnnParams, nout = kCnnParams + 1 + n;
+  TmpBuf<float> d;
+  CK(d.alloc_on((nin + nout) * 4, ctx->st));
+  float *dx = d.p, *dy = dx + n * fl, *dw = dy + n, *dg = dw + kCnnParams, *dl = dg + kCnnParams, *dp = dl + 1;
+  CK(cudaMemcpyAsync(dx, x, n * fl * 4, cudaMemcpyHostToDevice, ctx->st));
+  CK(cudaMemcpyAsync(dy, y, n * 4, cudaMemcpyHostToDevice, ctx->st));
+  CK(cudaMemcpyAsync(dw, params, kCnnParams * 4, cudaMemcpyHostToDevice, ctx->st));
+  CK(cudaMemsetAsync(dg, 0, (kCnnParams + 1) * 4, ctx->st));
+  launch_train(ctx->p.Bs, dx, dy, nullptr, 0, (int)n, dw, w_pos, dg, dl, dp, ctx->lc.num_sms, ctx->st);
+  CK(cudaGetLastError());
+  if (prob) CK(cudaMemcpyAsync(prob, dp, n * 4, cudaMemcpyDeviceToHost, ctx->st));
+  if (grad) CK(cudaMemcpyAsync(grad, dg, kCnnParams * 4, cudaMemcpyDeviceToHost, ctx->st));
+  if (loss) CK(cudaMemcpyAsync(loss, dl, 4, cudaMemcpyDeviceToHost, ctx->st));
   CK(cudaStreamSynchronize(ctx->st));
-  if (prob) CK(cudaMemcpy(prob, dp.p, n * 4, cudaMemcpyDeviceToHost));
-  if (grad) CK(cudaMemcpy(grad, dg.p, kCnnParams * 4, cudaMemcpyDeviceToHost));
-  if (loss) CK(cudaMemcpy(loss, dl.p, 4, cudaMemcpyDeviceToHost));
   return MR_OK;
 }
 
