@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(Stage3Smem<TY, TS>::NT, 2) k_stage3(PoolView p
     // Node 8 belongs to the lower half.
     auto commit = [&](int half, int j) {
       const int64_t at = own + t + NQ * (8 * half + j);
-      if (ST == 0 && !(half && j == 0) && src[at] != raw[j]) const_cast<TSRC*>(src)[at] = raw[j];
+      if (ST == 0 && !(half && j == 0) && differs(src[at], raw[j])) const_cast<TSRC*>(src)[at] = raw[j];
     };
     auto put = [&](int half) {  // the half column to the tile
 #pragma unroll
@@ -539,7 +539,7 @@ __global__ void __launch_bounds__(Stage3Smem<TY, TS>::NT, 2) k_stage3(PoolView p
 }
 
 // ---------------------------------------------------------------- details ----
-// Details of 17^3 blocks (k_details' evaluation).  P(R(B)) reads the coarse
+// Details of 17^3 blocks (Sec. 2.3: D = B - P(R(B)), x then y then z).  P(R(B)) reads the coarse
 // lattice of the tile only, and every coarse-lattice node of the ghost layer is
 // a node of its owner whatever the owner's level: 602 ghost nodes per block
 // (11^3 coarse nodes less the block's own 9^3) are all that is gathered, and
@@ -560,25 +560,6 @@ struct Det3Smem {
   static constexpr size_t TAB = ((size_t)kRingBytesD<3> + 15) / 16 * 16;
   static constexpr size_t GT = (4 * NG + 15) / 16 * 16;
   static constexpr size_t BYTES = TAB + GT + XB + sizeof(TT) * E;
-};
-
-// Largest |value| added, NaN ignored (as fmax does).  FP64 values are compared
-// on their bit patterns, which order as the magnitudes do: the comparison of
-// doubles would take the FP64 pipe, the bound of the FP64 details.
-template <typename T>
-struct AbsMax {
-  T m = T(0);
-  __device__ __forceinline__ void add(T v) { m = fmax(m, (T)fabs(v)); }
-  __device__ __forceinline__ T get() const { return m; }
-};
-template <>
-struct AbsMax<double> {
-  long long m = 0;
-  __device__ __forceinline__ void add(double v) {
-    const long long b = __double_as_longlong(v) & 0x7fffffffffffffffLL;
-    if (b > m && b <= 0x7ff0000000000000LL) m = b;
-  }
-  __device__ __forceinline__ double get() const { return __longlong_as_double(m); }
 };
 
 template <typename TS, typename TD, typename TT>
@@ -712,8 +693,8 @@ __global__ void __launch_bounds__(Col3::NT, sizeof(TS) == 8 ? 2 : 3) k_details3(
         for (int k = 0; k < B; ++k) raw[k] = k < B - 1 ? mid[NQ * k] : *top;
 #pragma unroll
         for (int k = 0; k < B; ++k) {
-          if ((x == B - 1 || yy == B - 1 || k == B - 1) && y[me + NQ * k] != raw[k]) y[me + NQ * k] = raw[k];
-          v[k] = (TT)raw[k];
+          if ((x == B - 1 || yy == B - 1 || k == B - 1) && differs(y[me + NQ * k], raw[k])) y[me + NQ * k] = raw[k];
+          v[k] = to_tile<TT>(raw[k]);
         }
       }
       for (int g = t; g < SM::NG; g += NT) {
@@ -758,8 +739,8 @@ __global__ void __launch_bounds__(Col3::NT, sizeof(TS) == 8 ? 2 : 3) k_details3(
         });
 #pragma unroll
         for (int k = 0; k < B; ++k) {
-          if (((other >> k) & 1) && y[me + NQ * k] != raw[k]) y[me + NQ * k] = raw[k];
-          v[k] = (TT)raw[k];
+          if (((other >> k) & 1) && differs(y[me + NQ * k], raw[k])) y[me + NQ * k] = raw[k];
+          v[k] = to_tile<TT>(raw[k]);
         }
       }
       for (int g = t; g < SM::NG; g += NT) {
@@ -849,7 +830,11 @@ __global__ void __launch_bounds__(Col3::NT, sizeof(TS) == 8 ? 2 : 3) k_details3(
                               reinterpret_cast<float*>(red[1]) + 32);
     double md = 0.0;  // thread 0's value is stored
     if constexpr (cert) {
-      // certified as in k_details: E bounds the FP32 evaluation's error
+      // FP32 values, FP64 decision: the FP32 evaluation differs from the FP64 one
+      // by at most ~20 u max|tile| (u = 2^-24, x/y/z passes of the 4-point rule and
+      // the subtraction); where its maximum is farther than 32 u max|tile| from eps
+      // the threshold decision (Sec. 2.3) is the FP64 one, otherwise the block is
+      // evaluated again in FP64
       const float err = 0x1p-19f * fmaxf(mtr, (float)mq) + 1e-37f;
       if (pv.norm_kind == 0 && certain_vs_eps(m0, err, td)) {
         md = (double)m0;

@@ -74,6 +74,31 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, int li
   return false;
 }
 
+// float(d), rounded to nearest even, on the integer pipes: a conversion takes the
+// FP64 pipe, which yields two results per clock and SM on GB300.  Values whose
+// float is not a normal number go through the conversion instruction.
+__device__ __forceinline__ float f64_to_f32(double d) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(d);
+  const unsigned hi = (unsigned)(u >> 32);
+  const unsigned e = (hi >> 20) & 0x7ffu;
+  if (e - 897u > 253u) return (float)d;  // exponent outside [-126, 127]
+  const unsigned long long w = u & 0x7fffffffffffffffULL;
+  const unsigned m = (unsigned)((w + 0x0fffffffULL + ((w >> 29) & 1ULL)) >> 29) - (896u << 23);
+  return __uint_as_float(m | (hi & 0x80000000u));
+}
+// Value in the tile's type.
+template <typename TT, typename TS>
+__device__ __forceinline__ TT to_tile(TS v) {
+  if constexpr (sizeof(TS) == 8 && sizeof(TT) == 4) return f64_to_f32(v);
+  else return (TT)v;
+}
+// a != b of two finite or infinite values, doubles on their bit patterns (as above).
+__device__ __forceinline__ bool differs(float a, float b) { return a != b; }
+__device__ __forceinline__ bool differs(double a, double b) {
+  const unsigned long long x = (unsigned long long)__double_as_longlong(a), z = (unsigned long long)__double_as_longlong(b);
+  return x != z && ((x | z) << 1) != 0;  // +0 equals -0; equal NaN patterns need no store
+}
+
 // Thread groups that cooperate on one block: the whole CTA, or one warp.
 struct CtaGroup {
   static constexpr int kSize = 0;  // size known at run time only

@@ -617,7 +617,10 @@ struct RefGeo {
 // Sec. 2.3: the synchronised mother tile is upsampled by the 4th-order
 // interpolating prediction and split into 2^d children (one treecode digit
 // appended); children are placed in the new active list in Hilbert order.
-// 2D blocks; 3D ones are refined by k_refine3 (mr_adv3.cuh).
+// 2D blocks; 3D ones are refined by k_refine3 (mr_adv3.cuh).  One CTA per mother
+// and variable: with the four variables of a mother in one CTA, 376 mothers of 33^2
+// nodes were 1.2 waves of 304 CTAs (335 us); 216 us with 1504 CTAs of a quarter
+// of the shared memory.
 template <int B, typename TS, int NT>
 __global__ void __launch_bounds__(NT, NT <= 128 ? 8 : 4) k_refine(PoolView pv, TS* __restrict__ y) {
   pdl_enter();
@@ -628,8 +631,8 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 8 : 4) k_refine(PoolView pv, T
   RingD<D>& R = *smem_as<RingD<D>>(0);
   __shared__ int cslot[8];
   TS* tile = smem_as<TS>(kRingBytesD<D>);
-  TS* cbox = tile + pv.nvar * Bx::TILE;
-  TS* scr = cbox + pv.nvar * Bx::CBOX;  // gather scratch, then the x pass of the upsampling
+  TS* cbox = tile + Bx::TILE;
+  TS* scr = cbox + Bx::CBOX;  // gather scratch, then the x pass of the upsampling
   TS* X = scr;
   const int nact = pv.cnt->n_act;
   const int n_alloc = pv.cnt->n_alloc, n_free = pv.cnt->n_free;
@@ -639,23 +642,30 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 8 : 4) k_refine(PoolView pv, T
   }
   if (n_alloc == 0) return;  // no block refines: the list stays as it is
   const int nv = pv.nvar;
-  for (int p = blockIdx.x; p < nact; p += gridDim.x) {
+  for (int64_t it = blockIdx.x; it < (int64_t)nact * nv; it += gridDim.x) {
+    const int p = (int)(it / nv), v = (int)(it % nv);
     const int slot = pv.act[p];
     const int e = pv.eoff[2 * p], a = pv.eoff[2 * p + 1];
     if (pv.flag[slot] != 1) {
-      if (threadIdx.x == 0) pv.act_next[e] = slot;
+      if (v == 0 && threadIdx.x == 0) pv.act_next[e] = slot;
       continue;
     }
+    // variable v as the only variable of blocks nvar * vs apart
+    PoolView pv1 = pv;
+    pv1.nvar = 1;
+    pv1.vs = pv.vs * nv;
+    const TS* yv = y + v * pv.vs;
     const BlockInfo b = load_block(pv, slot);
     const TreeDev& td = pv.trees[b.tree];
     build_ring<D, B>(pv, td, b, R);
     __syncthreads();
-    fill_tile<D, B, TS, TS, 1>(pv, b, y, y, tile, false, R, cbox, scr);
-    if (threadIdx.x == 0) {
+    fill_tile<D, B, TS, TS, 1>(pv1, b, yv, (TS*)yv, tile, false, R, cbox, scr);
+    if (threadIdx.x < Gm::NCH) cslot[threadIdx.x] = pv.freelist[n_free - n_alloc + a + threadIdx.x];
+    __syncthreads();
+    if (v == 0 && threadIdx.x == 0) {
       uint64_t key[8];
       int32_t cc[8][3];
       for (int ch = 0; ch < Gm::NCH; ++ch) {
-        cslot[ch] = pv.freelist[n_free - n_alloc + a + ch];
         for (int ax = 0; ax < 3; ++ax)
           cc[ch][ax] = ax < D ? (int32_t)(2 * b.c[ax] + ((ch >> ax) & 1)) : 0;
         key[ch] = block_key<D>(cc[ch], b.lvl + 1, td.Jmax);
@@ -673,41 +683,33 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 8 : 4) k_refine(PoolView pv, T
       }
     }
     __syncthreads();
-    // Separable upsampling, per variable: X = prediction along x on the
-    // mother's rows (y in [-1, B]), then y per child node -- the operations of
-    // the tensor product in the same order.
-    for (int v = 0; v < nv; ++v) {
-      const TS* tv = tile + v * Bx::TILE;
-      for (int idx = threadIdx.x; idx < RG::NX; idx += blockDim.x) {
-        const int ox = idx % RG::NF, jy = idx / RG::NF - 1;
-        const int fl = ox >> 1;
-        X[idx] = (ox & 1) ? dd4(tv[Bx::tix(fl - 1, jy, 0)], tv[Bx::tix(fl, jy, 0)], tv[Bx::tix(fl + 1, jy, 0)],
-                                tv[Bx::tix(fl + 2, jy, 0)])
-                          : tv[Bx::tix(fl, jy, 0)];
-      }
-      __syncthreads();
-      auto xr = [&](int ox, int jy) { return X[(jy + 1) * RG::NF + ox]; };
-      for (int idx = threadIdx.x; idx < Gm::NCH * Gm::NI; idx += blockDim.x) {
-        const int ch = idx / Gm::NI, q = idx % Gm::NI;
-        const int i = q % B, j = q / B;
-        const int ox = (ch & 1) * (B - 1) + i, oy = (ch >> 1) * (B - 1) + j;
-        const int fl = oy >> 1;
-        const TS val = (oy & 1) ? dd4(xr(ox, fl - 1), xr(ox, fl), xr(ox, fl + 1), xr(ox, fl + 2)) : xr(ox, fl);
-        y[((int64_t)cslot[ch] * nv + v) * pv.vs + q] = val;
-      }
-      __syncthreads();
+    // Separable upsampling: X = prediction along x on the mother's rows (y in
+    // [-1, B]), then y per child node -- the operations of the tensor product in
+    // the same order.
+    for (int idx = threadIdx.x; idx < RG::NX; idx += blockDim.x) {
+      const int ox = idx % RG::NF, jy = idx / RG::NF - 1;
+      const int fl = ox >> 1;
+      X[idx] = (ox & 1) ? dd4(tile[Bx::tix(fl - 1, jy, 0)], tile[Bx::tix(fl, jy, 0)], tile[Bx::tix(fl + 1, jy, 0)],
+                              tile[Bx::tix(fl + 2, jy, 0)])
+                        : tile[Bx::tix(fl, jy, 0)];
     }
+    __syncthreads();
+    auto xr = [&](int ox, int jy) { return X[(jy + 1) * RG::NF + ox]; };
+    for (int idx = threadIdx.x; idx < Gm::NCH * Gm::NI; idx += blockDim.x) {
+      const int ch = idx / Gm::NI, q = idx % Gm::NI;
+      const int i = q % B, j = q / B;
+      const int ox = (ch & 1) * (B - 1) + i, oy = (ch >> 1) * (B - 1) + j;
+      const int fl = oy >> 1;
+      const TS val = (oy & 1) ? dd4(xr(ox, fl - 1), xr(ox, fl), xr(ox, fl + 1), xr(ox, fl + 2)) : xr(ox, fl);
+      y[((int64_t)cslot[ch] * nv + v) * pv.vs + q] = val;
+    }
+    __syncthreads();
   }
 }
 
 // ---------------------------------------------------------------- details ----
-// Sec. 2.3: D = B - P(R(B)) on the synchronised tile (R keeps even tile nodes,
-// ghosts included; P predicts the odd ones).  Per block and variable the
-// largest |d| (warp-shuffle max, then across warps) and the largest |q_v|.
-// P is evaluated separably in the fixed order x, then y, then z: the x pass
-// over all coarse rows is stored in shared memory (X), the y and z passes run
-// per point; every output sees the same operations as the point-wise tensor
-// product.
+// Common parts of the details kernels (k_details2 in mr_det2.cuh, k_details3 in
+// mr_adv3.cuh).
 // The FP32 maximum m32 is within E of the FP64 one, and m32 + E < eps or
 // m32 - E >= eps holds in exact arithmetic: the sum is rounded up and compared
 // with eps rounded down, the difference rounded down and compared with eps
@@ -716,11 +718,35 @@ __device__ __forceinline__ bool certain_vs_eps(float m32, float E, const TreeDev
   return __fadd_ru(m32, E) < td.epsf[0] || __fsub_rd(m32, E) >= td.epsf[1];
 }
 
-template <int B>
-struct DetGeo {
-  static constexpr int NC = (B + 1) / 2 + 2;  // coarse rows -1 .. (B+1)/2
-  static constexpr int NX = NC * B;
+// Largest |value| added, NaN ignored (as fmax does).  FP64 values are compared
+// on their bit patterns, which order as the magnitudes do: a comparison of
+// doubles would take the FP64 pipe, the bound of the FP64 details.
+template <typename T>
+struct AbsMax {
+  T m = T(0);
+  __device__ __forceinline__ void add(T v) { m = fmax(m, (T)fabs(v)); }
+  __device__ __forceinline__ T get() const { return m; }
 };
+template <>
+struct AbsMax<double> {
+  long long m = 0;
+  __device__ __forceinline__ void add(double v) {
+    const long long b = __double_as_longlong(v) & 0x7fffffffffffffffLL;
+    if (b > m && b <= 0x7ff0000000000000LL) m = b;
+  }
+  __device__ __forceinline__ double get() const { return __longlong_as_double(m); }
+};
+
+// Maximum over the warp of non-negative values (not NaN), on their bit patterns.
+__device__ __forceinline__ float warp_max_pos(float v) {
+  return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+}
+__device__ __forceinline__ double warp_max_pos(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const unsigned hi = (unsigned)(b >> 32), top = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned lo = __reduce_max_sync(0xffffffffu, hi == top ? (unsigned)b : 0u);
+  return __longlong_as_double((long long)(((unsigned long long)top << 32) | lo));
+}
 
 // Maximum of v over the CTA (warp shuffles, then one value per warp in red);
 // every thread gets the result.  In the value's own type: FP64 operations are
@@ -756,456 +782,6 @@ __device__ __forceinline__ void block_max3(A& a, Bt& b, Ct& c, A* ra, Bt* rb, Ct
     b = fmax(b, rb[w]);
     c = fmax(c, rc[w]);
   }
-}
-
-// 2D detail index tables (per CTA, shared memory): the x pass on coarse rows
-// yc in [-1, NC - 2] (entry (yc + 1) B + x: tile index of its first source node,
-// x odd = 4 sources two nodes apart) and the odd interior points in row-major
-// order (tile index, first x-pass entry of the y pass, j odd = 4 entries B apart).
-template <int B>
-struct DetTab {
-  using Bx = Box<2, B, 2>;
-  using DG = DetGeo<B>;
-  static constexpr int NODD = B * B - ((B + 1) / 2) * ((B + 1) / 2);
-  static constexpr int INTS = DG::NX + NODD;
-  static_assert(Bx::NPTS < (1 << 12) && DG::NX < (1 << 12), "table entries fit their fields");
-  __device__ static void build(int32_t* xtab, int32_t* otab) {
-    for (int idx = threadIdx.x; idx < DG::NX; idx += blockDim.x) {
-      const int x = idx % B, yy = 2 * (idx / B - 1);
-      const int odd = x & 1;
-      const int b0 = odd ? Bx::tix(x - 3, yy, 0) : Bx::tix(x, yy, 0);
-      xtab[idx] = b0 | (odd << 16);
-    }
-    for (int k = threadIdx.x; k < NODD; k += blockDim.x) {
-      // rows j even hold (B - 1) / 2 odd points (odd i), rows j odd hold B
-      const int per2 = (B - 1) / 2 + B;
-      const int jp = k / per2, r = k % per2;
-      int i, j;
-      if (r < (B - 1) / 2) { j = 2 * jp; i = 2 * r + 1; }
-      else { j = 2 * jp + 1; i = r - (B - 1) / 2; }
-      const int jodd = j & 1;
-      const int xb = jodd ? ((j - 1) / 2) * B + i : (j / 2 + 1) * B + i;
-      otab[k] = Bx::tix(i, j, 0) | (xb << 12) | (jodd << 24);
-    }
-  }
-  // block maximum of |d| in type A over one variable's tile tv (G: CTA or warp;
-  // XA: NX values of scratch), the same operations as the point-wise evaluation
-  template <typename A, typename TV, typename G>
-  __device__ static A max_detail(const int32_t* xtab, const int32_t* otab, const TV* tv, A* XA, G g) {
-    for (int idx = g.rank(); idx < DG::NX; idx += g.size()) {
-      const int e = xtab[idx];
-      const TV* t0 = tv + (e & 0xffff);
-      XA[idx] = (e >> 16) ? dd4((A)t0[0], (A)t0[2], (A)t0[4], (A)t0[6]) : (A)t0[0];
-    }
-    g.sync();
-    A md = A(0);
-    for (int k = g.rank(); k < NODD; k += g.size()) {
-      const int e = otab[k];
-      const A val = (A)tv[e & 0xfff];
-      const A* xa = XA + ((e >> 12) & 0xfff);
-      const A pr = (e >> 24) ? dd4(xa[0], xa[B], xa[2 * B], xa[3 * B]) : xa[0];
-      md = fmax(md, (A)fabs(val - pr));
-    }
-    return md;
-  }
-  // the same, and from the same sweeps (per thread, not reduced): the largest
-  // |value| of the interior (mq; the odd points of the second sweep and the
-  // even-even interior nodes of the first) with a non-finite test (bad), and
-  // the largest |value| of the coarse lattice the first sweep reads (mt)
-  template <typename A, typename TV, typename G>
-  __device__ static A max_detail_ex(const int32_t* xtab, const int32_t* otab, const TV* tv, A* XA, G g, TV& mq,
-                                    float& mt, bool& bad) {
-    for (int idx = g.rank(); idx < DG::NX; idx += g.size()) {
-      const int e = xtab[idx];
-      const TV* t0 = tv + (e & 0xffff);
-      if (e >> 16) {
-        const TV a = t0[0], b = t0[2], c = t0[4], d = t0[6];
-        mt = fmaxf(fmaxf(mt, fmaxf(fabsf((float)a), fabsf((float)b))), fmaxf(fabsf((float)c), fabsf((float)d)));
-        XA[idx] = dd4((A)a, (A)b, (A)c, (A)d);
-      } else {
-        const TV a = t0[0];
-        mt = fmaxf(mt, fabsf((float)a));
-        const int row = idx / B;  // coarse row + 1: interior rows 1 .. (B + 1) / 2
-        if (row >= 1 && row <= (B + 1) / 2) {
-          mq = fmax(mq, (TV)fabs(a));
-          bad |= !isfinite(a);
-        }
-        XA[idx] = (A)a;
-      }
-    }
-    g.sync();
-    A md = A(0);
-    for (int k = g.rank(); k < NODD; k += g.size()) {
-      const int e = otab[k];
-      const TV tq = tv[e & 0xfff];
-      mq = fmax(mq, (TV)fabs(tq));
-      bad |= !isfinite(tq);
-      const A val = (A)tq;
-      const A* xa = XA + ((e >> 12) & 0xfff);
-      const A pr = (e >> 24) ? dd4(xa[0], xa[B], xa[2 * B], xa[3 * B]) : xa[0];
-      md = fmax(md, (A)fabs(val - pr));
-    }
-    return md;
-  }
-};
-
-// Shared memory of k_details after the ring and the tile: the coarse box and
-// prediction scratch of the gather, reused once the tile is complete for the x
-// pass of the prediction.
-template <int B, typename TT, typename TD>
-struct DetSmem {
-  using Bx = Box<2, B, 2>;
-  static constexpr size_t FILL = sizeof(TT) * (Bx::CBOX + Bx::SCR);  // per variable
-  static constexpr size_t PASS = (sizeof(TD) > 4 ? sizeof(TD) : 4) * DetGeo<B>::NX;
-  __host__ __device__ static size_t region(int nv) { return FILL * nv > PASS ? FILL * nv : PASS; }
-};
-
-// 2D blocks; the 3D details are k_details3 (mr_adv3.cuh).
-template <int B, typename TS, typename TD, int NT, typename TT = TS>
-__global__ void __launch_bounds__(NT, NT <= 128 ? 8 : 4) k_details(PoolView pv, TS* __restrict__ y) {
-  pdl_enter();
-  constexpr int D = 2;
-  using Gm = Geo<D, B>;
-  using Bx = Box<D, B, 2>;  // prediction from even nodes reaches two nodes
-  using DG = DetGeo<B>;
-  RingD<D>& R = *smem_as<RingD<D>>(0);
-  __shared__ double red[2][32];
-  TT* tile = smem_as<TT>(kRingBytesD<D>);  // tile type (TS or FP32); TD is the decision type
-  TT* cbox = tile + pv.nvar * Bx::TILE;
-  // gather scratch, reused for the passes once the tile is complete
-  TT* scr = cbox + pv.nvar * Bx::CBOX;
-  using DS = DetSmem<B, TT, TD>;
-  TD* X = reinterpret_cast<TD*>((reinterpret_cast<uintptr_t>(cbox) + 15) & ~(uintptr_t)15);
-  const int nact = pv.cnt->n_round;
-  const int nv = pv.nvar;
-  const bool all_blocks = pv.cnt->first_round != 0;
-  const int prev = pv.cnt->round_id - 1;
-  __shared__ int dirty;
-  using PL = Plan<D>;
-  __shared__ int32_t snb[PL::NB];
-  __shared__ int64_t snbo[PL::NB];  // pool offsets of the neighbours
-  __shared__ int32_t splan[2][PL::INTS];
-  // the stage plans are used while the tree is the one they were built for
-  // (the first round after the RK stages); the next block's plan is fetched
-  // while a block is processed
-  const bool plan_ok = pv.cnt->plan_topo == pv.cnt->topo;
-  const size_t xbytes = DS::region(nv);
-  int32_t* gtab = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(X) + ((xbytes + 15) & ~(size_t)15));
-  int32_t* xtab = gtab + Bx::NPTS;  // detail tables
-  int32_t* otab = xtab + DG::NX;
-  build_gtab<D, B, 2>(gtab);
-  DetTab<B>::build(xtab, otab);
-  // CTA-local work count and threshold scales (one atomic per CTA, not per block)
-  unsigned long long ndet = 0;
-  __shared__ double csv[kMaxVar];
-  __shared__ int csv_tree;
-  if (threadIdx.x < kMaxVar) csv[threadIdx.x] = 0.0;
-  if (threadIdx.x == 0) csv_tree = -1;
-  auto flush_csv = [&]() {
-    if (csv_tree >= 0 && threadIdx.x < nv && csv[threadIdx.x] > 0.0)
-      atomic_max_pos(&pv.svar[csv_tree * nv + threadIdx.x], csv[threadIdx.x]);
-  };
-  if (plan_ok && blockIdx.x < nact && threadIdx.x < PL::INTS)
-    splan[0][threadIdx.x] = pv.plan[(int64_t)blockIdx.x * PL::INTS + threadIdx.x];
-  __syncthreads();
-  int buf = 0;
-  for (int p = blockIdx.x; p < nact; p += gridDim.x, buf ^= 1) {
-    const int pn = p + gridDim.x;
-    int32_t pre = 0;
-    if (plan_ok && pn < nact && threadIdx.x < PL::INTS) pre = pv.plan[(int64_t)pn * PL::INTS + threadIdx.x];
-    BlockInfo b;
-    int q = 0;
-    if (plan_ok) {
-      b = plan_block<D>(splan[buf]);
-      q = threadIdx.x < PL::NB ? splan[buf][PL::NBO + threadIdx.x] : b.slot;
-    } else {
-      b = load_block(pv, pv.act[p]);
-      // equal-level neighbours, one lookup per thread: uniform when all exist
-      q = b.slot;
-      if (threadIdx.x < PL::NB) {
-        const int n = threadIdx.x;
-        const int o[2] = {n % 3 - 1, n / 3 - 1};
-        if (o[0] != 0 || o[1] != 0) {
-          const TreeDev& tdl = pv.trees[b.tree];
-          const int64_t cn[3] = {b.c[0] + o[0], b.c[1] + o[1], 0};
-          q = tab_get<D>(pv, tdl, b.lvl, cn);
-        }
-      }
-    }
-    const TreeDev& td = pv.trees[b.tree];
-    if (pv.norm_kind == 1 && b.tree != csv_tree) {  // block of another tree: flush the scales
-      flush_csv();
-      __syncthreads();
-      if (threadIdx.x < kMaxVar) csv[threadIdx.x] = 0.0;
-      if (threadIdx.x == 0) csv_tree = b.tree;
-    }
-    if (threadIdx.x < PL::NB) {
-      snb[threadIdx.x] = q;
-      snbo[threadIdx.x] = (int64_t)q * nv * pv.vs;
-    }
-    if (threadIdx.x == 0) dirty = all_blocks ? 1 : 0;
-    const bool uni = __syncthreads_and(q >= 0);
-    if (uni) {
-      // the ring's leaves are the block and its 3^d - 1 equal-level neighbours
-      if (!all_blocks && threadIdx.x < PL::NB && pv.stamp[q] == prev) dirty = 1;
-    } else if (plan_ok && all_blocks) {
-      // every block is evaluated and the tree is the stage plan's: its
-      // class-box owner table is ready
-      load_regions<D, CtaGroup>(pv, p, R);
-    } else {
-      build_ring<D, B>(pv, td, b, R);
-      __syncthreads();
-      if (!all_blocks && threadIdx.x < Gm::NR && R.slot[threadIdx.x] >= 0 &&
-          pv.stamp[R.slot[threadIdx.x]] == prev)
-        dirty = 1;
-    }
-    __syncthreads();
-    if (!dirty) {
-      // No leaf of the ring changed in the previous round: the synchronised
-      // tile, hence the details and norms stored for this block, are unchanged.
-      if (pv.norm_kind == 1 && threadIdx.x < nv)
-        csv[threadIdx.x] = fmax(csv[threadIdx.x], pv.bmax[(int64_t)b.slot * nv + threadIdx.x]);
-      if (plan_ok && pn < nact && threadIdx.x < PL::INTS) splan[buf ^ 1][threadIdx.x] = pre;
-      __syncthreads();
-      continue;
-    }
-    ndet += 1;
-    const int64_t own = (int64_t)b.slot * nv * pv.vs;
-    if (uni && nv == 1) {
-      gather_table<D, B, 2, 1, TS, TT>(pv, own, snbo, gtab, y, y, tile, true);
-    } else if (uni && nv == 4) {
-      gather_table<D, B, 2, 4, TS, TT>(pv, own, snbo, gtab, y, y, tile, true);
-    } else {
-      if (uni) {
-        build_ring<D, B>(pv, td, b, R);
-        __syncthreads();
-      }
-      const bool ready = !uni && plan_ok && all_blocks;
-      fill_tile<D, B, TS, TT, 2>(pv, b, y, y, tile, true, R, cbox, scr, ready);
-    }
-    __syncthreads();
-    // Block maximum of |d| over the interior with arithmetic type A: x pass on
-    // the coarse rows into X, then y per odd node.  With EX the same sweeps also
-    // give the interior's largest |value| and non-finite test (ex_mq, bad) and
-    // the coarse lattice's largest |value| (ex_mt), reduced with the detail
-    // maximum in one step.
-    TT ex_mq = TT(0);
-    float ex_mt = 0.f;
-    bool bad = false;
-    auto pass = [&](auto tag, const TT* tv, auto exc) -> decltype(tag) {
-      using A = decltype(tag);
-      A* XA = reinterpret_cast<A*>(X);
-      if constexpr (decltype(exc)::value) {
-        TT mq = TT(0);
-        float mt = 0.f;
-        A md = DetTab<B>::template max_detail_ex<A>(xtab, otab, tv, XA, CtaGroup{}, mq, mt, bad);
-        block_max3<A, TT, float>(md, mq, mt, reinterpret_cast<A*>(red[0]), reinterpret_cast<TT*>(red[1]),
-                                 reinterpret_cast<float*>(red[1]) + 32);
-        ex_mq = mq;
-        ex_mt = mt;
-        return md;
-      } else {
-        const A md = DetTab<B>::template max_detail<A>(xtab, otab, tv, XA, CtaGroup{});
-        return block_max<A>(md, reinterpret_cast<A*>(red[0]));
-      }
-    };
-    for (int v = 0; v < nv; ++v) {
-      const TT* tv = tile + v * Bx::TILE;
-      constexpr bool cert = sizeof(TT) == 4 && sizeof(TD) == 8;
-      // the first pass's sweeps (x pass and odd points) give the
-      // detail maximum, the interior's largest |value| (exact in its type), the
-      // non-finite test (any non-finite value makes the block norm NaN) and,
-      // for the certified FP32 decision, the largest |value| the evaluation
-      // reads (interior and coarse lattice), all in one CTA reduction
-      using A0 = std::conditional_t<cert, float, TD>;
-      const A0 m0 = pass(A0(0), tv, std::true_type{});
-      const TT mqt = ex_mq;
-      double md = 0.0;  // thread 0's value is stored
-      if constexpr (cert) {
-        // FP32 values, FP64 decision: the FP32 evaluation differs from the FP64
-        // one by at most ~20 u max|tile| (u = 2^-24, x/y/z passes of the
-        // 4-point rule and the subtraction); where its maximum is farther than
-        // 32 u max|tile| from eps the threshold decision (Sec. 2.3) is the
-        // FP64 one, otherwise the block is evaluated again in FP64.
-        const float mt = fmaxf(ex_mt, (float)mqt);
-        const float E = 0x1p-19f * mt + 1e-37f;
-        if (pv.norm_kind == 0 && certain_vs_eps(m0, E, td)) {
-          if (threadIdx.x == 0) md = (double)m0;
-        } else {
-          md = pass(double(0), tv, std::false_type{});
-        }
-      } else {
-        md = (double)m0;
-      }
-      if (threadIdx.x == 0) {
-        const double mq = (double)mqt;
-        pv.md[(int64_t)b.slot * nv + v] = md;
-        pv.bmax[(int64_t)b.slot * nv + v] = mq;
-        if (pv.norm_kind == 1) csv[v] = fmax(csv[v], mq);
-      }
-      __syncthreads();
-    }
-    if (plan_ok && pn < nact && threadIdx.x < PL::INTS) splan[buf ^ 1][threadIdx.x] = pre;
-    if (__syncthreads_or(bad) && threadIdx.x == 0)
-      pv.md[(int64_t)b.slot * nv] = __longlong_as_double(0x7ff8000000000000LL);
-  }
-  __syncthreads();
-  if (pv.norm_kind == 1) flush_csv();
-  if (threadIdx.x == 0 && ndet) atomicAdd(&pv.cnt->det_blocks, ndet);
-}
-
-// 2D details with one warp per block (single-variable fields without
-// normalisation): the same evaluation as k_details, with warp-level
-// synchronisation and reductions, for grids with many blocks.
-template <int B, typename TS, typename TD, int NT>
-struct DetW {
-  using Bx = Box<2, B, 2>;
-  using DG = DetGeo<B>;
-  static constexpr int NW = NT / 32;
-  static constexpr size_t GTAB = (4 * Bx::NPTS + 15) / 16 * 16;
-  static constexpr size_t TABS = (4 * DetTab<B>::INTS + 15) / 16 * 16;  // detail index tables
-  static constexpr size_t XB = sizeof(TS) * Bx::SCR > sizeof(TD) * DG::NX ? sizeof(TS) * Bx::SCR : sizeof(TD) * DG::NX;
-  static constexpr size_t TB = (kRingBytesD<2> + sizeof(TS) * (Bx::TILE + Bx::CBOX) + 15) / 16 * 16;
-  static constexpr size_t WAREA = TB + (XB + 15) / 16 * 16;
-  static constexpr size_t SMEM = GTAB + TABS + NW * WAREA;
-};
-
-template <typename T>
-__device__ __forceinline__ T warp_max(T v) {
-  for (int s = 16; s > 0; s >>= 1) v = fmax(v, (T)__shfl_xor_sync(0xffffffffu, v, s));
-  return v;
-}
-
-template <int B, typename TS, typename TD, int NT>
-__global__ void __launch_bounds__(NT, 1024 / NT) k_details_w(PoolView pv, TS* __restrict__ y) {
-  pdl_enter();
-  using Gm = Geo<2, B>;
-  using Bx = Box<2, B, 2>;
-  using DG = DetGeo<B>;
-  using PL = Plan<2>;
-  using DW = DetW<B, TS, TD, NT>;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned char* sm = smem_as<unsigned char>(0);
-  int32_t* gtab = reinterpret_cast<int32_t*>(sm);
-  int32_t* xtab = reinterpret_cast<int32_t*>(sm + DW::GTAB);
-  int32_t* otab = xtab + DG::NX;
-  unsigned char* wa = sm + DW::GTAB + DW::TABS + warp * DW::WAREA;
-  RingD<2>& R = *reinterpret_cast<RingD<2>*>(wa);
-  TS* tile = reinterpret_cast<TS*>(wa + kRingBytesD<2>);
-  TS* cbox = tile + Bx::TILE;
-  TS* scr = reinterpret_cast<TS*>(wa + DW::TB);  // gather scratch, then the x pass
-  __shared__ int64_t snbo[DW::NW][PL::NB];
-  build_gtab<2, B, 2>(gtab);
-  DetTab<B>::build(xtab, otab);
-  __syncthreads();
-  const int nact = pv.cnt->n_round;
-  const bool all_blocks = pv.cnt->first_round != 0;
-  const int prev = pv.cnt->round_id - 1;
-  const bool plan_ok = pv.cnt->plan_topo == pv.cnt->topo;
-  const int gw = blockIdx.x * DW::NW + warp, nwt = gridDim.x * DW::NW;
-  unsigned ndet = 0;
-  int32_t cur = (plan_ok && gw < nact && lane < PL::INTS) ? pv.plan[(int64_t)gw * PL::INTS + lane] : 0;
-  for (int p = gw; p < nact; p += nwt) {
-    const int pn = p + nwt;
-    const int32_t nxt = (plan_ok && pn < nact && lane < PL::INTS) ? pv.plan[(int64_t)pn * PL::INTS + lane] : 0;
-    BlockInfo b;
-    int q;
-    if (plan_ok) {
-      b.slot = __shfl_sync(0xffffffffu, cur, 0);
-      const int meta = __shfl_sync(0xffffffffu, cur, 1);
-      b.lvl = meta & 255;
-      b.tree = (meta >> 8) & 0xffff;
-      b.c[0] = __shfl_sync(0xffffffffu, cur, 2);
-      b.c[1] = __shfl_sync(0xffffffffu, cur, 3);
-      b.c[2] = 0;
-      const int32_t qq = __shfl_sync(0xffffffffu, cur, PL::NBO + (lane < PL::NB ? lane : 0));
-      q = lane < PL::NB ? qq : b.slot;
-    } else {
-      b = load_block(pv, pv.act[p]);
-      q = b.slot;
-      if (lane < PL::NB && lane != 4) {
-        const int64_t cn[3] = {b.c[0] + lane % 3 - 1, b.c[1] + lane / 3 - 1, 0};
-        q = tab_get<2>(pv, pv.trees[b.tree], b.lvl, cn);
-      }
-    }
-    const TreeDev& td = pv.trees[b.tree];
-    const bool uni = __all_sync(0xffffffffu, q >= 0);
-    bool ring = false;
-    bool dirty = all_blocks;
-    if (!all_blocks) {
-      if (uni) {
-        dirty = __any_sync(0xffffffffu, lane < PL::NB && pv.stamp[q] == prev);
-      } else {
-        build_ring<2, B, WarpGroup>(pv, td, b, R);
-        __syncwarp();
-        ring = true;
-        dirty = __any_sync(0xffffffffu, lane < Gm::NR && R.slot[lane] >= 0 && pv.stamp[R.slot[lane]] == prev);
-      }
-    }
-    if (dirty) {
-      ++ndet;
-      const int64_t own = (int64_t)b.slot * pv.vs;
-      if (uni) {
-        if (lane < PL::NB) snbo[warp][lane] = (int64_t)q * pv.vs;
-        __syncwarp();
-        gather_table<2, B, 2, 1, TS, TS, WarpGroup>(pv, own, snbo[warp], gtab, y, y, tile, true);
-      } else {
-        const bool ready = !ring && plan_ok && all_blocks;  // the stage plan's owner table
-        if (ready) load_regions<2, WarpGroup>(pv, p, R);
-        else if (!ring) build_ring<2, B, WarpGroup>(pv, td, b, R);
-        __syncwarp();
-        fill_tile<2, B, TS, TS, 2, WarpGroup>(pv, b, y, y, tile, true, R, cbox, scr, ready);
-      }
-      __syncwarp();
-      // the x pass over the coarse rows, then the y pass and the detail at
-      // each odd point, through the index tables (same operations as k_details)
-      auto pass = [&](auto tag) -> decltype(tag) {
-        using A = decltype(tag);
-        A* XA = reinterpret_cast<A*>(scr);
-        A md = DetTab<B>::template max_detail<A>(xtab, otab, tile, XA, WarpGroup{});
-        md = warp_max(md);
-        __syncwarp();
-        return md;
-      };
-      // largest |value| over the interior (stored, and the NaN check) and, for
-      // the certified FP32 evaluation, over the whole tile: one sweep, the
-      // interior flag from the gather table
-      constexpr bool cert = sizeof(TS) == 4 && sizeof(TD) == 8;
-      TS mqs = TS(0), mts = TS(0);
-      bool bad = false;
-      for (int qn = lane; qn < Bx::TILE; qn += 32) {
-        const TS sv = tile[qn];
-        const TS av = (TS)fabs(sv);
-        if (cert) mts = fmax(mts, av);
-        if ((gtab[qn] >> 21) & 1) {
-          mqs = fmax(mqs, av);
-          bad |= !isfinite(sv);
-        }
-      }
-      mqs = warp_max(mqs);
-      double md = 0.0;  // lane 0's value is stored
-      if constexpr (cert) {
-        // as in k_details: FP32 evaluation, FP64 only within the rounding bound of eps
-        const float m32 = pass(float(0));
-        const float E = 0x1p-19f * warp_max((float)mts) + 1e-37f;
-        if (certain_vs_eps(m32, E, td)) {
-          if (lane == 0) md = (double)m32;
-        } else {
-          md = pass(double(0));
-        }
-      } else {
-        md = (double)pass(TD(0));
-      }
-      if (__any_sync(0xffffffffu, bad)) md = __longlong_as_double(0x7ff8000000000000LL);
-      if (lane == 0) {
-        pv.md[b.slot] = md;
-        pv.bmax[b.slot] = (double)mqs;
-      }
-      __syncwarp();
-    }
-    cur = nxt;
-  }
-  if (lane == 0 && ndet) atomicAdd(&pv.cnt->det_blocks, (unsigned long long)ndet);
 }
 
 // ---------------------------------------------------------------- coarsen ----

@@ -6,6 +6,7 @@
 #include <cstdio>
 
 #include "mr_adv3.cuh"
+#include "mr_det2.cuh"
 #include "mr_kernels.cuh"
 
 namespace mr {
@@ -232,8 +233,8 @@ struct RefineRun {
     } else {
       constexpr int threads = Threads<B>::value;
       using Bx = Box<2, B, 1>;
-      const size_t scr = (size_t)std::max<int64_t>((int64_t)pv.nvar * Bx::SCR, RefGeo<B>::NX);
-      go(k_refine<B, TS, threads>, threads, kRingBytesD<2> + sizeof(TS) * (pv.nvar * (Bx::TILE + Bx::CBOX) + scr));
+      constexpr int scr = Bx::SCR > RefGeo<B>::NX ? Bx::SCR : RefGeo<B>::NX;
+      go(k_refine<B, TS, threads>, threads, kRingBytesD<2> + sizeof(TS) * (Bx::TILE + Bx::CBOX + scr));
     }
   }
 };
@@ -279,7 +280,9 @@ struct DetailsRun {
                   cudaStream_t st) {
     auto go = [&](auto k, int threads, size_t smem) {
       prep_smem(k, smem);
-      launch_k(lc.pdl, k, persistent_grid(k, threads, smem, lc, lc.grid_mult), threads, smem, st, pv, (TS*)f.y);
+      // a multiple of 4: k_details2's groups keep their variable
+      const int grid = (persistent_grid(k, threads, smem, lc, lc.grid_mult) + 3) / 4 * 4;
+      launch_k(lc.pdl, k, grid, threads, smem, st, pv, (TS*)f.y);
       count_launch();
     };
     // FP64 details for the plain FP64 form or when asked for (thresholds below
@@ -289,20 +292,8 @@ struct DetailsRun {
       if (d64) go(k_details3<TS, double, TS>, Col3::NT, Det3Smem<TS, double>::BYTES);
       else go(k_details3<TS, float, float>, Col3::NT, Det3Smem<float, float>::BYTES);
     } else {
-      constexpr int threads = Threads<B>::value;
-      const bool warp_form = pv.nvar == 1 && pv.norm_kind == 0 && sizeof(TS) == 4 &&
-                             (lc.stage_form == 1 || (lc.stage_form < 0 && lc.n_hint >= 8 * lc.num_sms));
-      if (warp_form) {  // one warp per block
-        if (d64) go(k_details_w<B, TS, double, threads>, threads, DetW<B, TS, double, threads>::SMEM);
-        else go(k_details_w<B, TS, TS, threads>, threads, DetW<B, TS, TS, threads>::SMEM);
-        return;
-      }
-      using Bx = Box<2, B, 2>;
-      const size_t tt = d64 ? sizeof(TS) : 4;  // tile type: the state type, FP32 for FP32 details
-      const size_t region = d64 ? DetSmem<B, TS, double>::region(pv.nvar) : DetSmem<B, float, float>::region(pv.nvar);
-      const size_t smem = kRingBytesD<2> + tt * pv.nvar * Bx::TILE + 16 + region + 16 + 4 * (Bx::NPTS + DetTab<B>::INTS);
-      if (d64) go(k_details<B, TS, double, threads>, threads, smem);
-      else go(k_details<B, TS, float, threads, float>, threads, smem);
+      if (d64) go(k_details2<B, TS, double, TS>, Det2<B>::NT, Det2Smem<B, TS, double>::BYTES);
+      else go(k_details2<B, TS, float, float>, Det2<B>::NT, Det2Smem<B, float, float>::BYTES);
     }
   }
 };
