@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(256) k_cnn_infer(PoolView pv, const float* __r
 
 // ---------------------------------------------------- training (fwd + bwd) ---
 // Samples [s0, s0 + nb) of the dataset (index list idx), mean weighted BCE, one
-// sample at a time per CTA.  FP32 multiply-adds throughout (1.6 M per sample of
+// sample at a time per CTA.  FP32 throughout (1.6 M multiply-adds per sample of
 // 25^2).  Shared-memory reads bound the kernel (a load writes a register per lane,
 // a broadcast one too, so every loaded value has to meet several others), and
 // every pass is tiled in registers:
@@ -271,8 +271,14 @@ __global__ void __launch_bounds__(256) k_cnn_infer(PoolView pv, const float* __r
 // consecutive words.  Products with a zero gradient are left out (a non-finite
 // input under an inactive unit has no gradient).
 // 3000 samples of 25^2: 5890 us with one output value per thread and loop, now
-// 485 us (shared-memory pipe 89 % of peak).  Larger tiles (two pixels in conv1, four
+// 510 us (shared-memory pipe near 90 % of peak).  Larger tiles (two pixels in conv1, four
 // in conv2, two blocks in da1) read less but leave threads idle: 490-510 us.
+// a + w x, product and sum each rounded: the forward pass rounds as k_cnn_infer does,
+// term by term (padding adds exact zeros), so both take the same maxima and ReLU
+// branches, whatever the tiling; a different rounding would move gradients between
+// nearly equal maxima.
+__device__ __forceinline__ float mul_add(float w, float x, float a) { return __fadd_rn(a, __fmul_rn(w, x)); }
+
 template <int T>
 struct TrainGeo {
   using CG = CnnGeo<T>;
@@ -362,10 +368,10 @@ __global__ void __launch_bounds__(TrainGeo<T>::NT, TrainGeo<T>::MINB)
 #pragma unroll
           for (int o4 = 0; o4 < 4; ++o4) {
             const float4 wv = wp[o4];
-            a[4 * o4] = fmaf(wv.x, xv, a[4 * o4]);
-            a[4 * o4 + 1] = fmaf(wv.y, xv, a[4 * o4 + 1]);
-            a[4 * o4 + 2] = fmaf(wv.z, xv, a[4 * o4 + 2]);
-            a[4 * o4 + 3] = fmaf(wv.w, xv, a[4 * o4 + 3]);
+            a[4 * o4] = mul_add(wv.x, xv, a[4 * o4]);
+            a[4 * o4 + 1] = mul_add(wv.y, xv, a[4 * o4 + 1]);
+            a[4 * o4 + 2] = mul_add(wv.z, xv, a[4 * o4 + 2]);
+            a[4 * o4 + 3] = mul_add(wv.w, xv, a[4 * o4 + 3]);
           }
         }
       const int at = G::h1at(0, i + 1, j + 1);
@@ -400,10 +406,10 @@ __global__ void __launch_bounds__(TrainGeo<T>::NT, TrainGeo<T>::MINB)
 #pragma unroll
           for (int m = 0; m < 2; ++m) {
             const float hv = v[2 * m + tap / 3][tap % 3];
-            a[m][0] = fmaf(wv.x, hv, a[m][0]);
-            a[m][1] = fmaf(wv.y, hv, a[m][1]);
-            a[m][2] = fmaf(wv.z, hv, a[m][2]);
-            a[m][3] = fmaf(wv.w, hv, a[m][3]);
+            a[m][0] = mul_add(wv.x, hv, a[m][0]);
+            a[m][1] = mul_add(wv.y, hv, a[m][1]);
+            a[m][2] = mul_add(wv.z, hv, a[m][2]);
+            a[m][3] = mul_add(wv.w, hv, a[m][3]);
           }
         }
       }
@@ -427,10 +433,10 @@ __global__ void __launch_bounds__(TrainGeo<T>::NT, TrainGeo<T>::MINB)
         for (int tap = 0; tap < 9; ++tap) {
           const float hv = hp[(c * P2 + tap / 3) * P2 + tap % 3];
           const float4 wv = w3[(c * 9 + tap) * 4 + og];
-          a[0] = fmaf(wv.x, hv, a[0]);
-          a[1] = fmaf(wv.y, hv, a[1]);
-          a[2] = fmaf(wv.z, hv, a[2]);
-          a[3] = fmaf(wv.w, hv, a[3]);
+          a[0] = mul_add(wv.x, hv, a[0]);
+          a[1] = mul_add(wv.y, hv, a[1]);
+          a[2] = mul_add(wv.z, hv, a[2]);
+          a[3] = mul_add(wv.w, hv, a[3]);
         }
 #pragma unroll
       for (int o = 0; o < 4; ++o) h3[(4 * og + o) * T3 * T3 + pix] = fmaxf(a[o], 0.f);
@@ -454,7 +460,7 @@ __global__ void __launch_bounds__(TrainGeo<T>::NT, TrainGeo<T>::MINB)
     __syncthreads();
     float logit = *bl;
 #pragma unroll
-    for (int o = 0; o < kC; ++o) logit = fmaf(wl[o], z[o], logit);
+    for (int o = 0; o < kC; ++o) logit = mul_add(wl[o], z[o], logit);
     const float p = 1.f / (1.f + expf(-logit));
     const float dl = (yv * w_pos * (p - 1.f) + (1.f - yv) * p) / nb;
     if (t == 0) {
