@@ -14,15 +14,6 @@ struct Col3 {
   static constexpr int NREG = RingD<3>::NREG;
 };
 
-// (f[-2] - f[2]) + 8 (f[1] - f[-1]): the product with 8 is exact, so the fused
-// form rounds the same value once (one instruction less per derivative).
-__device__ __forceinline__ float d1_sum(float fm2, float fm1, float f1, float f2) {
-  return __fmaf_rn(8.f, f1 - fm1, fm2 - f2);
-}
-__device__ __forceinline__ double d1_sum(double fm2, double fm1, double f1, double f2) {
-  return __fma_rn(8.0, f1 - fm1, fm2 - f2);
-}
-
 // Owner of the nodes of column (i, j) in one class box: node k is at
 // at(k) in the field when node(k), else it lies between the owner's nodes.
 struct ColOwn {
@@ -580,6 +571,7 @@ __global__ void __launch_bounds__(Col3::NT, sizeof(TS) == 8 ? 2 : 3) k_details3(
   __shared__ int csv_tree;
   const int t = threadIdx.x;
   const int nact = pv.cnt->n_round;
+  if ((int)blockIdx.x >= nact) return;  // no block for this CTA (small grids)
   const bool all_blocks = pv.cnt->first_round != 0;
   const int prev = pv.cnt->round_id - 1;
   const bool plan_ok = pv.cnt->plan_topo == pv.cnt->topo;
@@ -911,7 +903,8 @@ __global__ void __launch_bounds__(Col3::NT, sizeof(TS) == 8 ? 2 : 3) k_refine3(P
   for (int it = blockIdx.x; it < 4 * nact; it += gridDim.x) {
     const int p = it >> 2, quad = it & 3, qx = quad & 1, qy = quad >> 1;
     const int slot = pv.act[p];
-    const int e0 = pv.eoff[2 * p], a0 = pv.eoff[2 * p + 1];
+    const int2 off = new_offset(pv, p);
+    const int e0 = off.x, a0 = off.y;
     if (pv.flag[slot] != 1) {
       if (quad == 0 && t == 0) pv.act_next[e0] = slot;
       continue;

@@ -40,7 +40,7 @@ struct mr_ctx_s {
   int32_t* plan = nullptr;  // S x 32: stage plans of the active blocks
   int4* regs = nullptr;     // S x (NREG + 1): class-box owner tables built with the plans
   int32_t *crd = nullptr, *act = nullptr, *act_next = nullptr, *freelist = nullptr, *tab = nullptr,
-          *cells = nullptr, *emit = nullptr, *eoff = nullptr, *partial = nullptr, *pos = nullptr;
+          *cells = nullptr, *emit = nullptr, *eoff = nullptr, *grp = nullptr, *gof = nullptr, *partial = nullptr, *pos = nullptr;
   uint64_t* hkey = nullptr;
   double *md = nullptr, *mdet = nullptr, *bmax = nullptr, *lat = nullptr, *svar = nullptr;
   float* latf = nullptr;
@@ -154,7 +154,7 @@ PoolView view(mr_ctx c) {
   v.lvl = c->lvl; v.tree = c->tree; v.crd = c->crd; v.hkey = c->hkey; v.f1 = c->f1;
   v.flag = c->flag; v.md = c->md; v.mdet = c->mdet; v.bmax = c->bmax; v.act = c->act;
   v.act_next = c->act_next; v.freelist = c->freelist; v.tab = c->tab; v.lat = c->lat; v.latf = c->latf;
-  v.svar = c->svar; v.cells = c->cells; v.emit = c->emit; v.eoff = c->eoff;
+  v.svar = c->svar; v.cells = c->cells; v.emit = c->emit; v.eoff = c->eoff; v.grp = c->grp; v.gof = c->gof;
   v.partial = c->partial; v.pos_of_slot = c->pos; v.cnt = c->cnt; v.stamp = c->stamp;
   v.plan = c->plan;
   v.regs = c->regs;
@@ -771,6 +771,8 @@ mr_status mr_create(const mr_params* p, const mr_tree_desc* trees, mr_ctx* out) 
     if ((e = dalloc(ctx, &ctx->cells, 2 * ctx->ncells))) return e;
     if ((e = dalloc(ctx, &ctx->emit, 2 * ctx->nscan))) return e;
     if ((e = dalloc(ctx, &ctx->eoff, 2 * ctx->nscan))) return e;
+    if ((e = dalloc(ctx, &ctx->grp, 2 * (S / 8 + 1)))) return e;
+    if ((e = dalloc(ctx, &ctx->gof, 2 * (S / 8 + 1)))) return e;
     if ((e = dalloc(ctx, &ctx->partial, 2 * (ctx->nscan / kScanChunk + 2)))) return e;
     if ((e = dalloc(ctx, &ctx->lat, ctx->nlat))) return e;
     if ((e = dalloc(ctx, &ctx->latf, ctx->nlat))) return e;

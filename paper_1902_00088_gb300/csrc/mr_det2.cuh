@@ -21,11 +21,22 @@ struct Det2 {
   static constexpr int GS = B == 17 ? 32 : 128;        // threads per item
   static constexpr int NT = 128, ITEMS = NT / GS;      // threads and items per CTA
   static constexpr int K = (NI + GS - 1) / GS;         // nodes per thread
+  static constexpr int NE = 4 * (B - 1);               // edge nodes
+  // edge node e: lower edge from x = 0, right edge upward, upper edge back, left edge down
+  __device__ static __forceinline__ void edge(int e, int& i, int& j) {
+    const int s = e / (B - 1), r = e % (B - 1);
+    i = s == 0 ? r : s == 1 ? B - 1 : s == 2 ? B - 1 - r : 0;
+    j = s == 0 ? 0 : s == 1 ? r : s == 2 ? B - 1 : B - 1 - r;
+  }
+  __device__ static __forceinline__ int edge_of(int i, int j) {  // -1: not an edge node
+    return j == 0 && i < B - 1 ? i : i == B - 1 && j < B - 1 ? B - 1 + j : j == B - 1 && i > 0 ? 3 * (B - 1) - i
+           : i == 0 ? 4 * (B - 1) - j : -1;
+  }
   // place of node x in a row: coarse nodes (even x) from 1, odd ones after them
   __host__ __device__ static constexpr int place(int x) { return (x & 1) ? NC + x / 2 : 1 + x / 2; }
 };
 
-template <int B, typename TT, typename TD>
+template <int B, typename TS, typename TT, typename TD>
 struct Det2Smem {
   using D2 = Det2<B>;
   static constexpr size_t TABS = (4 * (D2::NI + D2::NG) + 15) / 16 * 16;  // per CTA
@@ -34,20 +45,22 @@ struct Det2Smem {
   // x pass of the FP64 evaluation of FP32 values
   static constexpr size_t XD = sizeof(TD) > sizeof(TT) ? sizeof(TD) * D2::NC * D2::NO : 0;
   static constexpr size_t NB = 80;                                          // neighbours' pool offsets
-  static constexpr size_t ITEM = RING + W + (XD + 15) / 16 * 16 + NB;
+  static constexpr size_t EV = sizeof(TS) * D2::NE;  // edge values (a multiple of 16 bytes)
+  static constexpr size_t ITEM = RING + W + (XD + 15) / 16 * 16 + EV + NB;
   static constexpr size_t BYTES = TABS + D2::ITEMS * ITEM;
 };
 
 // Bound by instruction issue and latency (48 % of the issue slots used); 12 CTAs per SM
 // spill, 6 hide less latency: 8 CTAs of 4 warps.  Measured, before with one CTA (or warp) per block over the gathered and
-// predicted 21^2 tile, variable after variable: 65536 FP32 blocks of 17^2 104 -> 84 us;
-// 16384 blocks of 4 FP64 variables 165 -> 109 us; the rounds of an adaptive step with 64
-// trees 168 -> 120 us, with 33^2 blocks of 4 variables 443 -> 365 us.
+// predicted 21^2 tile, variable after variable: 65536 FP32 blocks of 17^2 104 -> 78 us;
+// 16384 blocks of 4 FP64 variables 165 -> 101 us; the rounds of an adaptive step with 64
+// trees 168 -> 94 us, with 33^2 blocks of 4 variables 443 -> 238 us (a third of it by
+// looking the owners of a block's edge nodes up apart from its own nodes).
 template <int B, typename TS, typename TD, typename TT>
 __global__ void __launch_bounds__(128, 8) k_details2(PoolView pv, TS* __restrict__ y) {
   pdl_enter();
   using D2 = Det2<B>;
-  using SM = Det2Smem<B, TT, TD>;
+  using SM = Det2Smem<B, TS, TT, TD>;
   using PL = Plan<2>;
   using G = std::conditional_t<D2::GS == 32, WarpGroup, CtaGroup>;
   constexpr int NC = D2::NC, NO = D2::NO, RP = D2::RP, NI = D2::NI, GS = D2::GS, K = D2::K;
@@ -61,14 +74,18 @@ __global__ void __launch_bounds__(128, 8) k_details2(PoolView pv, TS* __restrict
   TT* E = reinterpret_cast<TT*>(mem + SM::RING);
   TD* XD = reinterpret_cast<TD*>(mem + SM::RING + SM::W);
   int64_t* nbo = reinterpret_cast<int64_t*>(mem + SM::ITEM - SM::NB);
+  TS* ev = reinterpret_cast<TS*>(mem + SM::ITEM - SM::NB - SM::EV);
   __shared__ double red[4];
+  const int nact = pv.cnt->n_round, nv = pv.nvar;
+  if ((int64_t)blockIdx.x * D2::ITEMS >= (int64_t)nact * nv) return;  // no item for this CTA (small grids)
   // nodes: place in the work array | kind << 12 (0 coarse, 1 odd x on a coarse row, 2
-  // odd y) | upper edge in x << 14, in y << 15
+  // odd y) | upper edge in x << 14, in y << 15 | edge node << 16 (0: none, else + 1)
   for (int q = threadIdx.x; q < NI; q += blockDim.x) {
     const int i = q % B, j = q / B;
     const int row = (j & 1) ? j / 2 : j / 2 + 1;  // first row of the y pass, or the node's own
     const int kind = (j & 1) ? 2 : (i & 1);
-    ntab[q] = (row * RP + D2::place(i)) | (kind << 12) | (i == B - 1 ? 1 << 14 : 0) | (j == B - 1 ? 1 << 15 : 0);
+    ntab[q] = (row * RP + D2::place(i)) | (kind << 12) | (i == B - 1 ? 1 << 14 : 0) | (j == B - 1 ? 1 << 15 : 0) |
+              ((D2::edge_of(i, j) + 1) << 16);
   }
   // ghost nodes: place | neighbour << 12 | offset in that neighbour (of a uniform
   // neighbourhood) << 16
@@ -102,7 +119,6 @@ __global__ void __launch_bounds__(128, 8) k_details2(PoolView pv, TS* __restrict
     if constexpr (GS == 32) return __any_sync(0xffffffffu, p);
     else return __syncthreads_or(p);
   };
-  const int nact = pv.cnt->n_round, nv = pv.nvar;
   const bool all_blocks = pv.cnt->first_round != 0;
   const int prev = pv.cnt->round_id - 1;
   const bool plan_ok = pv.cnt->plan_topo == pv.cnt->topo;
@@ -180,7 +196,7 @@ __global__ void __launch_bounds__(128, 8) k_details2(PoolView pv, TS* __restrict
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         const int n = rank + k * GS;
-        if (n < NI && (ntab[n] >> 14) && differs(me[n], raw[k])) me[n] = raw[k];
+        if (n < NI && (ntab[n] & (3 << 14)) && differs(me[n], raw[k])) me[n] = raw[k];
       }
     } else {
       if (!ring && plan_ok) {  // the stage plan's owner table
@@ -201,28 +217,26 @@ __global__ void __launch_bounds__(128, 8) k_details2(PoolView pv, TS* __restrict
         const int ox = 2 * i - (int)(int16_t)(e.z & 0xffff), oy = 2 * j - (e.z >> 16);
         return (int64_t)e.x * bs + vo + (ox >> sh) + B * (oy >> sh);
       };
-      unsigned other = 0;
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         const int n = rank + k * GS;
-        if (n >= NI) continue;
-        const int i = n % B, j = n / B;
-        if (i >= 1 && i <= B - 2 && j >= 1 && j <= B - 2) {
-          raw[k] = me[n];
-          continue;
-        }
+        if (n < NI) raw[k] = me[n];
+      }
+      for (int k = rank; k < D2::NE; k += GS) {
+        int i, j;
+        D2::edge(k, i, j);
         const int4 e = R.reg[reg_class<B>(i) + 7 * reg_class<B>(j)];
+        const int n = j * B + i;
+        TS val = me[n];
         if (e.x < 0) {
           lost = true;
-          raw[k] = TS(0);
-          continue;
+          val = TS(0);
+        } else if (e.x != b.slot) {
+          const TS mine = val;
+          val = y[owned(e, i, j)];
+          if (differs(mine, val)) me[n] = val;
         }
-        if (e.x == b.slot) {
-          raw[k] = me[n];
-        } else {
-          raw[k] = y[owned(e, i, j)];
-          other |= 1u << k;
-        }
+        ev[k] = val;
       }
       for (int k = rank; k < D2::NG; k += GS) {
         const int at = gtab[k] & 0xfff;
@@ -232,10 +246,11 @@ __global__ void __launch_bounds__(128, 8) k_details2(PoolView pv, TS* __restrict
         lost |= !ok;
         E[at] = ok ? to_tile<TT>(y[owned(e, i, j)]) : TT(0);
       }
+      g.sync();
 #pragma unroll
       for (int k = 0; k < K; ++k) {
         const int n = rank + k * GS;
-        if (((other >> k) & 1) && differs(me[n], raw[k])) me[n] = raw[k];
+        if (n < NI && (ntab[n] >> 16)) raw[k] = ev[(ntab[n] >> 16) - 1];
       }
       if (lost) set_err(pv, kErrGraded);
     }

@@ -113,21 +113,33 @@ struct WarpGroup {
   __device__ __forceinline__ void sync() const { __syncwarp(); }
 };
 
-__device__ __forceinline__ int64_t pmod64(int64_t a, int64_t n) {
-  int64_t r = a % n;
-  return r < 0 ? r + n : r;
+// a modulo n, n a power of two (blocks per axis at a level, lattice intervals): the
+// low bits of a, also for negative a.
+__device__ __forceinline__ int64_t pmod64(int64_t a, int64_t n) { return a & (n - 1); }
+// The low 16 (D = 2) or 10 (D = 3) bits of x, D - 1 zero bits between them.
+template <int D>
+__device__ __forceinline__ uint32_t spread_bits(uint32_t x) {
+  if constexpr (D == 2) {
+    x = (x | (x << 8)) & 0x00ff00ffu;
+    x = (x | (x << 4)) & 0x0f0f0f0fu;
+    x = (x | (x << 2)) & 0x33333333u;
+    x = (x | (x << 1)) & 0x55555555u;
+  } else {
+    x = (x | (x << 16)) & 0x030000ffu;
+    x = (x | (x << 8)) & 0x0300f00fu;
+    x = (x | (x << 4)) & 0x030c30c3u;
+    x = (x | (x << 2)) & 0x09249249u;
+  }
+  return x;
 }
-__device__ __forceinline__ int floordiv(int a, int b) {
-  int q = a / b;
-  return (a % b != 0 && ((a < 0) != (b < 0))) ? q - 1 : q;
-}
-
-// Morton index of a cell = treecode digits (Sec. 2.2), x bit lowest.
+// Morton index of a cell = treecode digits (Sec. 2.2), x bit lowest.  Levels reach
+// 11 (2D) and 8 (3D), so the index has at most 24 bits.
 template <int D>
 __device__ __forceinline__ uint64_t morton(const int64_t c[3], int lvl) {
-  uint64_t t = 0;
-  for (int b = lvl - 1; b >= 0; --b)
-    for (int a = D - 1; a >= 0; --a) t = (t << 1) | (uint64_t)((c[a] >> b) & 1);
+  static_assert(kMaxLevel <= 11, "2 x 11 bits in 2D");
+  const uint32_t m = (1u << lvl) - 1u;
+  uint32_t t = spread_bits<D>((uint32_t)c[0] & m) | (spread_bits<D>((uint32_t)c[1] & m) << 1);
+  if constexpr (D == 3) t |= spread_bits<D>((uint32_t)c[2] & m) << 2;
   return t;
 }
 
@@ -172,15 +184,13 @@ __device__ __forceinline__ uint64_t block_key(const int32_t* c, int lvl, int Jma
   return hilbert<D>(cell, Jmax);
 }
 
-// Slot of the leaf with block coordinates c at level m (periodic wrap), or -1.
+// Slot of the leaf with block coordinates c at level m (periodic wrap: morton
+// keeps the low m bits), or -1.
 template <int D>
 __device__ __forceinline__ int tab_get(const PoolView& pv, const TreeDev& td, int m,
                                        const int64_t c[3]) {
   if (m < td.Jmin || m > td.Jmax) return -1;
-  int64_t w[3] = {0, 0, 0};
-  const int64_t n = (int64_t)1 << m;
-  for (int a = 0; a < D; ++a) w[a] = pmod64(c[a], n);
-  return pv.tab[td.tab_off[m] + (int64_t)morton<D>(w, m)];
+  return pv.tab[td.tab_off[m] + (int64_t)morton<D>(c, m)];
 }
 
 template <int D, int B>
@@ -628,7 +638,9 @@ __device__ void coarse_passes(int nv, const TT* cbox, TT* tile, TT* scr, const P
 // of nvar x CBOX values for the coarse lattice (used when a coarser leaf
 // touches the block): every coarse node takes its owner's value, and ghost
 // nodes between coarse nodes are predicted from it.
-template <int D, int B, typename TF, typename TT, int W = kG, typename G = CtaGroup>
+// ES: tile layout, 1 = variable after variable, 4 = the four variables of a node
+// side by side.
+template <int D, int B, typename TF, typename TT, int W = kG, typename G = CtaGroup, int ES = 1>
 __device__ void fill_tile(const PoolView& pv, const BlockInfo& b, const TF* F, TF* Fw, TT* tile,
                           bool commit, RingD<D>& R, TT* cbox, TT* scr = nullptr, bool have_regions = false) {
   const G g{};
@@ -637,6 +649,7 @@ __device__ void fill_tile(const PoolView& pv, const BlockInfo& b, const TF* F, T
   // Each thread takes U points at a time: owners and addresses first, then the
   // U loads together, then the stores, so that the loads are in flight at once.
   constexpr int U = 4;
+  auto at_tile = [&](int v, int idx) { return ES == 1 ? v * Bx::TILE + idx : ES * idx + v; };
   const int nv = pv.nvar;
   const int64_t own = (int64_t)b.slot * nv * pv.vs;
   if (!R.mixed) {
@@ -678,10 +691,10 @@ __device__ void fill_tile(const PoolView& pv, const BlockInfo& b, const TF* F, T
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           if (!ok[u]) continue;
-          tile[v * Bx::TILE + idx[u]] = (TT)val[u];
+          tile[at_tile(v, idx[u])] = to_tile<TT>(val[u]);
           if (ed[u]) {
             const int64_t me = own + (int64_t)v * pv.vs + li[u];
-            if (F[me] != val[u]) Fw[me] = val[u];
+            if (differs(F[me], val[u])) Fw[me] = val[u];
           }
         }
       }
@@ -742,7 +755,7 @@ __device__ void fill_tile(const PoolView& pv, const BlockInfo& b, const TF* F, T
         for (int u = 0; u < U; ++u) val[u] = good[u] ? F[at[u] + (int64_t)v * pv.vs] : TF(0);
 #pragma unroll
         for (int u = 0; u < U; ++u)
-          if (ok[u]) cbox[v * Bx::CBOX + q0 + u * g.size()] = good[u] ? (TT)val[u] : TT(0);
+          if (ok[u]) cbox[v * Bx::CBOX + q0 + u * g.size()] = good[u] ? to_tile<TT>(val[u]) : TT(0);
       }
     }
     g.sync();
@@ -816,7 +829,7 @@ __device__ void fill_tile(const PoolView& pv, const BlockInfo& b, const TF* F, T
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         if (kind[u] == 5) continue;
-        TT* t = tile + v * Bx::TILE + idx[u];
+        TT* t = tile + at_tile(v, idx[u]);
         if (kind[u] == 3) {
           if (scr) {
             // last axis from the scratch: z in 3D (Y), y in 2D (X)
@@ -833,10 +846,10 @@ __device__ void fill_tile(const PoolView& pv, const BlockInfo& b, const TF* F, T
         } else if (kind[u] == 4) {
           *t = TT(0);
         } else {
-          *t = (TT)val[u];
+          *t = to_tile<TT>(val[u]);
           if (kind[u] == 1 && commit) {
             const int64_t me = own + (int64_t)v * pv.vs + li[u];
-            if (F[me] != val[u]) Fw[me] = val[u];
+            if (differs(F[me], val[u])) Fw[me] = val[u];
           }
         }
       }
@@ -1032,7 +1045,7 @@ __device__ void cta_scan2(const int32_t* in, int32_t* out, int n, int32_t* tot) 
 #pragma unroll
     for (int r = 0; r < PER; ++r) {
       const int i = base + threadIdx.x * PER + r;
-      loc[r] = i < n ? make_int2(__ldcg(in + 2 * i), __ldcg(in + 2 * i + 1)) : make_int2(0, 0);
+      loc[r] = i < n ? __ldcg(reinterpret_cast<const int2*>(in) + i) : make_int2(0, 0);
       s.x += loc[r].x;
       s.y += loc[r].y;
     }

@@ -127,8 +127,10 @@ struct PoolView {
   const float* latf;       // the same rounded to FP32 (FP32 stage velocities)
   double* svar;            // per tree x nvar threshold scale
   int32_t* cells;          // finest-cell marks (set_blocks validation / ranking)
-  int32_t* emit;           // scan input  [cap] x2 (int2)
-  int32_t* eoff;           // scan output [cap] x2 (int2)
+  int32_t* emit;           // new-list counts of the positions [cap] x2 (int2)
+  int32_t* eoff;           // their exclusive prefixes within groups of 8 positions [cap] x2
+  int32_t* grp;            // totals of the groups [cap / 8 + 1] x2
+  int32_t* gof;            // exclusive scan of the totals [cap / 8 + 1] x2
   int32_t* partial;        // scan partials
   int32_t* pos_of_slot;
   int32_t* stamp;          // per slot: round_id of the round that created the block (merges)
@@ -243,12 +245,13 @@ template <int B> void launch_stage_nss(const PoolView& pv, const Fields& f, int 
                                        const StageArgs& sa, const LaunchCfg& lc, cudaStream_t st);
 void launch_filter(const PoolView& pv, const Fields& f, bool copy, const LaunchCfg& lc, cudaStream_t st);
 
-// Exclusive scan of n int2 pairs (emit -> eoff); totals written to tot[0..1].
-// n_dev: device count (nullable), else n_host.
+// Exclusive scan of n int2 pairs; totals written to tot[0..1].  n_dev: device
+// count (nullable) of elements in groups of 2^shift, one pair per group; else n_host.
 // `partial` needs 2 * ceil(n_max / kScanChunk) + 2 ints.
 constexpr int kScanChunk = 2048;
 void launch_scan2(const int32_t* in, int32_t* out, int32_t* partial, const int32_t* n_dev,
-                  int64_t n_host, int32_t* tot, cudaStream_t st, int64_t n_expect = -1, bool pdl = false);
+                  int64_t n_host, int32_t* tot, cudaStream_t st, int64_t n_expect = -1, bool pdl = false,
+                  int shift = 0);
 void count_launch(int n = 1);
 int64_t kernel_launches();
 

@@ -33,6 +33,15 @@ template <typename T> __device__ __forceinline__ const T* lattice(const PoolView
 }
 
 
+// (f[-2] - f[2]) + 8 (f[1] - f[-1]): the product with 8 is exact, so the fused
+// form rounds the same value once (one instruction less per derivative).
+__device__ __forceinline__ float d1_sum(float fm2, float fm1, float f1, float f2) {
+  return __fmaf_rn(8.f, f1 - fm1, fm2 - f2);
+}
+__device__ __forceinline__ double d1_sum(double fm2, double fm1, double f1, double f2) {
+  return __fma_rn(8.0, f1 - fm1, fm2 - f2);
+}
+
 // ------------------------------------------------------------------ stage ----
 // One RK4 stage on every block (Sec. 3: 4th-order central FD + classic RK4):
 //   k = N(Y_s) on the synchronised tile, then the 3-register update
@@ -64,6 +73,7 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 8 : 4) k_stage_adv(PoolView pv
   __shared__ int32_t splan[2][PL::INTS];
   __shared__ int64_t snb[2][PL::NB];  // pool offsets of the plan's neighbours
   const int nact = pv.cnt->n_act;
+  if (blockIdx.x >= nact) return;  // no block for this CTA (small grids)
   if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&pv.cnt->stage_blocks, (unsigned long long)nact);
   build_gtab<D, B, 2>(gtab);
   if (blockIdx.x < nact && threadIdx.x < PL::INTS) {
@@ -210,11 +220,12 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_stage_adv_w(PoolView pv, cons
   TS* as = ys + SW::VS;
   TC* tile = reinterpret_cast<TC*>(un + SW::UNION);
   __shared__ int64_t snb[SW::NW][PL::NB];
+  const int nact = pv.cnt->n_act;
+  if ((int)blockIdx.x * SW::NW >= nact) return;  // no block for this CTA
   build_gtab<2, B, 2>(gtab);
   if (SW::TMA && lane == 0) mbar_init(bar, 1);
   __syncthreads();
   unsigned phase = 0;
-  const int nact = pv.cnt->n_act;
   if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&pv.cnt->stage_blocks, (unsigned long long)nact);
   const int gw = blockIdx.x * SW::NW + warp, nwt = gridDim.x * SW::NW;
   int32_t cur = (gw < nact && lane < PL::INTS) ? pv.plan[(int64_t)gw * PL::INTS + lane] : 0;
@@ -397,6 +408,39 @@ __global__ void k_round_begin(PoolView pv, double v) {
     c->round_id += 1;
   }
   for (int i = threadIdx.x; i < pv.ntrees * pv.nvar; i += blockDim.x) pv.svar[i] = v;
+}
+
+// ------------------------------------------------------- new-list offsets ----
+// New-list counts of 8 consecutive positions (one per warp of the CTA, in warp
+// order): each position's exclusive prefix within them, and their total.  The
+// totals are scanned later, so a scan works on an eighth of the list (7500 blocks
+// of 64 trees: 18 -> 4 us in the last CTA of k_flags).
+__device__ __forceinline__ void emit_group(const PoolView& pv, int g, int n, int2 (*sh)[8], int par, int2 e) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (lane == 0) sh[par][w] = e;
+  __syncthreads();
+  if (w == 0 && lane < 8) {
+    const int2 own = sh[par][lane];
+    int2 v = own;
+    for (int o = 1; o < 8; o <<= 1) {
+      const int x = __shfl_up_sync(0xffu, v.x, o), z = __shfl_up_sync(0xffu, v.y, o);
+      if (lane >= o) { v.x += x; v.y += z; }
+    }
+    if (8 * g + lane < n) reinterpret_cast<int2*>(pv.eoff)[8 * g + lane] = make_int2(v.x - own.x, v.y - own.y);
+    if (lane == 7) reinterpret_cast<int2*>(pv.grp)[g] = v;
+  }
+}
+// Scan of the group totals by the calling (last) CTA of 256 threads.
+__device__ __forceinline__ void scan_groups(const PoolView& pv, int n) {
+  const int ng = (n + 7) >> 3;
+  if (ng <= 1024) cta_scan2<256, 4>(pv.grp, pv.gof, ng, &pv.cnt->n_new);
+  else cta_scan2<256, 16>(pv.grp, pv.gof, ng, &pv.cnt->n_new);
+}
+// Position of the first entry of list position p in the new list, and of its first
+// slot among those requested (refinement) or freed (merge).
+__device__ __forceinline__ int2 new_offset(const PoolView& pv, int p) {
+  const int2 g = reinterpret_cast<const int2*>(pv.gof)[p >> 3], l = reinterpret_cast<const int2*>(pv.eoff)[p];
+  return make_int2(g.x + l.x, g.y + l.y);
 }
 
 // ------------------------------------------------------------- NS stage ----
@@ -619,8 +663,8 @@ struct RefGeo {
 // appended); children are placed in the new active list in Hilbert order.
 // 2D blocks; 3D ones are refined by k_refine3 (mr_adv3.cuh).  One CTA per mother
 // and variable: with the four variables of a mother in one CTA, 376 mothers of 33^2
-// nodes were 1.2 waves of 304 CTAs (335 us); 216 us with 1504 CTAs of a quarter
-// of the shared memory.
+// nodes were 1.2 waves of 304 CTAs (335 us); 216 us with 1504 items of a quarter of
+// the shared memory, 138 us with odd and even nodes apart (see below).
 template <int B, typename TS, int NT>
 __global__ void __launch_bounds__(NT, NT <= 128 ? 8 : 4) k_refine(PoolView pv, TS* __restrict__ y) {
   pdl_enter();
@@ -645,7 +689,8 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 8 : 4) k_refine(PoolView pv, T
   for (int64_t it = blockIdx.x; it < (int64_t)nact * nv; it += gridDim.x) {
     const int p = (int)(it / nv), v = (int)(it % nv);
     const int slot = pv.act[p];
-    const int e = pv.eoff[2 * p], a = pv.eoff[2 * p + 1];
+    const int2 off = new_offset(pv, p);
+    const int e = off.x, a = off.y;
     if (pv.flag[slot] != 1) {
       if (v == 0 && threadIdx.x == 0) pv.act_next[e] = slot;
       continue;
@@ -660,48 +705,50 @@ __global__ void __launch_bounds__(NT, NT <= 128 ? 8 : 4) k_refine(PoolView pv, T
     build_ring<D, B>(pv, td, b, R);
     __syncthreads();
     fill_tile<D, B, TS, TS, 1>(pv1, b, yv, (TS*)yv, tile, false, R, cbox, scr);
-    if (threadIdx.x < Gm::NCH) cslot[threadIdx.x] = pv.freelist[n_free - n_alloc + a + threadIdx.x];
-    __syncthreads();
-    if (v == 0 && threadIdx.x == 0) {
-      uint64_t key[8];
-      int32_t cc[8][3];
-      for (int ch = 0; ch < Gm::NCH; ++ch) {
-        for (int ax = 0; ax < 3; ++ax)
-          cc[ch][ax] = ax < D ? (int32_t)(2 * b.c[ax] + ((ch >> ax) & 1)) : 0;
-        key[ch] = block_key<D>(cc[ch], b.lvl + 1, td.Jmax);
-      }
-      for (int ch = 0; ch < Gm::NCH; ++ch) {
+    if (threadIdx.x < Gm::NCH) {
+      const int ch = threadIdx.x;
+      const int cs = pv.freelist[n_free - n_alloc + a + ch];
+      cslot[ch] = cs;
+      if (v == 0) {
+        // light data of the children, in the order of their Hilbert keys
+        const int32_t cc[3] = {(int32_t)(2 * b.c[0] + (ch & 1)), (int32_t)(2 * b.c[1] + (ch >> 1)), 0};
+        const uint64_t key = block_key<D>(cc, b.lvl + 1, td.Jmax);
         int rank = 0;
-        for (int o = 0; o < Gm::NCH; ++o) rank += key[o] < key[ch];
-        const int cs = cslot[ch];
+        for (int o = 0; o < Gm::NCH; ++o) rank += __shfl_sync((1u << Gm::NCH) - 1u, key, o) < key;
         pv.act_next[e + rank] = cs;
         pv.lvl[cs] = (int8_t)(b.lvl + 1);
         pv.tree[cs] = (int16_t)b.tree;
-        for (int ax = 0; ax < 3; ++ax) pv.crd[3 * cs + ax] = cc[ch][ax];
-        pv.hkey[cs] = key[ch];
+        for (int ax = 0; ax < 3; ++ax) pv.crd[3 * cs + ax] = cc[ax];
+        pv.hkey[cs] = key;
         pv.flag[cs] = 0;
       }
     }
     __syncthreads();
     // Separable upsampling: X = prediction along x on the mother's rows (y in
     // [-1, B]), then y per child node -- the operations of the tensor product in
-    // the same order.
-    for (int idx = threadIdx.x; idx < RG::NX; idx += blockDim.x) {
-      const int ox = idx % RG::NF, jy = idx / RG::NF - 1;
-      const int fl = ox >> 1;
-      X[idx] = (ox & 1) ? dd4(tile[Bx::tix(fl - 1, jy, 0)], tile[Bx::tix(fl, jy, 0)], tile[Bx::tix(fl + 1, jy, 0)],
-                              tile[Bx::tix(fl + 2, jy, 0)])
-                        : tile[Bx::tix(fl, jy, 0)];
+    // the same order; odd nodes (4-point rule) before even ones (copies), so that
+    // their warps hold one kind (the rule on the FP64 pipe bounds the FP64 form).
+    constexpr int H = B - 1, NR = RG::NR, NF = RG::NF;
+    for (int idx = threadIdx.x; idx < NR * H; idx += blockDim.x) {
+      const int row = idx / H, m = idx % H;
+      const TS* t = tile + Bx::tix(m - 1, row - 1, 0);
+      X[row * NF + 2 * m + 1] = dd4(t[0], t[1], t[2], t[3]);
+    }
+    for (int idx = threadIdx.x; idx < NR * B; idx += blockDim.x) {
+      const int row = idx / B, m = idx % B;
+      X[row * NF + 2 * m] = tile[Bx::tix(m, row - 1, 0)];
     }
     __syncthreads();
-    auto xr = [&](int ox, int jy) { return X[(jy + 1) * RG::NF + ox]; };
-    for (int idx = threadIdx.x; idx < Gm::NCH * Gm::NI; idx += blockDim.x) {
-      const int ch = idx / Gm::NI, q = idx % Gm::NI;
-      const int i = q % B, j = q / B;
-      const int ox = (ch & 1) * (B - 1) + i, oy = (ch >> 1) * (B - 1) + j;
-      const int fl = oy >> 1;
-      const TS val = (oy & 1) ? dd4(xr(ox, fl - 1), xr(ox, fl), xr(ox, fl + 1), xr(ox, fl + 2)) : xr(ox, fl);
-      y[((int64_t)cslot[ch] * nv + v) * pv.vs + q] = val;
+    // child ch, odd rows j = 2m + 1, then even ones j = 2m (fine row (ch >> 1)(B - 1) + j)
+    constexpr int NO = H / 2, NE = NO + 1;
+    for (int idx = threadIdx.x; idx < 4 * NO * B; idx += blockDim.x) {
+      const int i = idx % B, m = (idx / B) % NO, ch = idx / (B * NO);
+      const TS* t = X + ((ch >> 1) * NO + m) * NF + (ch & 1) * H + i;  // mother rows fl - 1 .. fl + 2, from -1
+      y[((int64_t)cslot[ch] * nv + v) * pv.vs + (2 * m + 1) * B + i] = dd4(t[0], t[NF], t[2 * NF], t[3 * NF]);
+    }
+    for (int idx = threadIdx.x; idx < 4 * NE * B; idx += blockDim.x) {
+      const int i = idx % B, m = (idx / B) % NE, ch = idx / (B * NE);
+      y[((int64_t)cslot[ch] * nv + v) * pv.vs + 2 * m * B + i] = X[((ch >> 1) * NO + m + 1) * NF + (ch & 1) * H + i];
     }
     __syncthreads();
   }
@@ -789,112 +836,230 @@ __device__ __forceinline__ void block_max3(A& a, Bt& b, Ct& c, A* ra, Bt* rb, Ct
 // (every second node); a mother node on a line shared by two children is read
 // from the child in which it has local index 0.  The mother takes the slot of
 // the family member that comes first in Hilbert order.
-// One kernel per round: each CTA merges families (the mother's data, then the
+// One kernel per round: families are merged (the mother's data, then the
 // family's table entries, light data and freed slots -- the family's 2^d
 // members sit at consecutive list positions, a Hilbert-curve property), and
 // the CTA that finishes last copies the new active list in place, updates the
 // counters and prepares the next round (RoundCtl).
-template <int D, int B, typename TS>
-__global__ void __launch_bounds__(256) k_coarsen(PoolView pv, TS* __restrict__ y, RoundCtl rc) {
+
+// Counters a round works with, read at its start (they change at its end).
+struct RoundState {
+  int nround, n_free, n_new, n_alloc, rid, rounds, topo;
+  bool done, none;
+  __device__ __forceinline__ explicit RoundState(const Counters* c) {
+    nround = c->n_round;
+    n_free = c->n_free;
+    n_new = c->n_new;
+    n_alloc = c->n_alloc;
+    rid = c->round_id;
+    rounds = c->rounds;
+    topo = c->topo;
+    done = c->done != 0;
+    none = n_new == nround;  // no family merges: the tree and the list are unchanged
+  }
+};
+
+// Table entry, light data and slot of member s (list position q, block m) of a
+// merged family whose mother takes `slot`.
+template <int D>
+__device__ __forceinline__ void merge_member(const PoolView& pv, const TreeDev& td, const RoundState& rs, int q, int s,
+                                             const BlockInfo& m, int slot) {
+  pv.tab[td.tab_off[m.lvl] + (int64_t)morton<D>(m.c, m.lvl)] = -1;
+  if (s == slot) {
+    const int64_t pc[3] = {m.c[0] >> 1, m.c[1] >> 1, m.c[2] >> 1};
+    pv.tab[td.tab_off[m.lvl - 1] + (int64_t)morton<D>(pc, m.lvl - 1)] = s;
+    pv.stamp[s] = rs.rid;
+    pv.lvl[s] = (int8_t)(m.lvl - 1);
+    const int32_t c32[3] = {(int32_t)pc[0], (int32_t)pc[1], (int32_t)pc[2]};
+    for (int a = 0; a < 3; ++a) pv.crd[3 * s + a] = c32[a];
+    pv.hkey[s] = block_key<D>(c32, m.lvl - 1, td.Jmax);
+  } else {
+    pv.lvl[s] = -1;
+    pv.freelist[rs.n_free + new_offset(pv, q).y] = s;
+  }
+}
+
+// List position of work item it, nq = ceil(n / 2^d): the first members of the families
+// sit 2^d positions apart, so consecutive items take positions 2^d apart (in list
+// order with a grid of a multiple of 2^d CTAs, only every 2^d-th CTA had families).
+template <int D>
+__device__ __forceinline__ int merge_position(int it, int nq) {
+  return (it % nq) * (1 << D) + it / nq;
+}
+
+// End of a round, by the CTA of the grid that finishes last: the new list in place
+// (every entry of act_next is written by now), the counters, and the next round, if
+// one runs (a family merged and fewer than max_rounds ran): the blocks it evaluates,
+// its id, its threshold scales (the last round's stay for the next step's proposal
+// features); in a captured step the while node's condition.
+template <int D>
+__device__ __forceinline__ void finish_round(const PoolView& pv, const RoundState& rs, const RoundCtl& rc) {
+  const int ncopy = rs.done || rs.none ? 0 : rs.n_new;
+  const int n4 = ncopy >> 2;
+  const int4* from = reinterpret_cast<const int4*>(pv.act_next);
+  int4* to = reinterpret_cast<int4*>(pv.act);
+  for (int p = threadIdx.x; p < n4; p += 4 * blockDim.x) {
+    int4 t[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      if (p + r * (int)blockDim.x < n4) t[r] = __ldcg(from + p + r * blockDim.x);
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      if (p + r * (int)blockDim.x < n4) to[p + r * blockDim.x] = t[r];
+  }
+  if ((int)threadIdx.x < (ncopy & 3)) pv.act[4 * n4 + threadIdx.x] = __ldcg(pv.act_next + 4 * n4 + threadIdx.x);
+  // a round that is not skipped works on the whole list
+  const int merged = rs.done ? 0 : (rs.nround - rs.n_new) / ((1 << D) - 1);
+  const bool done = rs.done || merged == 0;
+  const bool next = !done && rs.rounds + 1 < rc.max_rounds;
+  if (next)
+    for (int i = threadIdx.x; i < pv.ntrees * pv.nvar; i += blockDim.x) pv.svar[i] = rc.svar_v;
+  if (threadIdx.x == 0) {
+    Counters* c = pv.cnt;
+    c->first_round = 0;
+    if (!rs.done) {
+      c->merged = merged;
+      c->n_free = rs.n_free + rs.n_alloc;
+      c->n_act = rs.n_new;
+      if (done) c->done = 1;
+      else c->topo = rs.topo + 1;
+    }
+    c->rounds = rs.rounds + 1;
+    c->n_round = done ? 0 : rs.n_new;
+    if (next) c->round_id = rs.rid + 1;
+    if (rc.has_h) {
+      c->graph_rounds += 1;
+      cudaGraphSetConditional(rc.h, next ? 1u : 0u);
+    }
+    c->ctas_done = 0;
+  }
+}
+
+// 2D: one warp per family of 17^2 blocks with one variable, else one CTA (9 or 10
+// values per thread, read before the first is written: the mother takes a child's
+// slot).  Blocks that do not merge only enter the new list.  Latency-bound: a chain of
+// list entry, block data, children's nodes and tables.  With a CTA of 256 threads per
+// block, through shared memory, in list order: 47 -> 12 us for the first round of 64
+// trees (7472 blocks), 64 -> 35 us for 2944 blocks of 33^2 x 4 FP64 values.
+template <int B, int NV>
+struct Coarsen2 {
+  static constexpr int N = NV * B * B;
+  static constexpr int GS = N <= 320 ? 32 : (N <= 1280 ? 128 : 512);  // threads per family
+  static constexpr int NT = GS == 32 ? 128 : GS;
+  static constexpr int K = (N + GS - 1) / GS;
+};
+template <int B, int NV, typename TS>
+__global__ void __launch_bounds__(Coarsen2<B, NV>::NT) k_coarsen2(PoolView pv, TS* __restrict__ y, RoundCtl rc) {
   pdl_enter();
-  using Gm = Geo<D, B>;
-  TS* buf = smem_as<TS>(0);
-  __shared__ int cs[8];
-  Counters* c = pv.cnt;
-  const int nround = c->n_round, n_free = c->n_free, n_new = c->n_new, rid = c->round_id;
-  const bool done = c->done != 0;
-  const bool none = n_new == nround;  // no family merges: the tree and the list are unchanged
-  const int nv = pv.nvar;
-  for (int p = blockIdx.x; !none && p < nround; p += gridDim.x) {
+  using CO = Coarsen2<B, NV>;
+  using G = std::conditional_t<CO::GS == 32, WarpGroup, CtaGroup>;
+  constexpr int GS = CO::GS, K = CO::K, NI = B * B, ITEMS = CO::NT / GS;
+  const G g{};
+  const int rank = threadIdx.x % GS, item = threadIdx.x / GS;
+  __shared__ int scs[ITEMS][4];
+  int* cs = scs[item];
+  const RoundState rs(pv.cnt);
+  const int64_t bs = (int64_t)NV * pv.vs;
+  const int nq = (rs.nround + 3) / 4;
+  for (int it = blockIdx.x * ITEMS + item; !rs.none && it < 4 * nq; it += gridDim.x * ITEMS) {
+    const int p = merge_position<2>(it, nq);
+    if (p >= rs.nround || !pv.emit[2 * p]) continue;  // a member of a family merged at its first member
     const int slot = pv.act[p];
-    const int emit = pv.emit[2 * p], e = pv.eoff[2 * p];
-    if (!emit) continue;  // a member of a family merged by the CTA of its first member
-    if (threadIdx.x == 0) pv.act_next[e] = slot;
+    if (rank == 0) pv.act_next[new_offset(pv, p).x] = slot;
     if (pv.flag[slot] != -2) continue;
     const BlockInfo b = load_block(pv, slot);
     const TreeDev& td = pv.trees[b.tree];
-    if (threadIdx.x < Gm::NCH) {
-      int64_t cc[3] = {0, 0, 0};
-      for (int a = 0; a < D; ++a) cc[a] = (b.c[a] & ~(int64_t)1) | ((threadIdx.x >> a) & 1);
-      cs[threadIdx.x] = tab_get<D>(pv, td, b.lvl, cc);
+    // the family: positions p .. p + 3
+    BlockInfo m = b;
+    if (rank < 4) {
+      cs[rank] = -1;
+      if (p + rank < rs.nround) m = load_block(pv, pv.act[p + rank]);
+      else m.tree = -1;
+    }
+    g.sync();
+    if (rank < 4 && m.tree == b.tree && m.lvl == b.lvl && (m.c[0] >> 1) == (b.c[0] >> 1) &&
+        (m.c[1] >> 1) == (b.c[1] >> 1))
+      cs[(m.c[0] & 1) + 2 * (m.c[1] & 1)] = m.slot;
+    g.sync();
+    if (cs[0] < 0 || cs[1] < 0 || cs[2] < 0 || cs[3] < 0) {  // cannot happen for a complete family
+      if (rank == 0) set_err(pv, kErrGraded);
+      g.sync();
+      continue;
+    }
+    TS val[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const int idx = rank + k * GS;
+      if (idx >= CO::N) continue;
+      const int v = idx / NI, q = idx % NI, i = q % B, j = q / B;
+      const int bx = 2 * i >= B - 1, by = 2 * j >= B - 1;
+      val[k] = y[(int64_t)cs[bx + 2 * by] * bs + v * pv.vs + (2 * i - bx * (B - 1)) + B * (2 * j - by * (B - 1))];
+    }
+    g.sync();
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      const int idx = rank + k * GS;
+      if (idx >= CO::N) continue;
+      const int v = idx / NI, q = idx % NI;
+      y[(int64_t)slot * bs + v * pv.vs + q] = val[k];
+    }
+    if (rank < 4) merge_member<2>(pv, td, rs, p + rank, m.slot, m, slot);
+    g.sync();
+  }
+  if (last_cta_all(pv.cnt)) finish_round<2>(pv, rs, rc);
+}
+
+// 3D: one CTA per family, the mother's nodes through shared memory.
+template <int B, typename TS>
+__global__ void __launch_bounds__(256) k_coarsen3(PoolView pv, TS* __restrict__ y, RoundCtl rc) {
+  pdl_enter();
+  using Gm = Geo<3, B>;
+  TS* buf = smem_as<TS>(0);
+  __shared__ int cs[8];
+  const RoundState rs(pv.cnt);
+  const int nq = (rs.nround + 7) / 8;
+  for (int it = blockIdx.x; !rs.none && it < 8 * nq; it += gridDim.x) {
+    const int p = merge_position<3>(it, nq);
+    if (p >= rs.nround || !pv.emit[2 * p]) continue;  // a member of a family merged by the CTA of its first member
+    const int slot = pv.act[p];
+    if (threadIdx.x == 0) pv.act_next[new_offset(pv, p).x] = slot;
+    if (pv.flag[slot] != -2) continue;
+    const BlockInfo b = load_block(pv, slot);
+    const TreeDev& td = pv.trees[b.tree];
+    if (threadIdx.x < 8) {
+      int64_t cc[3];
+      for (int a = 0; a < 3; ++a) cc[a] = (b.c[a] & ~(int64_t)1) | ((threadIdx.x >> a) & 1);
+      cs[threadIdx.x] = tab_get<3>(pv, td, b.lvl, cc);
     }
     __syncthreads();
     bool missing = false;
-    for (int ch = 0; ch < Gm::NCH; ++ch) missing |= cs[ch] < 0;
+    for (int ch = 0; ch < 8; ++ch) missing |= cs[ch] < 0;
     if (missing) {  // cannot happen for a complete family; never read slot -1
       if (threadIdx.x == 0) set_err(pv, kErrGraded);
       __syncthreads();
       continue;
     }
-    for (int idx = threadIdx.x; idx < nv * Gm::NI; idx += blockDim.x) {
-      const int v = idx / Gm::NI, q = idx % Gm::NI;
-      const int I[3] = {q % B, (q / B) % B, D == 3 ? q / (B * B) : 0};
-      int cb = 0, li[3] = {0, 0, 0};
-      for (int a = 0; a < D; ++a) {
+#pragma unroll 4
+    for (int q = threadIdx.x; q < Gm::NI; q += 256) {
+      const int I[3] = {q % B, (q / B) % B, q / (B * B)};
+      int cb = 0, li[3];
+      for (int a = 0; a < 3; ++a) {
         const int bit = (2 * I[a] >= B - 1) ? 1 : 0;
         cb |= bit << a;
         li[a] = 2 * I[a] - bit * (B - 1);
       }
-      buf[idx] = pool_at<D, B>(pv, y, cs[cb], v, li);
+      buf[q] = y[(int64_t)cs[cb] * pv.vs + Gm::lin(li[0], li[1], li[2])];
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < nv * Gm::NI; idx += blockDim.x) {
-      const int v = idx / Gm::NI, q = idx % Gm::NI;
-      y[((int64_t)slot * nv + v) * pv.vs + q] = buf[idx];
-    }
-    // the family's tables and light data (positions p .. p + 2^d - 1)
-    if (threadIdx.x < Gm::NCH) {
-      const int q = p + threadIdx.x;
-      const int s = pv.act[q];
-      const BlockInfo m = load_block(pv, s);
-      pv.tab[td.tab_off[m.lvl] + (int64_t)morton<D>(m.c, m.lvl)] = -1;
-      if (s == slot) {
-        const int64_t pc[3] = {m.c[0] >> 1, m.c[1] >> 1, m.c[2] >> 1};
-        pv.tab[td.tab_off[m.lvl - 1] + (int64_t)morton<D>(pc, m.lvl - 1)] = s;
-        pv.stamp[s] = rid;
-        pv.lvl[s] = (int8_t)(m.lvl - 1);
-        const int32_t c32[3] = {(int32_t)pc[0], (int32_t)pc[1], (int32_t)pc[2]};
-        for (int a = 0; a < 3; ++a) pv.crd[3 * s + a] = c32[a];
-        pv.hkey[s] = block_key<D>(c32, m.lvl - 1, td.Jmax);
-      } else {
-        pv.lvl[s] = -1;
-        pv.freelist[n_free + pv.eoff[2 * q + 1]] = s;
-      }
+    for (int q = threadIdx.x; q < Gm::NI; q += 256) y[(int64_t)slot * pv.vs + q] = buf[q];
+    // the family's tables and light data (positions p .. p + 7)
+    if (threadIdx.x < 8) {
+      const int s = pv.act[p + threadIdx.x];
+      merge_member<3>(pv, td, rs, p + threadIdx.x, s, load_block(pv, s), slot);
     }
     __syncthreads();
   }
-  if (last_cta_all(c)) {
-    // the new list in place (every entry of act_next is written by now)
-    const int ncopy = done || none ? 0 : n_new;
-    for (int p = threadIdx.x; p < ncopy; p += blockDim.x) pv.act[p] = __ldcg(pv.act_next + p);
-    if (threadIdx.x == 0) {
-      c->first_round = 0;
-      if (!done) {
-        const int nch = 1 << D;
-        c->merged = (c->n_act - n_new) / (nch - 1);
-        c->n_free = n_free + c->n_alloc;
-        c->n_act = n_new;
-        if (c->merged == 0) c->done = 1;
-        else c->topo += 1;
-      }
-      // the next round, if one runs (a family merged and fewer than max_rounds
-      // ran): the blocks it evaluates, its id, its threshold scales (the last
-      // round's stay for the next step's proposal features); in a captured
-      // step the while node's condition
-      c->rounds += 1;
-      const bool next = !c->done && c->rounds < rc.max_rounds;
-      c->n_round = c->done ? 0 : c->n_act;
-      if (next) {
-        c->round_id += 1;
-        for (int i = 0; i < pv.ntrees * pv.nvar; ++i) pv.svar[i] = rc.svar_v;
-      }
-      if (rc.has_h) {
-        c->graph_rounds += 1;
-        cudaGraphSetConditional(rc.h, next ? 1u : 0u);
-      }
-      c->ctas_done = 0;
-    }
-  }
+  if (last_cta_all(pv.cnt)) finish_round<3>(pv, rs, rc);
 }
 
 // --------------------------------------------------------------------- IC ----
@@ -1043,26 +1208,36 @@ __global__ void k_error(PoolView pv, const TS* __restrict__ y, int tree, const d
 }
 
 // ------------------------------------------------------- tree maintenance ----
-// SCAN: the CTA that finishes last also scans the counts (short lists), which
-// saves the separate scan launch.
+// One thread per block: its flag, and the new-list counts in groups of 8 positions
+// (see emit_group).  SCAN: the CTA that finishes last also scans the group totals.
 template <int D, bool SCAN>
 __global__ void __launch_bounds__(256) k_refine_count(PoolView pv, int mode, const int8_t* mask) {
   pdl_enter();
   const int nact = pv.cnt->n_act;
   const int nch = 1 << D;
-  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < nact; p += gridDim.x * blockDim.x) {
-    const int s = pv.act[p];
-    const int l = pv.lvl[s];
-    const TreeDev& td = pv.trees[pv.tree[s]];
-    // mode 2: flags already set on the device (learned proposal + closure)
-    const bool r = l < td.Jmax && (mode == MR_ADAPT_REFINE_ALL || (mode == 2 ? pv.flag[s] == 1 : (mask && mask[p] > 0)));
-    pv.flag[s] = r ? 1 : 0;
-    pv.emit[2 * p] = r ? nch : 1;
-    pv.emit[2 * p + 1] = r ? nch : 0;
+  for (int base = blockIdx.x * blockDim.x; base < nact; base += gridDim.x * blockDim.x) {
+    const int p = base + threadIdx.x;
+    int2 own = make_int2(0, 0);
+    if (p < nact) {
+      const int s = pv.act[p];
+      const int l = pv.lvl[s];
+      const TreeDev& td = pv.trees[pv.tree[s]];
+      // mode 2: flags already set on the device (learned proposal + closure)
+      const bool r = l < td.Jmax && (mode == MR_ADAPT_REFINE_ALL || (mode == 2 ? pv.flag[s] == 1 : (mask && mask[p] > 0)));
+      pv.flag[s] = r ? 1 : 0;
+      own = make_int2(r ? nch : 1, r ? nch : 0);
+    }
+    int2 v = own;
+    for (int o = 1; o < 8; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, v.x, o, 8), z = __shfl_up_sync(0xffffffffu, v.y, o, 8);
+      if ((threadIdx.x & 7) >= o) { v.x += x; v.y += z; }
+    }
+    if (p < nact) reinterpret_cast<int2*>(pv.eoff)[p] = make_int2(v.x - own.x, v.y - own.y);
+    if ((threadIdx.x & 7) == 7 && (p & ~7) < nact) reinterpret_cast<int2*>(pv.grp)[p >> 3] = v;
   }
   if constexpr (SCAN) {
     if (last_cta_all(pv.cnt)) {
-      cta_scan2<256, 8>(pv.emit, pv.eoff, nact, &pv.cnt->n_new);
+      scan_groups(pv, nact);
       if (threadIdx.x == 0) pv.cnt->ctas_done = 0;
     }
   }
@@ -1100,13 +1275,14 @@ __global__ void k_refine_commit(PoolView pv) {
         const BlockInfo b = load_block(pv, s);
         const TreeDev& td = pv.trees[b.tree];
         pv.tab[td.tab_off[b.lvl] + (int64_t)morton<D>(b.c, b.lvl)] = -1;
-        const int e = pv.eoff[2 * p];
+        const int2 off = new_offset(pv, p);
+        const int e = off.x;
         for (int r = 0; r < nch; ++r) {
           const int cs = pv.act_next[e + r];
           int64_t cc[3] = {pv.crd[3 * cs], pv.crd[3 * cs + 1], pv.crd[3 * cs + 2]};
           pv.tab[td.tab_off[b.lvl + 1] + (int64_t)morton<D>(cc, b.lvl + 1)] = cs;
         }
-        pv.freelist[n_free - n_alloc + pv.eoff[2 * p + 1] / nch] = s;
+        pv.freelist[n_free - n_alloc + off.y / nch] = s;
         pv.lvl[s] = -1;
         pv.flag[s] = 0;
       }
@@ -1145,105 +1321,96 @@ __global__ void __launch_bounds__(256) k_flags(PoolView pv) {
   // whose normalised detail is below eps, above Jmin, and no leaf one level
   // finer touches any sister: the cells of level l+1 around the family,
   // [-1, 4]^d relative to its lower corner minus the family itself (the
-  // union of the sisters' rings).  One warp per block; the sister lookups,
-  // their details and the ring lookups are spread over the lanes.
+  // union of the sisters' rings).  One warp per block, a lane per sister and
+  // variable: the FP64 division of the normalisation is one sequence per warp
+  // (with a lane per sister it took 78 us for 16384 blocks of 4 variables, all
+  // FP64 pipe); the ring lookups are spread over the lanes.
   constexpr int NS = 1 << D;
   constexpr int NBOX = D == 3 ? 6 * 6 * 6 : 6 * 6;  // [-1, 4]^d around a family
+  static_assert(NS * kMaxVar <= 32 && kMaxVar == 4, "a lane per sister and variable");
+  __shared__ int2 sh[2][8];
   const int nact = pv.cnt->n_round;
-  const int lane = threadIdx.x & 31;
-  const int wpb = blockDim.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nv = pv.nvar;
-  for (int p = blockIdx.x * wpb + (threadIdx.x >> 5); p < nact; p += gridDim.x * wpb) {
-    const int s = pv.act[p];
-    const BlockInfo b = load_block(pv, s);
-    const TreeDev& td = pv.trees[b.tree];
-    int64_t fc[3] = {0, 0, 0};
-    for (int a = 0; a < D; ++a) fc[a] = b.c[a] & ~(int64_t)1;
-    // normalised detail m of leaf t (NaN if a variable's is) and m < eps
-    auto detail = [&](int t, double& m) -> bool {
-      if (pv.norm_kind == 0) {
-        // unnormalised: a maximum of non-negative values (or NaN), taken and
-        // compared with eps > 0 on their bit patterns, which order as the values
-        long long mb = 0;
-        bool nan = false;
-        for (int v = 0; v < nv; ++v) {
-          const long long x = __double_as_longlong(pv.md[(int64_t)t * nv + v]);
-          nan |= (x & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL;
-          mb = x > mb ? x : mb;
-        }
-        if (nan) mb = 0x7ff8000000000000LL;
-        m = __longlong_as_double(mb);
-        return !nan && mb < __double_as_longlong(td.eps);
-      }
-      bool nan = false;
-      m = 0.0;
-      for (int v = 0; v < nv; ++v) {
-        double sv = pv.svar[b.tree * nv + v];
-        if (sv == 0.0) sv = 1.0;
-        const double mv = pv.md[(int64_t)t * nv + v];
-        nan |= isnan(mv);
-        m = fmax(m, mv / sv);
-      }
-      if (nan) m = __longlong_as_double(0x7ff8000000000000LL);
-      return m < td.eps;
-    };
-    if (b.lvl <= td.Jmin) {
+  int par = 0;
+  for (int g = blockIdx.x; 8 * g < nact; g += gridDim.x, par ^= 1) {
+    const int p = 8 * g + warp;
+    int2 e = make_int2(0, 0);
+    if (p < nact) {
+      const int s = pv.act[p];
+      const BlockInfo b = load_block(pv, s);
+      // lane 31: is the previous list entry a member of the same family
+      const bool prev = lane == 31 && p > 0 && same_family(pv, s, pv.act[p - 1]);
+      const TreeDev& td = pv.trees[b.tree];
+      const int sis = lane >> 2, v = lane & 3;
+      const int own = (int)((b.c[0] & 1) | ((b.c[1] & 1) << 1) | (D > 2 ? (b.c[2] & 1) << 2 : 0));
+      int64_t fc[3] = {0, 0, 0};
+      for (int a = 0; a < D; ++a) fc[a] = b.c[a] & ~(int64_t)1;
       // a family at Jmin never merges: only the block's own detail is recorded
+      const bool above = b.lvl > td.Jmin;
+      int t = -1;
+      if (sis == own) {
+        t = s;
+      } else if (above && sis < NS) {
+        int64_t c[3] = {0, 0, 0};
+        for (int a = 0; a < D; ++a) c[a] = fc[a] | ((sis >> a) & 1);
+        t = tab_get<D>(pv, td, b.lvl, c);
+      }
+      // normalised detail of the lane's sister: the maximum over the variables
+      // of non-negative values (NaN if a variable's is), on their bit patterns,
+      // which order as the values
+      long long mb = 0;
+      bool nan = false;
+      if (t >= 0 && v < nv) {
+        double mv = pv.md[(int64_t)t * nv + v];
+        if (pv.norm_kind != 0) {
+          double sv = pv.svar[b.tree * nv + v];
+          if (sv == 0.0) sv = 1.0;
+          mv = mv / sv;
+        }
+        mb = __double_as_longlong(mv);
+        nan = (mb & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL;
+        if (nan) mb = 0;
+      }
+      for (int o = 1; o < 4; o <<= 1) {
+        const long long x = __shfl_xor_sync(0xffffffffu, mb, o);
+        mb = x > mb ? x : mb;
+      }
+      const unsigned nans = __ballot_sync(0xffffffffu, nan);
+      nan = (nans >> (4 * sis)) & 15u;
+      if (nan) mb = 0x7ff8000000000000LL;
+      bool ok = sis >= NS || (t >= 0 && !nan && mb < __double_as_longlong(td.eps));
+      const double m = __longlong_as_double(__shfl_sync(0xffffffffu, mb, 4 * own));
+      // no finer leaf around the family: cells of [-1, 4]^d outside [0, 3]^d
+      // (looked up only for a family whose members are all candidates)
+      const bool sisters = __all_sync(0xffffffffu, ok) && above;
+      for (int u = lane; sisters && u < NBOX; u += 32) {
+        const int q[3] = {u % 6 - 1, (u / 6) % 6 - 1, D == 3 ? u / 36 - 1 : 0};
+        bool in = true;
+        for (int a = 0; a < D; ++a) in &= q[a] >= 0 && q[a] <= 3;
+        if (in) continue;
+        int64_t cell[3] = {0, 0, 0};
+        for (int a = 0; a < D; ++a) cell[a] = 2 * fc[a] + q[a];
+        if (tab_get<D>(pv, td, b.lvl + 1, cell) >= 0) ok = false;
+      }
+      const bool all = __all_sync(0xffffffffu, ok) && above;
+      const bool first = all && !__any_sync(0xffffffffu, prev);
+      e = make_int2(!all || first ? 1 : 0, all && !first ? 1 : 0);
       if (lane == 0) {
-        double m;
-        detail(s, m);
         pv.mdet[s] = m;
         if (isnan(m)) set_err(pv, kErrNaN);
-        pv.flag[s] = 0;
-        pv.emit[2 * p] = 1;
-        pv.emit[2 * p + 1] = 0;
-      }
-      continue;
-    }
-    // sisters: exist as leaves and below eps
-    bool ok = true;
-    double mine = 0.0;
-    if (lane < NS) {
-      int64_t c[3] = {0, 0, 0};
-      for (int a = 0; a < D; ++a) c[a] = fc[a] | ((lane >> a) & 1);
-      const int t = tab_get<D>(pv, td, b.lvl, c);
-      if (t < 0) {
-        ok = false;
-      } else {
-        double m = 0.0;
-        ok = detail(t, m);
-        if (t == s) mine = m;
+        pv.flag[s] = all ? -2 : 0;
+        pv.emit[2 * p] = e.x;
+        pv.emit[2 * p + 1] = e.y;
       }
     }
-    // no finer leaf around the family: cells of [-1, 4]^d outside [0, 3]^d
-    // (looked up only for a family whose members are all candidates)
-    const bool sisters = __all_sync(0xffffffffu, ok);
-    for (int u = lane; sisters && u < NBOX; u += 32) {
-      const int q[3] = {u % 6 - 1, (u / 6) % 6 - 1, D == 3 ? u / 36 - 1 : 0};
-      bool in = true;
-      for (int a = 0; a < D; ++a) in &= q[a] >= 0 && q[a] <= 3;
-      if (in) continue;
-      int64_t cell[3] = {0, 0, 0};
-      for (int a = 0; a < D; ++a) cell[a] = 2 * fc[a] + q[a];
-      if (tab_get<D>(pv, td, b.lvl + 1, cell) >= 0) ok = false;
-    }
-    const bool all = __all_sync(0xffffffffu, ok) && b.lvl > td.Jmin;
-    const double m = __shfl_sync(0xffffffffu, mine, (int)(((b.c[0] & 1) | (D > 1 ? (b.c[1] & 1) << 1 : 0) |
-                                                          (D > 2 ? (b.c[2] & 1) << 2 : 0))));
-    if (lane == 0) {
-      pv.mdet[s] = m;
-      if (isnan(m)) set_err(pv, kErrNaN);
-      pv.flag[s] = all ? -2 : 0;
-      const bool first = all && (p == 0 || !same_family(pv, s, pv.act[p - 1]));
-      pv.emit[2 * p] = (!all || first) ? 1 : 0;
-      pv.emit[2 * p + 1] = (all && !first) ? 1 : 0;
-    }
+    emit_group(pv, g, nact, sh, par, e);
   }
-  // SCAN: the CTA that finishes last scans the new-list counts (short lists),
-  // which saves the separate scan launch
+  // SCAN: the CTA that finishes last scans the totals, which saves the separate
+  // scan launch
   if constexpr (SCAN) {
     if (last_cta_all(pv.cnt)) {
-      cta_scan2<256, 8>(pv.emit, pv.eoff, nact, &pv.cnt->n_new);
+      scan_groups(pv, nact);
       if (threadIdx.x == 0) pv.cnt->ctas_done = 0;
     }
   }

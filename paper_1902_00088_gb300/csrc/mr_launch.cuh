@@ -31,9 +31,10 @@ static inline int flat_grid(const PoolView& pv, int threads) {
   return (int)(g < 1 ? 1 : g);
 }
 
-// Lists up to this length are scanned by the last CTA of the kernel that wrote
-// the counts (one CTA, a few passes) instead of a separate scan launch.
-constexpr int64_t kFusedScanMax = 8192;
+// Lists up to this length are scanned (the totals of their groups of 8) by the last
+// CTA of the kernel that wrote the counts, in at most two passes, instead of
+// separate scan launches (65536 blocks: 5 against 40 us).
+constexpr int64_t kFusedScanMax = 65536;
 
 // ---------------------------------------------------------------- stage ------
 // 2D blocks of 17^2 nodes: 128-thread CTAs, so small grids run in one wave.
@@ -251,8 +252,8 @@ void launch_refine(const PoolView& pv, const Fields& f, int mode, const int8_t* 
   } else {
     launch_k(lc.pdl, k_refine_count<D, false>, flat_grid(pv, 256), 256, 0, st, pv, mode, mask);
     count_launch();
-    launch_scan2(pv.emit, pv.eoff, pv.partial, &pv.cnt->n_act, pv.cap, &pv.cnt->n_new, st, 2 * (int64_t)lc.n_hint,
-                 lc.pdl != 0);
+    launch_scan2(pv.grp, pv.gof, pv.partial, &pv.cnt->n_act, pv.cap / 8 + 1, &pv.cnt->n_new, st,
+                 2 * (int64_t)lc.n_hint / 8, lc.pdl != 0, 3);
   }
   dispatch_bs<D, RefineRun>(pv, f, lc, st);
   launch_k(lc.pdl, k_refine_commit<D>, flat_grid(pv, 256), 256, 0, st, pv);
@@ -292,20 +293,25 @@ struct DetailsRun {
       if (d64) go(k_details3<TS, double, TS>, Col3::NT, Det3Smem<TS, double>::BYTES);
       else go(k_details3<TS, float, float>, Col3::NT, Det3Smem<float, float>::BYTES);
     } else {
-      if (d64) go(k_details2<B, TS, double, TS>, Det2<B>::NT, Det2Smem<B, TS, double>::BYTES);
-      else go(k_details2<B, TS, float, float>, Det2<B>::NT, Det2Smem<B, float, float>::BYTES);
+      if (d64) go(k_details2<B, TS, double, TS>, Det2<B>::NT, Det2Smem<B, TS, TS, double>::BYTES);
+      else go(k_details2<B, TS, float, float>, Det2<B>::NT, Det2Smem<B, TS, float, float>::BYTES);
     }
   }
 };
 template <int D, int B, typename TS>
 struct CoarsenRun {
   static void run(const PoolView& pv, const Fields& f, const RoundCtl& rc, const LaunchCfg& lc, cudaStream_t st) {
-    constexpr int threads = 256;
-    const size_t smem = sizeof(TS) * pv.nvar * Geo<D, B>::NI;
-    auto k = k_coarsen<D, B, TS>;
-    prep_smem(k, smem);
-    launch_k(lc.pdl, k, persistent_grid(k, threads, smem, lc, 0), threads, smem, st, pv, (TS*)f.y, rc);
-    count_launch();
+    auto go = [&](auto k, int threads, size_t smem) {
+      prep_smem(k, smem);
+      launch_k(lc.pdl, k, persistent_grid(k, threads, smem, lc, 0), threads, smem, st, pv, (TS*)f.y, rc);
+      count_launch();
+    };
+    if constexpr (D == 3) {
+      go(k_coarsen3<B, TS>, 256, sizeof(TS) * Geo<3, B>::NI);
+    } else {
+      if (pv.nvar == 1) go(k_coarsen2<B, 1, TS>, Coarsen2<B, 1>::NT, 0);
+      else go(k_coarsen2<B, 4, TS>, Coarsen2<B, 4>::NT, 0);
+    }
   }
 };
 
@@ -337,8 +343,8 @@ void launch_round_merge(const PoolView& pv, const Fields& f, bool merge, const R
     launch_k(lc.pdl, k_flags<D, false>, grid, 256, 0, st, pv);
     count_launch();
     if (!merge) return;
-    launch_scan2(pv.emit, pv.eoff, pv.partial, &pv.cnt->n_round, pv.cap, &pv.cnt->n_new, st, 4 * (int64_t)lc.n_hint,
-                 lc.pdl != 0);
+    launch_scan2(pv.grp, pv.gof, pv.partial, &pv.cnt->n_round, pv.cap / 8 + 1, &pv.cnt->n_new, st,
+                 4 * (int64_t)lc.n_hint / 8, lc.pdl != 0, 3);
   }
   dispatch_bs<D, CoarsenRun>(pv, f, rc, lc, st);
   (void)nch;

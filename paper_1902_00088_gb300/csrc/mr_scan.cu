@@ -13,8 +13,8 @@ int64_t kernel_launches() { return g_launches.load(); }
 constexpr int kScanThreads = 256;
 constexpr int kPer = kScanChunk / kScanThreads;  // 8 pairs per thread
 
-__device__ __forceinline__ int64_t scan_n(const int32_t* n_dev, int64_t n_host) {
-  return n_dev ? (int64_t)*n_dev : n_host;
+__device__ __forceinline__ int64_t scan_n(const int32_t* n_dev, int64_t n_host, int shift) {
+  return n_dev ? ((int64_t)*n_dev + (1 << shift) - 1) >> shift : n_host;
 }
 
 // inclusive block scan of (a, b) over 256 threads
@@ -39,10 +39,11 @@ __device__ __forceinline__ int2 block_incl_scan(int2 v, int2* warp_tot) {
   return v;
 }
 
-__global__ void k_scan_reduce(const int32_t* in, const int32_t* n_dev, int64_t n_host, int32_t* partial) {
+__global__ void k_scan_reduce(const int32_t* in, const int32_t* n_dev, int64_t n_host, int32_t* partial,
+                              int shift) {
   pdl_enter();
   __shared__ int2 wt[kScanThreads / 32];
-  const int64_t n = scan_n(n_dev, n_host);
+  const int64_t n = scan_n(n_dev, n_host, shift);
   const int64_t start = (int64_t)blockIdx.x * kScanChunk;
   int2 s = make_int2(0, 0);
   for (int r = 0; r < kPer; ++r) {
@@ -79,10 +80,10 @@ __global__ void k_scan_partials(int32_t* partial, int nchunks, int32_t* tot) {
 }
 
 __global__ void k_scan_final(const int32_t* in, int32_t* out, const int32_t* n_dev, int64_t n_host,
-                             const int32_t* partial) {
+                             const int32_t* partial, int shift) {
   pdl_enter();
   __shared__ int2 wt[kScanThreads / 32];
-  const int64_t n = scan_n(n_dev, n_host);
+  const int64_t n = scan_n(n_dev, n_host, shift);
   const int64_t start = (int64_t)blockIdx.x * kScanChunk;
   if (start >= n) return;
   int2 loc[kPer];
@@ -106,10 +107,10 @@ __global__ void k_scan_final(const int32_t* in, int32_t* out, const int32_t* n_d
 // device-side count, so it serves lists up to a few million entries.
 constexpr int kSingleThreads = 1024, kSinglePer = 4;
 __global__ void __launch_bounds__(kSingleThreads) k_scan_single(const int32_t* in, int32_t* out, const int32_t* n_dev,
-                                                                int64_t n_host, int32_t* tot) {
+                                                                int64_t n_host, int32_t* tot, int shift) {
   pdl_enter();
   __shared__ int2 wt[kSingleThreads / 32];
-  const int64_t n = scan_n(n_dev, n_host);
+  const int64_t n = scan_n(n_dev, n_host, shift);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   int2 carry = make_int2(0, 0);
   for (int64_t base = 0; base < n; base += (int64_t)kSingleThreads * kSinglePer) {
@@ -155,19 +156,19 @@ __global__ void __launch_bounds__(kSingleThreads) k_scan_single(const int32_t* i
 }
 
 void launch_scan2(const int32_t* in, int32_t* out, int32_t* partial, const int32_t* n_dev,
-                  int64_t n_host, int32_t* tot, cudaStream_t st, int64_t n_expect, bool pdl) {
+                  int64_t n_host, int32_t* tot, cudaStream_t st, int64_t n_expect, bool pdl, int shift) {
   // one CTA while the list is expected to be short (its passes are serial)
   const int64_t n_est = n_expect >= 0 ? n_expect : n_host;
   if (n_est <= 32768) {
-    launch_k(pdl, k_scan_single, 1, kSingleThreads, 0, st, in, out, n_dev, n_host, tot);
+    launch_k(pdl, k_scan_single, 1, kSingleThreads, 0, st, in, out, n_dev, n_host, tot, shift);
     count_launch(1);
     return;
   }
   const int nchunks = (int)((n_host + kScanChunk - 1) / kScanChunk);
   const int g = nchunks < 1 ? 1 : nchunks;
-  launch_k(pdl, k_scan_reduce, g, kScanThreads, 0, st, in, n_dev, n_host, partial);
+  launch_k(pdl, k_scan_reduce, g, kScanThreads, 0, st, in, n_dev, n_host, partial, shift);
   launch_k(pdl, k_scan_partials, 1, kScanThreads, 0, st, partial, g, tot);
-  launch_k(pdl, k_scan_final, g, kScanThreads, 0, st, in, out, n_dev, n_host, partial);
+  launch_k(pdl, k_scan_final, g, kScanThreads, 0, st, in, out, n_dev, n_host, partial, shift);
   count_launch(3);
 }
 
