@@ -883,67 +883,6 @@ __device__ __forceinline__ BlockInfo plan_block(const int32_t* pl) {
   return b;
 }
 
-// Ghost gather for a block with a uniform neighbourhood: node i of an axis
-// comes from the left neighbour (i < 0, local i + B - 1), the block itself
-// (0 <= i <= B - 2) or the right neighbour (i >= B - 1, local i - (B - 1));
-// the tile box of width W is filled (NV variables, TF -> TT).  Loads are issued
-// U at a time before their stores so that they are in flight together.  With
-// commit, block-edge nodes taken from a neighbour are written back into Fw
-// where they differ (the neighbour owns them).
-template <int D, int B, int W, int NV, typename TF, typename TT>
-__device__ __forceinline__ void gather_uniform(const PoolView& pv, const BlockInfo& b, const int32_t* nb,
-                                               const TF* F, TF* Fw, TT* tile, bool commit) {
-  using Gm = Geo<D, B>;
-  using Bx = Box<D, B, W>;
-  constexpr int U = 4;
-  const int64_t own = (int64_t)b.slot * NV * pv.vs;
-  for (int q0 = threadIdx.x; q0 < Bx::NPTS; q0 += U * blockDim.x) {
-    int64_t at[U];
-    int idx[U], li[U];
-    bool ok[U], ed[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int q = q0 + u * blockDim.x;
-      ok[u] = q < Bx::NPTS;
-      const int qq = ok[u] ? q : 0;
-      const int ijk[3] = {qq % Bx::S - W, (qq / Bx::S) % Bx::S - W, D == 3 ? qq / (Bx::S * Bx::S) - W : 0};
-      int n = 0, mul = 1, l3[3] = {0, 0, 0};
-      bool inner = true;
-#pragma unroll
-      for (int a = 0; a < D; ++a) {
-        const int x = ijk[a];
-        const int s = x < 0 ? 0 : (x <= B - 2 ? 1 : 2);
-        l3[a] = x - (s - 1) * (B - 1);
-        n += s * mul;
-        mul *= 3;
-        inner &= (x >= 0 && x <= B - 1);
-      }
-      const int slot = nb[n];
-      at[u] = (int64_t)slot * NV * pv.vs + Gm::lin(l3[0], l3[1], l3[2]);
-      idx[u] = Bx::tix(ijk[0], ijk[1], ijk[2]);
-      li[u] = Gm::lin(ijk[0], ijk[1], ijk[2]);
-      ed[u] = commit && inner && slot != b.slot;
-    }
-    TF v[U][NV];
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-#pragma unroll
-      for (int w = 0; w < NV; ++w) v[u][w] = ok[u] ? F[at[u] + (int64_t)w * pv.vs] : TF(0);
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (!ok[u]) continue;
-#pragma unroll
-      for (int w = 0; w < NV; ++w) {
-        tile[w * Bx::TILE + idx[u]] = (TT)v[u][w];
-        if (ed[u]) {
-          const int64_t me = own + (int64_t)w * pv.vs + li[u];
-          if (F[me] != v[u][w]) Fw[me] = v[u][w];
-        }
-      }
-    }
-  }
-}
-
 // Gather table of a tile box, the same for every block: entry q (tile index
 // of node (i, j, k), x fastest) = local offset of the node in the block that
 // owns it in a uniform neighbourhood | neighbour index (0 .. 3^d - 1) << 16 |
@@ -970,7 +909,6 @@ __device__ void build_gtab(int32_t* gtab) {
 
 // Uniform-neighbourhood gather through the gather table: nbase[n] is the pool
 // offset of neighbour n's variable 0 (slot * NV * vs), own the block's.
-// Same values as gather_uniform.
 template <int D, int B, int W, int NV, typename TF, typename TT, typename G = CtaGroup>
 __device__ __forceinline__ void gather_table(const PoolView& pv, int64_t own, const int64_t* nbase,
                                              const int32_t* gtab, const TF* F, TF* Fw, TT* tile, bool commit) {

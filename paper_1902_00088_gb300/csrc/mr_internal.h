@@ -236,11 +236,13 @@ template <int D> void launch_set_blocks(const PoolView& pv, const Fields& f, int
                                         cudaStream_t st);
 template <int D> void launch_error(const PoolView& pv, const Fields& f, int tree, const double* ex,
                                    double* out4, const LaunchCfg& lc, cudaStream_t st);
-// Navier-Stokes of Sec. 4 (mr_ns.cu): RK stage in the skew-symmetric form
-// (2D, B = 17 or 33), and the shock-capturing filter of the state, in place,
+// Navier-Stokes of Sec. 4 (mr_ns.cu): RK stage in the flux form and in the
+// skew-symmetric form (2D, B = 17 or 33), and the shock-capturing filter of the state, in place,
 // from the copy of the state in the stage type in Yb (written by the last RK
 // stage with StageArgs::copy_state, or first by the filter itself with copy);
 // it needs the stage plan of the current grid.
+template <int B> void launch_stage_ns(const PoolView& pv, const Fields& f, int stage,
+                                      const StageArgs& sa, const LaunchCfg& lc, cudaStream_t st);
 template <int B> void launch_stage_nss(const PoolView& pv, const Fields& f, int stage,
                                        const StageArgs& sa, const LaunchCfg& lc, cudaStream_t st);
 void launch_filter(const PoolView& pv, const Fields& f, bool copy, const LaunchCfg& lc, cudaStream_t st);

@@ -443,212 +443,6 @@ __device__ __forceinline__ int2 new_offset(const PoolView& pv, int p) {
   return make_int2(g.x + l.x, g.y + l.y);
 }
 
-// ------------------------------------------------------------- NS stage ----
-// One RK4 stage of the 2D compressible Navier-Stokes equations (Sec. 4), ideal
-// gas with constant c_p, in conservative flux form, q = (rho, rho u, rho v, E):
-//   N(q) = -(dF/dx + dG/dy),
-//   F = (rho u, rho u u + p - txx, rho u v - txy, (E + p) u - (u txx + v txy) - kap dth/dx),
-//   G = (rho v, rho v u - txy, rho v v + p - tyy, (E + p) v - (u txy + v tyy) - kap dth/dy),
-//   txx = mu (2 ux - 2/3 div), tyy = mu (2 vy - 2/3 div), txy = mu (uy + vx),
-//   p = (gamma - 1)(E - (rho u u + rho v v)/2), th = p / rho,
-//   kap = mu gamma / ((gamma - 1) Pr)  (R_s cancels in the heat flux),
-// every derivative the 4th-order central D1.  Primitives on the whole tile,
-// gradients and fluxes on nodes -2..B+1, flux divergence on the interior; the
-// RK4 update is the same 3-register form as for advection, on 4 variables
-// (with StageArgs::copy_state the last stage also stores the new state in the
-// stage type into ynext, the shock filter's source).
-template <int B>
-struct NsGeo {
-  static constexpr int NF = (B + 4) * B;  // F on i in [-2, B+1], j in [0, B-1]
-  static constexpr int NG = B * (B + 4);  // G on i in [0, B-1], j in [-2, B+1]
-};
-
-template <int B, typename TS, typename TY, typename TSRC>
-__global__ void __launch_bounds__(256) k_stage_ns(PoolView pv, const TSRC* __restrict__ src,
-                                                  TS* __restrict__ y, TS* __restrict__ acc,
-                                                  TY* __restrict__ ynext, TY* __restrict__ yn, int stage,
-                                                  StageArgs sa) {
-  pdl_enter();
-  using Gm = Geo<2, B>;
-  using NG = NsGeo<B>;
-  using TC = TY;
-  constexpr int T = Gm::T, G = Gm::G;
-  RingD<2>& R = *smem_as<RingD<2>>(0);
-  TC* tile = smem_as<TC>(kRingBytesD<2>);  // 4 x TILE conserved variables
-  TC* cbox = tile + 4 * Gm::TILE;         // 4 x CBOX
-  TC* pu = cbox + 4 * Gm::CBOX;           // primitives u, v, p, th: 4 x TILE
-  TC* pvv = pu + Gm::TILE;
-  TC* pp = pvv + Gm::TILE;
-  TC* pth = pp + Gm::TILE;
-  TC* F = pth + Gm::TILE;                 // 4 x NF
-  TC* Gf = F + 4 * NG::NF;                // 4 x NG
-  static_assert(Box<2, B, kG>::SCR <= Gm::TILE, "prediction scratch fits in the primitive arrays");
-  using PL = Plan<2>;
-  __shared__ int32_t splan[2][PL::INTS];
-  const int nact = pv.cnt->n_act;
-  if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&pv.cnt->stage_blocks, (unsigned long long)nact);
-  auto I = [&](int i, int j) { return (j + G) * T + (i + G); };
-  auto fI = [&](int i, int j) { return j * (B + 4) + (i + 2); };
-  auto gI = [&](int i, int j) { return (j + 2) * B + i; };
-  if (blockIdx.x < nact && threadIdx.x < PL::INTS)
-    splan[0][threadIdx.x] = pv.plan[(int64_t)blockIdx.x * PL::INTS + threadIdx.x];
-  __syncthreads();
-  int buf = 0;
-  for (int p = blockIdx.x; p < nact; p += gridDim.x, buf ^= 1) {
-    const int pn = p + gridDim.x;
-    int32_t pre = 0;
-    if (pn < nact && threadIdx.x < PL::INTS) pre = pv.plan[(int64_t)pn * PL::INTS + threadIdx.x];
-    const int32_t* pl = splan[buf];
-    const BlockInfo b = plan_block<2>(pl);
-    const TreeDev& td = pv.trees[b.tree];
-    if ((pl[1] >> 30) & 1) {
-      gather_uniform<2, B, kG, 4, TSRC, TC>(pv, b, pl + PL::NBO, src, (TSRC*)src, tile, stage == 0);
-    } else {
-      load_regions<2, CtaGroup>(pv, p, R);
-      __syncthreads();
-      // prediction scratch: the primitive arrays, unused until the tile is complete
-      fill_tile<2, B, TSRC, TC>(pv, b, src, (TSRC*)src, tile, stage == 0, R, cbox, pu, true);
-    }
-    __syncthreads();
-    // gamma - 1, mu and kappa = mu gamma / ((gamma - 1) Pr), formed once per tree
-    TC gm1, mu, kap;
-    if constexpr (sizeof(TC) == 4) { gm1 = td.nsf[0]; mu = td.nsf[1]; kap = td.nsf[2]; }
-    else { gm1 = td.nsd[0]; mu = td.nsd[1]; kap = td.nsd[2]; }
-    const TC c23 = (TC)(2.0 / 3.0);
-    const TC c = tree_cD<TC>(td, b.lvl);
-    const TC* r_ = tile;
-    const TC* m1_ = tile + Gm::TILE;
-    const TC* m2_ = tile + 2 * Gm::TILE;
-    const TC* E_ = tile + 3 * Gm::TILE;
-    for (int idx = threadIdx.x; idx < Gm::TILE; idx += blockDim.x) {
-      const TC r = r_[idx], m1 = m1_[idx], m2 = m2_[idx], E = E_[idx];
-      const TC uu = m1 / r, vv = m2 / r;
-      const TC prs = gm1 * (E - TC(0.5) * (m1 * uu + m2 * vv));
-      pu[idx] = uu;
-      pvv[idx] = vv;
-      pp[idx] = prs;
-      pth[idx] = prs / r;
-    }
-    __syncthreads();
-    auto dx = [&](const TC* f, int i, int j) {
-      return ((f[I(i - 2, j)] - f[I(i + 2, j)]) + TC(8) * (f[I(i + 1, j)] - f[I(i - 1, j)])) * c;
-    };
-    auto dy = [&](const TC* f, int i, int j) {
-      return ((f[I(i, j - 2)] - f[I(i, j + 2)]) + TC(8) * (f[I(i, j + 1)] - f[I(i, j - 1)])) * c;
-    };
-    constexpr int W = B + 4;
-    for (int idx = threadIdx.x; idx < W * W; idx += blockDim.x) {
-      const int i = idx % W - 2, j = idx / W - 2;
-      const bool needF = j >= 0 && j < B, needG = i >= 0 && i < B;
-      if (!needF && !needG) continue;
-      const TC ux = dx(pu, i, j), vx = dx(pvv, i, j), uy = dy(pu, i, j), vy = dy(pvv, i, j);
-      const TC div = ux + vy;
-      const TC txy = mu * (uy + vx);
-      const int t0 = I(i, j);
-      const TC m1 = m1_[t0], m2 = m2_[t0], E = E_[t0];
-      const TC uu = pu[t0], vv = pvv[t0], prs = pp[t0];
-      if (needF) {
-        const TC txx = mu * (TC(2) * ux - c23 * div);
-        const TC thx = dx(pth, i, j);
-        const int f0 = fI(i, j);
-        F[f0] = m1;
-        F[NG::NF + f0] = m1 * uu + prs - txx;
-        F[2 * NG::NF + f0] = m1 * vv - txy;
-        F[3 * NG::NF + f0] = (E + prs) * uu - (uu * txx + vv * txy) - kap * thx;
-      }
-      if (needG) {
-        const TC tyy = mu * (TC(2) * vy - c23 * div);
-        const TC thy = dy(pth, i, j);
-        const int g0 = gI(i, j);
-        Gf[g0] = m2;
-        Gf[NG::NG + g0] = m2 * uu - txy;
-        Gf[2 * NG::NG + g0] = m2 * vv + prs - tyy;
-        Gf[3 * NG::NG + g0] = (E + prs) * vv - (uu * txy + vv * tyy) - kap * thy;
-      }
-    }
-    __syncthreads();
-    const StageCoef<TS> cs(pv, sa, b.tree, stage);
-    const StageCoef<TC> cf(pv, sa, b.tree, stage);
-    const int64_t base = (int64_t)b.slot * 4 * pv.vs;
-    const TS cas = cs.ca, cys = cs.cy;  // RK weights in the state type
-    const TC casf = cf.ca, cysf = cf.cy;  // and in the stage type
-    // UC points per thread at a time: state and accumulator loads first.  With
-    // an FP64 state and FP32 stages the next stage field needs y_n only in FP32:
-    // stage 0 takes it from the tile (the committed state, rounded) and keeps
-    // it in yn for stages 1 and 2, which then read no FP64 state.
-    constexpr bool MIX = sizeof(TS) == 8 && sizeof(TC) == 4;
-    constexpr int UC = 4, NT = 256;
-    for (int i0 = threadIdx.x; i0 < 4 * Gm::NI; i0 += UC * NT) {
-      TS yv[UC], av[UC];
-      TC yf[UC];
-#pragma unroll
-      for (int u = 0; u < UC; ++u) {
-        const int idx = i0 + u * NT;
-        yv[u] = av[u] = TS(0);
-        yf[u] = TC(0);
-        if (idx >= 4 * Gm::NI) continue;
-        const int v = idx / Gm::NI, q = idx % Gm::NI;
-        const int64_t at = base + (int64_t)v * pv.vs + q;
-        if (stage == 0 || (!MIX && stage <= 2)) yv[u] = y[at];
-        if (stage >= 1) av[u] = acc[at];
-        if constexpr (MIX) {
-          if (stage == 0) {
-            yf[u] = tile[v * Gm::TILE + I(q % B, q / B)];
-            yn[at] = yf[u];
-          } else if (stage <= 2) {
-            yf[u] = yn[at];
-          }
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < UC; ++u) {
-        const int idx = i0 + u * NT;
-        if (idx >= 4 * Gm::NI) continue;
-        const int v = idx / Gm::NI, q = idx % Gm::NI;
-        const int i = q % B, j = q / B;
-        const TC* Fv = F + v * NG::NF;
-        const TC* Gv = Gf + v * NG::NG;
-        const TC dFx = ((Fv[fI(i - 2, j)] - Fv[fI(i + 2, j)]) + TC(8) * (Fv[fI(i + 1, j)] - Fv[fI(i - 1, j)])) * c;
-        const TC dGy = ((Gv[gI(i, j - 2)] - Gv[gI(i, j + 2)]) + TC(8) * (Gv[gI(i, j + 1)] - Gv[gI(i, j - 1)])) * c;
-        const int64_t at = base + (int64_t)v * pv.vs + q;
-        if constexpr (sizeof(TS) == 8 && sizeof(TC) == 4) {
-          // FP64 state, FP32 stages: the increments dt k are formed in FP32 and
-          // only accumulated in FP64 (one conversion and one FP64 add per
-          // update; FP64 arithmetic is a small fraction of the FP32 rate here),
-          // the FP32 stage value from the FP32-rounded state
-          const TC kc = -(dFx + dGy);
-          if (stage == 0) {
-            acc[at] = yv[u] + (TS)(casf * kc);
-            ynext[at] = (TY)(yf[u] + cysf * kc);
-          } else if (stage == 1 || stage == 2) {
-            acc[at] = av[u] + (TS)(casf * kc);
-            ynext[at] = (TY)(yf[u] + cysf * kc);
-          } else {
-            const TS yn = av[u] + (TS)(casf * kc);
-            y[at] = yn;
-            if (sa.copy_state) ynext[at] = (TY)yn;
-          }
-        } else {
-          const TS kk = (TS)(-(dFx + dGy));
-          if (stage == 0) {
-            acc[at] = yv[u] + cas * kk;
-            ynext[at] = (TY)(yv[u] + cys * kk);
-          } else if (stage == 1 || stage == 2) {
-            acc[at] = av[u] + cas * kk;
-            ynext[at] = (TY)(yv[u] + cys * kk);
-          } else {
-            const TS yn = av[u] + cas * kk;
-            y[at] = yn;
-            if (sa.copy_state) ynext[at] = (TY)yn;
-          }
-        }
-      }
-    }
-    if (pn < nact && threadIdx.x < PL::INTS) splan[buf ^ 1][threadIdx.x] = pre;
-    __syncthreads();
-  }
-}
-
 // ----------------------------------------------------------------- refine ----
 // x pass of the upsampling: fine x in [0, 2(B-1)] on mother rows y in [-1, B]
 template <int B>

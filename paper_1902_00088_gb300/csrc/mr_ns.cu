@@ -1,50 +1,65 @@
-// Launchers of the Navier-Stokes kernels of Sec. 4 (skew-symmetric stage and
+// Launchers of the Navier-Stokes kernels of Sec. 4 (the stages of both forms and the
 // shock-capturing filter), 2D, Bs 17 and 33.
 #include "mr_launch.cuh"
 #include "mr_ns.cuh"
 
 namespace mr {
 
-template <int B, typename TS, typename TY>
-static void stage_nss_impl(const PoolView& pv, const Fields& f, int stage, const StageArgs& sa,
-                           const LaunchCfg& lc, cudaStream_t st) {
-  constexpr int threads = NssCfg<B>::NT;
-  constexpr size_t smem = nss_smem<B, TY>();
-  // stage s reads y, Ya, Yb, Ya and writes Ya, Yb, Ya, (Yb: the new state's copy for the filter)
+// One stage of either form: stage s reads y, Ya, Yb, Ya and writes Ya, Yb, Ya, (Yb:
+// the new state's copy for the filter).
+template <int B, bool SKEW, typename TS, typename TY>
+static void stage_form(const PoolView& pv, const Fields& f, int stage, const StageArgs& sa,
+                       const LaunchCfg& lc, cudaStream_t st) {
+  constexpr int threads = SKEW ? NssCfg<B, TY>::NT : NsCfg<B, TY>::NT;
+  constexpr size_t smem = SKEW ? NssSmem<B, TY>::BYTES : NsSmem<B, TY>::BYTES;
   TY* ynext = (TY*)(stage == 1 || stage == 3 ? f.Yb : f.Ya);
-  if (stage == 0) {
-    auto k = k_stage_nss<B, TS, TY, TS>;
-    prep_smem(k, smem);
-    launch_k(lc.pdl, k, persistent_grid(k, threads, smem, lc, lc.grid_mult), threads, smem, st, pv,
-             (const TS*)f.y, (TS*)f.y, (TS*)f.acc, ynext, (TY*)f.Yn, stage, sa);
-  } else {
-    const TY* src = (const TY*)(stage == 2 ? f.Yb : f.Ya);
-    auto k = k_stage_nss<B, TS, TY, TY>;
+  auto go = [&](auto k, auto src) {
     prep_smem(k, smem);
     launch_k(lc.pdl, k, persistent_grid(k, threads, smem, lc, lc.grid_mult), threads, smem, st, pv, src,
              (TS*)f.y, (TS*)f.acc, ynext, (TY*)f.Yn, stage, sa);
+  };
+  const TY* src = (const TY*)(stage == 2 ? f.Yb : f.Ya);
+  if constexpr (SKEW) {
+    if (stage == 0) go(k_stage_nss<B, TS, TY, TS>, (const TS*)f.y);
+    else go(k_stage_nss<B, TS, TY, TY>, src);
+  } else {
+    if (stage == 0) go(k_stage_ns<B, TS, TY, TS>, (const TS*)f.y);
+    else go(k_stage_ns<B, TS, TY, TY>, src);
   }
   count_launch();
 }
 
-template <int B>
-void launch_stage_nss(const PoolView& pv, const Fields& f, int stage, const StageArgs& sa,
-                      const LaunchCfg& lc, cudaStream_t st) {
+template <int B, bool SKEW>
+static void stage_prec_ns(const PoolView& pv, const Fields& f, int stage, const StageArgs& sa,
+                          const LaunchCfg& lc, cudaStream_t st) {
   switch (pv.prec) {
-    case MR_PREC_FP64: stage_nss_impl<B, double, double>(pv, f, stage, sa, lc, st); break;
-    case MR_PREC_FP32: stage_nss_impl<B, float, float>(pv, f, stage, sa, lc, st); break;
-    default: stage_nss_impl<B, double, float>(pv, f, stage, sa, lc, st); break;
+    case MR_PREC_FP64: stage_form<B, SKEW, double, double>(pv, f, stage, sa, lc, st); break;
+    case MR_PREC_FP32: stage_form<B, SKEW, float, float>(pv, f, stage, sa, lc, st); break;
+    default: stage_form<B, SKEW, double, float>(pv, f, stage, sa, lc, st); break;
   }
 }
-template void launch_stage_nss<17>(const PoolView&, const Fields&, int, const StageArgs&, const LaunchCfg&,
-                                   cudaStream_t);
-template void launch_stage_nss<33>(const PoolView&, const Fields&, int, const StageArgs&, const LaunchCfg&,
-                                   cudaStream_t);
+template <int B>
+void launch_stage_ns(const PoolView& pv, const Fields& f, int stage, const StageArgs& sa, const LaunchCfg& lc,
+                     cudaStream_t st) {
+  stage_prec_ns<B, false>(pv, f, stage, sa, lc, st);
+}
+template <int B>
+void launch_stage_nss(const PoolView& pv, const Fields& f, int stage, const StageArgs& sa, const LaunchCfg& lc,
+                      cudaStream_t st) {
+  stage_prec_ns<B, true>(pv, f, stage, sa, lc, st);
+}
+#define MR_NS_STAGE(B)                                                                                                \
+  template void launch_stage_ns<B>(const PoolView&, const Fields&, int, const StageArgs&, const LaunchCfg&,           \
+                                   cudaStream_t);                                                                     \
+  template void launch_stage_nss<B>(const PoolView&, const Fields&, int, const StageArgs&, const LaunchCfg&,          \
+                                    cudaStream_t);
+MR_NS_STAGE(17)
+MR_NS_STAGE(33)
 
 template <int B, typename TS, typename TC, int KIND>
 static void filter_impl(const PoolView& pv, const Fields& f, bool copy, const LaunchCfg& lc, cudaStream_t st) {
   constexpr int threads = kFilterThreads;
-  constexpr size_t smem = filter_smem<B, TC>();
+  constexpr size_t smem = FilterSmem<B, TC>::BYTES;
   if (copy) {
     launch_k(lc.pdl, k_state_copy<TS, TC>, lc.num_sms * 8, 256, 0, st, pv, (const TS*)f.y, (TC*)f.Yb);
     count_launch();
