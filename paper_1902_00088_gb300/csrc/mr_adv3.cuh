@@ -33,7 +33,7 @@ struct ColOwn {
 };
 
 // ------------------------------------------------------------------ stage ----
-// RK4 stage of the 3D advection equation (k_stage_adv's formulas and order of
+// RK4 stage of the 3D advection equation (k_stage2's formulas and order of
 // operations).  The stencil is a cross, so only the six face layers of width 2
 // are gathered: 3468 ghost nodes per block instead of the 4348 with edges and
 // corners, and of a coarser neighbour only the layers of its face are
@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(Stage3Smem<TY, TS>::NT, 2) k_stage3(PoolView p
         if constexpr (PRE) {
 #pragma unroll
           for (int j = 0; j < NZ; ++j) {
-            if constexpr (NEEDY || Y0MEM) yv[j] = y[me + NQ * j];
+            if constexpr (NEEDY || Y0MEM) yv[j] = (Y0MEM ? committed(y, src) : y)[me + NQ * j];
             if constexpr (ST >= 1) av[j] = acc[me + NQ * j];
           }
         }
@@ -516,7 +516,7 @@ __global__ void __launch_bounds__(Stage3Smem<TY, TS>::NT, 2) k_stage3(PoolView p
       TS yk = TS(0), ak = TS(0);
       if (NEEDY) yk = ROWS ? yrow[q] : y[own + q];
       if (ST >= 1) ak = ROWS ? arow[q] : acc[own + q];
-      if (ST == 0) yk = sizeof(TS) == sizeof(TC) ? (TS)zl[z + 2] : y[own + q];
+      if (ST == 0) yk = sizeof(TS) == sizeof(TC) ? (TS)zl[z + 2] : committed(y, src)[own + q];
       node(own + q, tile + SM::at(B - 1, B - 1) + k, tile + SM::at(B - 3, B - 1) + k, tile + SM::at(B - 2, B - 1) + k,
            tile + SM::at(B, B - 1) + k, tile + SM::at(B + 1, B - 1) + k, zl[z], zl[z + 1], zl[z + 3], zl[z + 4], yk, ak);
     }

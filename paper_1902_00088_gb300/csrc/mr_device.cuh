@@ -99,6 +99,15 @@ __device__ __forceinline__ bool differs(double a, double b) {
   return x != z && ((x | z) << 1) != 0;  // +0 equals -0; equal NaN patterns need no store
 }
 
+// The state y after its edge nodes were stored through another pointer to it (src),
+// past a barrier: both are __restrict__ kernel arguments, so without this the
+// compiler may take loads of y before those stores, or through the read-only path.
+template <typename T>
+__device__ __forceinline__ const T* committed(const T* y, const void* src) {
+  asm volatile("" : "+l"(y) : "l"(src) : "memory");
+  return y;
+}
+
 // Thread groups that cooperate on one block: the whole CTA, or one warp.
 struct CtaGroup {
   static constexpr int kSize = 0;  // size known at run time only
@@ -881,85 +890,6 @@ __device__ __forceinline__ BlockInfo plan_block(const int32_t* pl) {
 #pragma unroll
   for (int a = 0; a < 3; ++a) b.c[a] = a < D ? pl[2 + a] : 0;
   return b;
-}
-
-// Gather table of a tile box, the same for every block: entry q (tile index
-// of node (i, j, k), x fastest) = local offset of the node in the block that
-// owns it in a uniform neighbourhood | neighbour index (0 .. 3^d - 1) << 16 |
-// (node inside the block) << 21.
-template <int D, int B, int W>
-__device__ void build_gtab(int32_t* gtab) {
-  using Bx = Box<D, B, W>;
-  using Gm = Geo<D, B>;
-  for (int q = threadIdx.x; q < Bx::NPTS; q += blockDim.x) {
-    const int ijk[3] = {q % Bx::S - W, (q / Bx::S) % Bx::S - W, D == 3 ? q / (Bx::S * Bx::S) - W : 0};
-    int n = 0, mul = 1, l3[3] = {0, 0, 0};
-    bool inner = true;
-    for (int a = 0; a < D; ++a) {
-      const int x = ijk[a];
-      const int s = x < 0 ? 0 : (x <= B - 2 ? 1 : 2);
-      l3[a] = x - (s - 1) * (B - 1);
-      n += s * mul;
-      mul *= 3;
-      inner &= (x >= 0 && x <= B - 1);
-    }
-    gtab[q] = Gm::lin(l3[0], l3[1], l3[2]) | (n << 16) | ((inner ? 1 : 0) << 21);
-  }
-}
-
-// Uniform-neighbourhood gather through the gather table: nbase[n] is the pool
-// offset of neighbour n's variable 0 (slot * NV * vs), own the block's.
-template <int D, int B, int W, int NV, typename TF, typename TT, typename G = CtaGroup>
-__device__ __forceinline__ void gather_table(const PoolView& pv, int64_t own, const int64_t* nbase,
-                                             const int32_t* gtab, const TF* F, TF* Fw, TT* tile, bool commit) {
-  const G g{};
-  using Bx = Box<D, B, W>;
-  using Gm = Geo<D, B>;
-  constexpr int U = 4;
-  // points q0 + u * stride, u < UU: table entries, then the UU loads together
-  auto chunk = [&](auto uu, int q0, int stride) {
-    constexpr int UU = decltype(uu)::value;
-    int64_t at[UU];
-    bool ok[UU], ed[UU];
-#pragma unroll
-    for (int u = 0; u < UU; ++u) {
-      const int q = q0 + u * stride;
-      ok[u] = q < Bx::NPTS;
-      const int e = gtab[ok[u] ? q : 0];
-      const int64_t nbv = nbase[(e >> 16) & 31];
-      at[u] = nbv + (e & 0xffff);
-      ed[u] = commit && ((e >> 21) & 1) && nbv != own;
-    }
-    TF v[UU][NV];
-#pragma unroll
-    for (int u = 0; u < UU; ++u)
-#pragma unroll
-      for (int w = 0; w < NV; ++w) v[u][w] = ok[u] ? F[at[u] + (int64_t)w * pv.vs] : TF(0);
-#pragma unroll
-    for (int u = 0; u < UU; ++u) {
-      if (!ok[u]) continue;
-      const int q = q0 + u * stride;
-#pragma unroll
-      for (int w = 0; w < NV; ++w) {
-        tile[w * Bx::TILE + q] = (TT)v[u][w];
-        if (ed[u]) {
-          const int i = q % Bx::S - W, j = (q / Bx::S) % Bx::S - W, k = D == 3 ? q / (Bx::S * Bx::S) - W : 0;
-          const int64_t me = own + (int64_t)w * pv.vs + Gm::lin(i, j, k);
-          if (F[me] != v[u][w]) Fw[me] = v[u][w];
-        }
-      }
-    }
-  };
-  if constexpr (G::kSize > 0) {
-    // group size known at compile time: full chunks of U, then one chunk just
-    // wide enough for the remaining points
-    constexpr int SZ = G::kSize, FULL = Bx::NPTS / (U * SZ) * (U * SZ);
-    constexpr int UT = (Bx::NPTS - FULL + SZ - 1) / SZ;
-    for (int q0 = g.rank(); q0 < FULL; q0 += U * SZ) chunk(std::integral_constant<int, U>{}, q0, SZ);
-    if constexpr (UT > 0) chunk(std::integral_constant<int, UT>{}, FULL + g.rank(), SZ);
-  } else {
-    for (int q0 = g.rank(); q0 < Bx::NPTS; q0 += U * g.size()) chunk(std::integral_constant<int, U>{}, q0, g.size());
-  }
 }
 
 template <typename T>

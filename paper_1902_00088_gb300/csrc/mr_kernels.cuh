@@ -42,311 +42,7 @@ __device__ __forceinline__ double d1_sum(double fm2, double fm1, double f1, doub
   return __fma_rn(8.0, f1 - fm1, fm2 - f2);
 }
 
-// ------------------------------------------------------------------ stage ----
-// One RK4 stage on every block (Sec. 3: 4th-order central FD + classic RK4):
-//   k = N(Y_s) on the synchronised tile, then the 3-register update
-//   s0: acc = y + dt/6 k, Y1 = y + dt/2 k      s1: acc += dt/3 k, Y2 = y + dt/2 k
-//   s2: acc += dt/3 k,    Y3 = y + dt k        s3: y = acc + dt/6 k
-// Advection RHS: -(u Dx phi + v Dy phi),
-//   D1 f = ((f[-2] - f[2]) + 8 (f[1] - f[-1])) / (12 dx).
-// 2D blocks; the 3D stage is k_stage3 (mr_adv3.cuh).
-//
-// The block's plan (k_plan) is read from shared memory, the next block's plan
-// is fetched while this one is processed; blocks with a uniform neighbourhood
-// take the direct gather, the others the general one through their ring.
-template <int B, int RHS, typename TS, typename TY, typename TSRC, int NT, int ST>
-__global__ void __launch_bounds__(NT, NT <= 128 ? 8 : 4) k_stage_adv(PoolView pv, const TSRC* __restrict__ src, TS* __restrict__ y,
-                            TS* __restrict__ acc, TY* __restrict__ ynext, int stage_arg, StageArgs sa) {
-  pdl_enter();
-  constexpr int stage = ST;  // the RK stage, fixed at compile time
-  static_assert(ST >= 0 && ST <= 3, "RK4 stage");
-  constexpr int D = 2;
-  using Bx = Box<D, B, 2>;  // the stencils reach two nodes
-  using PL = Plan<D>;
-  using TC = TY;  // stencil arithmetic type
-  static_assert(NT >= PL::INTS, "one thread per plan entry");
-  RingD<D>& R = *smem_as<RingD<D>>(0);
-  TC* tile = smem_as<TC>(kRingBytesD<D>);  // nvar == 1
-  TC* cbox = tile + Bx::TILE;
-  TC* scr = cbox + Bx::CBOX;
-  int32_t* gtab = reinterpret_cast<int32_t*>(scr + Bx::SCR);  // gather table
-  __shared__ int32_t splan[2][PL::INTS];
-  __shared__ int64_t snb[2][PL::NB];  // pool offsets of the plan's neighbours
-  const int nact = pv.cnt->n_act;
-  if (blockIdx.x >= nact) return;  // no block for this CTA (small grids)
-  if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&pv.cnt->stage_blocks, (unsigned long long)nact);
-  build_gtab<D, B, 2>(gtab);
-  if (blockIdx.x < nact && threadIdx.x < PL::INTS) {
-    const int32_t v = pv.plan[(int64_t)blockIdx.x * PL::INTS + threadIdx.x];
-    splan[0][threadIdx.x] = v;
-    if (threadIdx.x >= PL::NBO && threadIdx.x < PL::NBO + PL::NB) snb[0][threadIdx.x - PL::NBO] = (int64_t)v * pv.vs;
-  }
-  __syncthreads();
-  int buf = 0;
-  for (int p = blockIdx.x; p < nact; p += gridDim.x, buf ^= 1) {
-    const int pn = p + gridDim.x;
-    int32_t pre = 0;
-    if (pn < nact && threadIdx.x < PL::INTS) pre = pv.plan[(int64_t)pn * PL::INTS + threadIdx.x];
-    const int32_t* pl = splan[buf];
-    const BlockInfo b = plan_block<D>(pl);
-    const TreeDev& td = pv.trees[b.tree];
-    if ((pl[1] >> 30) & 1) {
-      gather_table<D, B, 2, 1, TSRC, TC>(pv, (int64_t)b.slot * pv.vs, snb[buf], gtab, src, (TSRC*)src, tile,
-                                         stage == 0);
-    } else {
-      load_regions<D, CtaGroup>(pv, p, R);
-      __syncthreads();
-      fill_tile<D, B, TSRC, TC, 2>(pv, b, src, (TSRC*)src, tile, stage == 0, R, cbox, scr, true);
-    }
-    __syncthreads();
-    const TC c = tree_cD<TC>(td, b.lvl);
-    const StageCoef<TS> cs(pv, sa, b.tree, stage);  // RK weights in the state type
-    const TC ct = StageCoef<TC>(pv, sa, b.tree, stage).ct;
-    const int64_t base = (int64_t)b.slot * pv.vs;  // nvar == 1
-    const int sh = td.Jmax - b.lvl;
-    const TS cas = cs.ca, cys = cs.cy;
-    {
-      // thread = (column i, rows j0, j0 + G, ...): the column's velocity
-      // factors are loaded once; the rows' loads are issued together
-      constexpr int G = NT / B, RU = (B + G - 1) / G;
-      const int t = threadIdx.x;
-      if (t < G * B) {
-        const int i = t % B, j0 = t / B;
-        TC ax = 0, bx = 0;  // swirl factors in the stencil type
-        const TC* A = lattice<TC>(pv) + td.lat_off + (int64_t)kLatSwA * td.N;
-        const TC* Bt = lattice<TC>(pv) + td.lat_off + (int64_t)kLatSwB * td.N;
-        if (RHS == MR_RHS_SWIRL) {
-          const int64_t Ux = pmod64((b.c[0] * (B - 1) + i) << sh, td.N);
-          ax = A[Ux];
-          bx = Bt[Ux];
-        }
-        TS yv[RU], av[RU];
-        TC u0[RU], u1[RU];  // velocity in the stencil type (constant: once per block)
-        const TC uc0 = tree_rhs<TC>(td, 0), uc1 = tree_rhs<TC>(td, 1);
-#pragma unroll
-        for (int r = 0; r < RU; ++r) {
-          const int j = j0 + r * G;
-          yv[r] = av[r] = TS(0);
-          u0[r] = uc0;
-          u1[r] = uc1;
-          if (j >= B) continue;
-          const int q = j * B + i;
-          if (stage <= 2) yv[r] = y[base + q];  // stage 0: committed (synchronised) y_n
-          if (stage >= 1) av[r] = acc[base + q];
-          if (RHS == MR_RHS_SWIRL) {
-            const int64_t Uy = pmod64((b.c[1] * (B - 1) + j) << sh, td.N);
-            u0[r] = ct * (ax * Bt[Uy]);
-            u1[r] = -(ct * (A[Uy] * bx));
-          }
-        }
-#pragma unroll
-        for (int r = 0; r < RU; ++r) {
-          const int j = j0 + r * G;
-          if (j >= B) continue;
-          const TC* t0 = tile + Bx::tix(i, j, 0);
-          const TC dxv = ((t0[-2] - t0[2]) + TC(8) * (t0[1] - t0[-1])) * c;
-          const TC dyv = ((t0[-2 * Bx::S] - t0[2 * Bx::S]) + TC(8) * (t0[Bx::S] - t0[-Bx::S])) * c;
-          const TC s = u0[r] * dxv + u1[r] * dyv;
-          const TS kk = (TS)(-s);
-          const int64_t at = base + j * B + i;
-          if (stage == 0) {
-            acc[at] = yv[r] + cas * kk;
-            ynext[at] = (TY)(yv[r] + cys * kk);
-          } else if (stage == 1 || stage == 2) {
-            acc[at] = av[r] + cas * kk;
-            ynext[at] = (TY)(yv[r] + cys * kk);
-          } else {
-            y[at] = av[r] + cas * kk;
-          }
-        }
-      }
-    }
-    if (pn < nact && threadIdx.x < PL::INTS) {
-      splan[buf ^ 1][threadIdx.x] = pre;
-      if (threadIdx.x >= PL::NBO && threadIdx.x < PL::NBO + PL::NB) snb[buf ^ 1][threadIdx.x - PL::NBO] = (int64_t)pre * pv.vs;
-    }
-    __syncthreads();
-  }
-}
-
-// 2D form of k_stage_adv with one warp per block: each warp of the CTA walks
-// its own sequence of blocks (gather, stencils, update) with warp-level
-// synchronisation only, so the per-block work (plan, coefficients, barriers)
-// is done by 32 threads instead of a whole CTA.  Same values as k_stage_adv.
-template <int B, int RHS, typename TS, typename TY, typename TSRC, int NT>
-struct StageW {
-  using Bx = Box<2, B, 2>;
-  static constexpr int NW = NT / 32;
-  // FP32 state: the block's state and accumulator rows are staged in shared
-  // memory by the bulk-copy (TMA) engine, one mbarrier per warp
-  static constexpr bool TMA = sizeof(TS) == 4;
-  static constexpr int VS = (B * B + 3) / 4 * 4;  // padded block: the pool's per-variable stride
-  // per warp: mbarrier; a region holding either the ring and the coarse-box
-  // scratch of a block whose neighbourhood is not uniform, or the staged rows;
-  // the tile
-  static constexpr size_t BAR = TMA ? 16 : 0;
-  static constexpr size_t RINGSCR = kRingBytesD<2> + sizeof(TY) * (Bx::CBOX + Bx::SCR);
-  static constexpr size_t ROWS = TMA ? 2 * sizeof(TS) * VS : 0;
-  static constexpr size_t UNION = ((RINGSCR > ROWS ? RINGSCR : ROWS) + 15) / 16 * 16;
-  static constexpr size_t GTAB = (4 * Bx::NPTS + 15) / 16 * 16;
-  static constexpr size_t WAREA = (BAR + UNION + sizeof(TY) * Bx::TILE + 15) / 16 * 16;
-  static constexpr size_t SMEM = GTAB + NW * WAREA;
-};
-
-// ST: the RK stage, fixed at compile time (the per-point loads, stores and
-// updates of each stage without run-time branches).
-template <int B, int RHS, typename TS, typename TY, typename TSRC, int NT, int ST>
-__global__ void __launch_bounds__(NT, 1024 / NT) k_stage_adv_w(PoolView pv, const TSRC* __restrict__ src, TS* __restrict__ y,
-                                                   TS* __restrict__ acc, TY* __restrict__ ynext, int staging,
-                                                   StageArgs sa) {
-  pdl_enter();
-  constexpr int stage = ST;
-  static_assert(ST >= 0 && ST <= 3, "RK4 stage");
-  using Gm = Geo<2, B>;
-  using Bx = Box<2, B, 2>;
-  using PL = Plan<2>;
-  using SW = StageW<B, RHS, TS, TY, TSRC, NT>;
-  using TC = TY;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned char* sm = smem_as<unsigned char>(0);
-  int32_t* gtab = reinterpret_cast<int32_t*>(sm);
-  unsigned char* wa = sm + SW::GTAB + warp * SW::WAREA;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(wa);
-  unsigned char* un = wa + SW::BAR;  // ring + coarse-box scratch, or the staged rows
-  RingD<2>& R = *reinterpret_cast<RingD<2>*>(un);
-  TC* cbox = reinterpret_cast<TC*>(un + kRingBytesD<2>);
-  TC* scr = cbox + Bx::CBOX;
-  TS* ys = reinterpret_cast<TS*>(un);
-  TS* as = ys + SW::VS;
-  TC* tile = reinterpret_cast<TC*>(un + SW::UNION);
-  __shared__ int64_t snb[SW::NW][PL::NB];
-  const int nact = pv.cnt->n_act;
-  if ((int)blockIdx.x * SW::NW >= nact) return;  // no block for this CTA
-  build_gtab<2, B, 2>(gtab);
-  if (SW::TMA && lane == 0) mbar_init(bar, 1);
-  __syncthreads();
-  unsigned phase = 0;
-  if (blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(&pv.cnt->stage_blocks, (unsigned long long)nact);
-  const int gw = blockIdx.x * SW::NW + warp, nwt = gridDim.x * SW::NW;
-  int32_t cur = (gw < nact && lane < PL::INTS) ? pv.plan[(int64_t)gw * PL::INTS + lane] : 0;
-  for (int p = gw; p < nact; p += nwt) {
-    const int pn = p + nwt;
-    const int32_t nxt = (pn < nact && lane < PL::INTS) ? pv.plan[(int64_t)pn * PL::INTS + lane] : 0;
-    BlockInfo b;
-    b.slot = __shfl_sync(0xffffffffu, cur, 0);
-    const int meta = __shfl_sync(0xffffffffu, cur, 1);
-    b.lvl = meta & 255;
-    b.tree = (meta >> 8) & 0xffff;
-    b.c[0] = __shfl_sync(0xffffffffu, cur, 2);
-    b.c[1] = __shfl_sync(0xffffffffu, cur, 3);
-    b.c[2] = 0;
-    const TreeDev& td = pv.trees[b.tree];
-    // stage 0 reads the state from the tile; the other stages stage the rows
-    // (FP32, unless switched off) or load them
-    const bool staged = SW::TMA && stage >= 1 && staging != 0;
-    const bool uni = (meta >> 30) & 1;
-    auto stage_rows = [&]() {
-      if (lane == 0) {
-        constexpr unsigned rows = (stage <= 2 ? 2 : 1) * sizeof(TS) * SW::VS;
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        mbar_expect_tx(bar, rows);
-        if (stage <= 2) bulk_g2s(ys, y + (int64_t)b.slot * pv.vs, sizeof(TS) * SW::VS, bar);
-        bulk_g2s(as, acc + (int64_t)b.slot * pv.vs, sizeof(TS) * SW::VS, bar);
-      }
-    };
-    // uniform neighbourhood: the rows travel while the ghost layer is
-    // gathered; otherwise the gather needs the shared region first
-    if (staged && uni) stage_rows();
-    if (uni) {
-      if (lane >= PL::NBO && lane < PL::NBO + PL::NB) snb[warp][lane - PL::NBO] = (int64_t)cur * pv.vs;
-      __syncwarp();
-      gather_table<2, B, 2, 1, TSRC, TC, WarpGroup>(pv, (int64_t)b.slot * pv.vs, snb[warp], gtab, src, (TSRC*)src,
-                                                    tile, stage == 0);
-    } else {
-      load_regions<2, WarpGroup>(pv, p, R);
-      __syncwarp();
-      fill_tile<2, B, TSRC, TC, 2, WarpGroup>(pv, b, src, (TSRC*)src, tile, stage == 0, R, cbox, scr, true);
-    }
-    __syncwarp();
-    if (staged && !uni) stage_rows();
-    if (staged) {
-      // bounded wait: a copy that never lands is reported, not waited for
-      if (!mbar_wait(bar, phase, 1 << 20)) {
-        if (lane == 0) set_err(pv, kErrTimeout);
-        return;
-      }
-      phase ^= 1;
-    }
-    const TC c = tree_cD<TC>(td, b.lvl);
-    const StageCoef<TS> cs(pv, sa, b.tree, stage);
-    const TC ct = StageCoef<TC>(pv, sa, b.tree, stage).ct;
-    const TS cas = cs.ca, cys = cs.cy;
-    const int64_t base = (int64_t)b.slot * pv.vs;
-    const int sh = td.Jmax - b.lvl;
-    const TC uc0 = tree_rhs<TC>(td, 0), uc1 = tree_rhs<TC>(td, 1);
-    // points q0 + 32 u, u < UC: state, accumulator and velocity loads first,
-    // then the stencils and the updates
-    auto chunk = [&](auto ucc, int q0) {
-      constexpr int UC = decltype(ucc)::value;
-      TS yv[UC], av[UC];
-      TC u0[UC], u1[UC];
-#pragma unroll
-      for (int u = 0; u < UC; ++u) {
-        const int q = q0 + u * 32;
-        yv[u] = av[u] = TS(0);
-        u0[u] = uc0;
-        u1[u] = uc1;
-        if (q >= Gm::NI) continue;
-        if constexpr (SW::TMA) {
-          // stage 0: the committed (synchronised) y_n is the tile's value
-          if (stage == 0) yv[u] = (TS)tile[Bx::tix(q % B, q / B, 0)];
-          if (stage == 1 || stage == 2) yv[u] = staged ? ys[q] : y[base + q];
-          if (stage >= 1) av[u] = staged ? as[q] : acc[base + q];
-        } else {
-          if (stage <= 2) yv[u] = y[base + q];  // stage 0: committed (synchronised) y_n
-          if (stage >= 1) av[u] = acc[base + q];
-        }
-        if (RHS == MR_RHS_SWIRL) {
-          const int i = q % B, j = q / B;
-          const int64_t Ux = pmod64((b.c[0] * (B - 1) + i) << sh, td.N);
-          const int64_t Uy = pmod64((b.c[1] * (B - 1) + j) << sh, td.N);
-          const TC* A = lattice<TC>(pv) + td.lat_off + (int64_t)kLatSwA * td.N;
-          const TC* Bt = lattice<TC>(pv) + td.lat_off + (int64_t)kLatSwB * td.N;
-          u0[u] = ct * (A[Ux] * Bt[Uy]);
-          u1[u] = -(ct * (A[Uy] * Bt[Ux]));
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < UC; ++u) {
-        const int q = q0 + u * 32;
-        if (q >= Gm::NI) continue;
-        const int i = q % B, j = q / B;
-        const TC* t0 = tile + Bx::tix(i, j, 0);
-        const TC dxv = ((t0[-2] - t0[2]) + TC(8) * (t0[1] - t0[-1])) * c;
-        const TC dyv = ((t0[-2 * Bx::S] - t0[2 * Bx::S]) + TC(8) * (t0[Bx::S] - t0[-Bx::S])) * c;
-        const TC s = u0[u] * dxv + u1[u] * dyv;
-        const TS kk = (TS)(-s);
-        const int64_t at = base + q;
-        if (stage == 0) {
-          acc[at] = yv[u] + cas * kk;
-          ynext[at] = (TY)(yv[u] + cys * kk);
-        } else if (stage == 1 || stage == 2) {
-          acc[at] = av[u] + cas * kk;
-          ynext[at] = (TY)(yv[u] + cys * kk);
-        } else {
-          y[at] = av[u] + cas * kk;
-        }
-      }
-    };
-    // full chunks of 4 points per lane, then one chunk for the remainder
-    constexpr int UC = 4, FULL = Gm::NI / (UC * 32) * (UC * 32), UT = (Gm::NI - FULL + 31) / 32;
-    for (int q0 = lane; q0 < FULL; q0 += UC * 32) chunk(std::integral_constant<int, UC>{}, q0);
-    if constexpr (UT > 0) chunk(std::integral_constant<int, UT>{}, FULL + lane);
-    __syncwarp();
-    cur = nxt;
-  }
-}
-
+// ------------------------------------------------------------- stage plans ----
 // Stage plans of all active blocks, one warp per block (layout in Plan<D>):
 // the 3^d - 1 equal-level neighbours, one lookup per lane in the dense leaf
 // tables; for a block whose neighbourhood is not uniform, also its ring and

@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <cstdio>
 
+#include "mr_adv2.cuh"
 #include "mr_adv3.cuh"
 #include "mr_det2.cuh"
 #include "mr_kernels.cuh"
@@ -37,60 +38,51 @@ static inline int flat_grid(const PoolView& pv, int threads) {
 constexpr int64_t kFusedScanMax = 65536;
 
 // ---------------------------------------------------------------- stage ------
-// 2D blocks of 17^2 nodes: 128-thread CTAs, so small grids run in one wave.
+// One CTA per block: about half the block's nodes (17^2) or a quarter (33^2) per
+// pass.  Measured per step of four launches, 4096 blocks of 33^2: 288 threads 72 us
+// (FP32), 564 (FP64); 384 82 and 593; 256 70 and 572.  Small grids, where a launch
+// is one wave, do not depend on it (76 blocks of 17^2 FP64: 33 us with 160 to 256).
 template <int B>
-struct Threads { static constexpr int value = B == 17 ? 128 : 256; };
+struct Threads { static constexpr int value = B == 17 ? 160 : 288; };
 
 template <int B, int RHS, typename TS, typename TY>
 static void stage_impl(const PoolView& pv, const Fields& f, int stage, const StageArgs& sa,
                        const LaunchCfg& lc, cudaStream_t st) {
-  constexpr int threads = Threads<B>::value;
-  using Bx = Box<2, B, 2>;
-  const size_t smem = kRingBytesD<2> + sizeof(TY) * (Bx::TILE + Bx::CBOX + Bx::SCR) + 4 * Bx::NPTS;
   TY* ynext = (TY*)(stage == 1 ? f.Yb : f.Ya);
-  // one warp per block when the grid holds enough blocks to fill the GPU
-  // several times over (or as tuned), else one CTA per block (shorter latency)
-  const bool warp_form = lc.stage_form == 1 || (lc.stage_form < 0 && lc.n_hint >= 8 * lc.num_sms);
-  if constexpr (B == 17) {  // 17^2 blocks: 289 points per warp
-    if (warp_form) {
-      // one instantiation per stage: stage 0 reads the committed state, the
-      // others the previous stage value
-      auto go_nt = [&](auto stc, auto ntc) {
-        constexpr int S = decltype(stc)::value, NT = decltype(ntc)::value;
-        using TSRC = std::conditional_t<S == 0, TS, TY>;
-        using SW = StageW<B, RHS, TS, TY, TSRC, NT>;
-        const TSRC* src = S == 0 ? (const TSRC*)f.y : (const TSRC*)(S == 2 ? f.Yb : f.Ya);
-        auto k = k_stage_adv_w<B, RHS, TS, TY, TSRC, NT, S>;
-        prep_smem(k, SW::SMEM);
-        const int grid = persistent_grid(k, NT, SW::SMEM, lc, lc.grid_mult);
-        launch_k(lc.pdl, k, grid, NT, SW::SMEM, st, pv, src, (TS*)f.y, (TS*)f.acc, ynext, lc.staging, sa);
-      };
-      // blocks (warps) per CTA: tuned for the FP32 forms, 4 otherwise
-      auto go = [&](auto stc) {
-        if constexpr (sizeof(TS) == 4) {
-          if (lc.warp_blocks == 2) return go_nt(stc, std::integral_constant<int, 64>{});
-          if (lc.warp_blocks == 8) return go_nt(stc, std::integral_constant<int, 256>{});
-        }
-        go_nt(stc, std::integral_constant<int, threads>{});
-      };
-      switch (stage) {
-        case 0: go(std::integral_constant<int, 0>{}); break;
-        case 1: go(std::integral_constant<int, 1>{}); break;
-        case 2: go(std::integral_constant<int, 2>{}); break;
-        default: go(std::integral_constant<int, 3>{}); break;
-      }
-      count_launch();
-      return;
-    }
-  }
-  auto go = [&](auto stc) {
-    constexpr int S = decltype(stc)::value;
+  // One warp per block when the grid holds enough blocks to fill the GPU several
+  // times over (or as tuned), else one CTA per block (shorter latency).  n_hint
+  // counts the blocks before the refinement of the step.  Measured per launch, CTA
+  // against warp: FP32 state 256 blocks 4.9 / 6.5 us, 1024 6.9 / 6.8, 4096 10.2 /
+  // 8.9, 65536 105 / 62; FP64 state, bound by the FP64 pipe in either form, 1024
+  // 15.0 / 21.8, 4096 44.3 / 48.3, 16384 161 / 158, 65536 627 / 598.
+  constexpr int kWarpFrom = sizeof(TS) == 4 ? 8 : 32;  // blocks per SM
+  const bool warp_form =
+      B == 17 && (lc.stage_form == 1 || (lc.stage_form < 0 && lc.n_hint >= kWarpFrom * lc.num_sms));
+  // one instantiation per stage: stage 0 reads the committed state, the others
+  // the previous stage value
+  auto run = [&](auto stc, auto gtc, auto nwc) {
+    constexpr int S = decltype(stc)::value, GT = decltype(gtc)::value, NW = decltype(nwc)::value;
     using TSRC = std::conditional_t<S == 0, TS, TY>;
+    using SM = Stage2<B, TS, TY, GT, NW, S>;
     const TSRC* src = S == 0 ? (const TSRC*)f.y : (const TSRC*)(S == 2 ? f.Yb : f.Ya);
-    auto k = k_stage_adv<B, RHS, TS, TY, TSRC, threads, S>;
-    prep_smem(k, smem);
-    const int grid = persistent_grid(k, threads, smem, lc, lc.grid_mult);
-    launch_k(lc.pdl, k, grid, threads, smem, st, pv, src, (TS*)f.y, (TS*)f.acc, ynext, stage, sa);
+    auto k = k_stage2<B, RHS, TS, TY, TSRC, GT, NW, S>;
+    prep_smem(k, SM::BYTES);
+    launch_k(lc.pdl, k, persistent_grid(k, GT * NW, SM::BYTES, lc, lc.grid_mult), GT * NW, SM::BYTES, st, pv, src,
+             (TS*)f.y, (TS*)f.acc, ynext, lc.staging, sa);
+  };
+  auto go = [&](auto stc) {
+    using C32 = std::integral_constant<int, 32>;
+    if constexpr (B == 17) {
+      if (warp_form) {
+        // blocks (warps) per CTA: tuned for the FP32 forms, 4 otherwise
+        if constexpr (sizeof(TS) == 4) {
+          if (lc.warp_blocks == 2) return run(stc, C32{}, std::integral_constant<int, 2>{});
+          if (lc.warp_blocks == 8) return run(stc, C32{}, std::integral_constant<int, 8>{});
+        }
+        return run(stc, C32{}, std::integral_constant<int, 4>{});
+      }
+    }
+    run(stc, std::integral_constant<int, Threads<B>::value>{}, std::integral_constant<int, 1>{});
   };
   switch (stage) {
     case 0: go(std::integral_constant<int, 0>{}); break;

@@ -272,11 +272,12 @@ __global__ void __launch_bounds__(NsCfg<B, TY>::NT, NsCfg<B, TY>::MINB) k_stage_
     const StageCoef<TS> cs(pv, sa, b.tree, stage);  // RK weights in the state type
     const StageCoef<TC> cf(pv, sa, b.tree, stage);  // and in the stage type
     const int64_t base = (int64_t)b.slot * 4 * pv.vs;
+    const TS* yc = stage == 0 ? committed(y, src) : y;
     for (int q = threadIdx.x; q < NI; q += blockDim.x) {
       const int i = q % B, j = q / B;
       NsUpdate<TS, TC> up[4];
 #pragma unroll
-      for (int v = 0; v < 4; ++v) up[v].load(y, acc, yn, base + v * pv.vs + q, stage);
+      for (int v = 0; v < 4; ++v) up[v].load(yc, acc, yn, base + v * pv.vs + q, stage);
       const TC* f0 = F + fI(i, j);
       const TC* g0 = Gf + gI(i, j);
       const Vec4<TC> fa = ld4(f0 - 8), fb = ld4(f0 - 4), fc = ld4(f0 + 4), fd = ld4(f0 + 8);
@@ -419,12 +420,13 @@ __global__ void __launch_bounds__(NssCfg<B, TY>::NT, NssCfg<B, TY>::MINB) k_stag
     const StageCoef<TS> cs(pv, sa, b.tree, stage);
     const StageCoef<TC> cf(pv, sa, b.tree, stage);
     const int64_t base = (int64_t)b.slot * 4 * pv.vs;
+    const TS* yc = stage == 0 ? committed(y, src) : y;
     for (int q = threadIdx.x; q < NI; q += blockDim.x) {
       const int i = q % B, j = q / B;
       const int o = I(i, j);
       NsUpdate<TS, TC> up[4];
 #pragma unroll
-      for (int v = 0; v < 4; ++v) up[v].load(y, acc, yn, base + v * pv.vs + q, stage);
+      for (int v = 0; v < 4; ++v) up[v].load(yc, acc, yn, base + v * pv.vs + q, stage);
       const Vec2<TC> w0 = ld2(uv + 2 * o);
       const Vec4<TC> s0 = ld4(tile + 4 * o);
       const TC uu = w0.a, vv = w0.b, f = s0.a;
