@@ -67,3 +67,21 @@ def test_certified_decisions(mr, oracle_mod, Bs, name):  # noqa: F811
     o.flags(0)
     g.adapt("flags_only")
     assert np.array_equal(g.get_flags()[0], o.blocks()["flag"])
+
+
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** -1020, 2.0 ** -1060, 2.0 ** 1000])
+def test_prediction_at_the_ends_of_fp64(mr, oracle_mod, scale):  # noqa: F811
+    # the prediction's division by 16 next to and below the smallest normal number
+    lvl, crd = treegen.as_arrays(TREES["random"]())
+    f = np.random.default_rng(8).standard_normal((len(lvl), 1, 17, 17)) * scale
+    o, g = make_pair(mr, oracle_mod, config(17, 1, 1.0))
+    o.set_blocks(lvl, crd, f)
+    g.set_blocks(lvl, crd, f)
+    o.details()  # synchronises the redundant copies, as the library's details do
+    o.flags(0)
+    g.adapt("flags_only")
+    assert np.array_equal(g.get_flags()[1], o.blocks()["mdet"])
+    o.refine(0)
+    g.adapt("refine_all")
+    ob, gfl = assert_same_tree(o, g)
+    assert np.array_equal(gfl, ob["fields"])
