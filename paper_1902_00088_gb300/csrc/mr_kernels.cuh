@@ -57,6 +57,9 @@ __global__ void __launch_bounds__(128) k_plan(PoolView pv) {
   constexpr int NW = 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   RingD<D>& R = *smem_as<RingD<D>>((size_t)warp * kRingBytesD<D>);
+  // The plans of this tree stand (a step on a grid that did not change): nothing to do.
+  // plan_topo changes only after the last CTA has read it.  65536 blocks: 22 -> 4 us.
+  if (pv.cnt->plan_topo == pv.cnt->topo) return;
   const int nact = pv.cnt->n_act;
   for (int p = blockIdx.x * NW + warp; p < nact; p += gridDim.x * NW) {
     const int s = pv.act[p];
@@ -90,7 +93,14 @@ __global__ void __launch_bounds__(128) k_plan(PoolView pv) {
       __syncwarp();
     }
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) pv.cnt->plan_topo = pv.cnt->topo;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    if (atomicAdd(&pv.cnt->ctas_done, 1u) == gridDim.x - 1) {
+      pv.cnt->ctas_done = 0;
+      pv.cnt->plan_topo = pv.cnt->topo;
+    }
+  }
 }
 
 // Start of a coarsening round: the blocks it works on (none once a round

@@ -112,6 +112,31 @@ __global__ void __launch_bounds__(kSingleThreads) k_scan_single(const int32_t* i
   __shared__ int2 wt[kSingleThreads / 32];
   const int64_t n = scan_n(n_dev, n_host, shift);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  if (n_dev && n > kSingleThreads) {
+    // Totals first, every load in flight at once: a list whose blocks all stay (one
+    // entry each, no slot requested or freed) is left as it is and needs no offsets.
+    // 65536 blocks: 14 -> 7 us.
+    const int2* v = reinterpret_cast<const int2*>(in);
+    int2 s = make_int2(0, 0);
+#pragma unroll 8
+    for (int64_t i = threadIdx.x; i < n; i += kSingleThreads) {
+      const int2 e = v[i];
+      s.x += e.x;
+      s.y |= e.y;
+    }
+    s.x = (int)__reduce_add_sync(0xffffffffu, (unsigned)s.x);
+    s.y = (int)__reduce_or_sync(0xffffffffu, (unsigned)s.y);
+    if (lane == 0) wt[w] = s;
+    __syncthreads();
+    s = wt[lane];
+    s.x = (int)__reduce_add_sync(0xffffffffu, (unsigned)s.x);
+    s.y = (int)__reduce_or_sync(0xffffffffu, (unsigned)s.y);
+    if (s.y == 0 && s.x == *n_dev) {
+      if (threadIdx.x == 0 && tot) { tot[0] = s.x; tot[1] = 0; }
+      return;
+    }
+    __syncthreads();
+  }
   int2 carry = make_int2(0, 0);
   for (int64_t base = 0; base < n; base += (int64_t)kSingleThreads * kSinglePer) {
     int2 loc[kSinglePer];

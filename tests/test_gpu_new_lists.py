@@ -74,3 +74,39 @@ def test_lists_beyond_one_scan(mr):  # noqa: F811
     back, f = g.get_blocks()
     assert np.array_equal(back["level"], coarse["level"]) and np.array_equal(back["coords"], coarse["coords"])
     assert (f == 1.0).all()
+
+
+@pytest.mark.parametrize("dim,Bs", [(2, 17), (2, 33), (3, 17)])
+def test_plans_stand_while_the_tree_does(mr, oracle_mod, dim, Bs):  # noqa: F811
+    # eps = 0: no family merges and the finest level cannot refine, so the stage plans
+    # of the first step serve the next ones; then another tree takes their place, twice
+    c = cfg2d(dim=dim, Bs=Bs, Jmin=1, Jmax=2, eps=0.0, ic="none", rhs_params=(0.9, -0.7, 0.4))
+    o = oracle_mod.Oracle(c)
+    g = mr.Forest(dim=dim, Bs=Bs, precision="fp64", rhs="adv", capacity=512,
+                  trees=[{q: c[q] for q in ("Jmin", "Jmax", "eps", "ic", "rhs_params")}])
+    dt = 0.1 / ((Bs - 1) * 4)
+    uniform = sorted(treegen.uniform_tree(dim, 2))
+    for k, leaves in enumerate((uniform, treegen.random_graded_tree(dim, 1, 2, 1, 3), uniform)):
+        lvl, crd = treegen.as_arrays(leaves)
+        f = np.random.default_rng(20 + k).standard_normal((len(lvl), 1) + (Bs,) * dim)
+        o.set_blocks(lvl, crd, f)
+        g.set_blocks(lvl, crd, f)
+        for s in range(2):
+            o.step(s * dt, dt)
+            g.step(s * dt, dt)
+            ob = o.blocks()
+            info, got = g.get_blocks()
+            assert np.array_equal(info["coords"].astype(np.int64), ob["coords"])
+            assert np.array_equal(got, ob["fields"])
+
+
+def test_long_list_without_changes(mr):  # noqa: F811
+    # 65536 blocks: the scan finds that every block stays and writes no offsets
+    g = mr.Forest(dim=2, precision="fp32", capacity=66_000, trees=[dict(Jmin=8, Jmax=8, eps=1e-3, ic="none")])
+    lvl, crd = treegen.as_arrays(sorted(treegen.uniform_tree(2, 8)))
+    g.set_blocks(lvl, crd, np.ones((len(lvl), 1, 17, 17)))
+    before, _ = g.get_blocks(fields=False)
+    for s in range(2):
+        g.step(0.0, 1e-5)
+    after, f = g.get_blocks()
+    assert np.array_equal(before["hilbert_key"], after["hilbert_key"]) and (f == 1.0).all()
