@@ -537,10 +537,12 @@ __global__ void __launch_bounds__(Stage3Smem<TY, TS>::NT, 2) k_stage3(PoolView p
 // nothing is predicted.  The x pass goes to shared memory (11 x 11 rows), the y
 // pass of a column is kept in its thread's registers and feeds the z pass, and
 // the block's own values go from memory straight to registers.  Per-block latency
-// bounds it (five barriers per block, 3 CTAs per SM).  Measured, before with a
-// gathered 21^3 tile and its predicted ghosts: 2078 -> 466 us on a uniform grid of
-// 32768 blocks (FP32); the four rounds of an adaptive FP32 step with 2736 blocks
-// evaluated 426 -> 134 us, the three of an FP64 step with 4119 blocks 1750 -> 677 us.
+// bounds it (four barriers per block, 3 CTAs per SM; 4 CTAs spill: 487 us instead of
+// 460, with three more barriers).  Measured, before with a gathered 21^3 tile and its
+// predicted ghosts: 2078 -> 400 us on a uniform grid of 32768 blocks (FP32); the three
+// rounds of an adaptive FP32 step with 1632 blocks 426 -> 120 us; of an FP64 step with
+// 2584 blocks 1750 -> 470 us, where maxima, the non-finite test and the division by 16
+// are kept off the FP64 pipe.
 template <typename TT, typename TD>
 struct Det3Smem {
   static constexpr int CN = 11;
@@ -566,7 +568,7 @@ __global__ void __launch_bounds__(Col3::NT, sizeof(TS) == 8 ? 2 : 3) k_details3(
   __shared__ double red[2][32];
   __shared__ int32_t splan[2][PL::INTS];
   __shared__ int32_t snb[PL::NB];
-  __shared__ int dirty;
+  __shared__ int nonfinite;
   __shared__ double csv;
   __shared__ int csv_tree;
   const int t = threadIdx.x;
@@ -609,6 +611,7 @@ __global__ void __launch_bounds__(Col3::NT, sizeof(TS) == 8 ? 2 : 3) k_details3(
   if (t == 0) {
     csv = 0.0;
     csv_tree = -1;
+    nonfinite = 0;
   }
   auto flush_csv = [&]() {
     if (csv_tree >= 0 && t == 0 && csv > 0.0) atomic_max_pos(&pv.svar[csv_tree], csv);
@@ -647,20 +650,29 @@ __global__ void __launch_bounds__(Col3::NT, sizeof(TS) == 8 ? 2 : 3) k_details3(
         csv_tree = b.tree;
       }
     }
-    if (t < PL::NB) snb[t] = q;
-    if (t == 0) dirty = all_blocks ? 1 : 0;
-    const bool uni = __syncthreads_and(q >= 0);
-    if (uni) {
-      if (!all_blocks && t < PL::NB && pv.stamp[q] == prev) dirty = 1;
-    } else if (plan_ok && all_blocks) {
-      const int4* rsrc = plan_regions<3>(pv, p);
-      for (int r = t; r < Col3::NREG; r += NT) R.reg[r] = rsrc[r];
+    // With a plan and every block due (the first round of a step) a block with a
+    // uniform neighbourhood gathers without a barrier.
+    bool uni;
+    if (plan_ok) {
+      uni = (splan[buf][1] >> 30) & 1;
     } else {
-      build_ring<3, B>(pv, td, b, R);
-      __syncthreads();
-      if (!all_blocks && t < Geo<3, B>::NR && R.slot[t] >= 0 && pv.stamp[R.slot[t]] == prev) dirty = 1;
+      if (t < PL::NB) snb[t] = q;
+      uni = __syncthreads_and(q >= 0);
     }
-    __syncthreads();
+    const int32_t* nbs = plan_ok ? splan[buf] + PL::NBO : snb;  // slots of the 3^3 blocks
+    if (!uni) {
+      if (plan_ok && all_blocks) {
+        const int4* rsrc = plan_regions<3>(pv, p);
+        for (int r = t; r < Col3::NREG; r += NT) R.reg[r] = rsrc[r];
+      } else {
+        build_ring<3, B>(pv, td, b, R);
+      }
+      __syncthreads();
+    }
+    bool dirty = all_blocks;
+    if (!all_blocks)
+      dirty = __syncthreads_or(uni ? t < PL::NB && pv.stamp[q] == prev
+                                   : t < Geo<3, B>::NR && R.slot[t] >= 0 && pv.stamp[R.slot[t]] == prev);
     if (!dirty) {
       // no leaf of the ring changed in the previous round: the stored details
       // and norms are those of the unchanged tile
@@ -678,8 +690,8 @@ __global__ void __launch_bounds__(Col3::NT, sizeof(TS) == 8 ? 2 : 3) k_details3(
       if (col) {
         const int sx = x == B - 1 ? 2 : 1, sy = yy == B - 1 ? 2 : 1;
         const int lxy = (x - (sx - 1) * (B - 1)) + B * (yy - (sy - 1) * (B - 1));
-        const TS* mid = y + (int64_t)snb[sx + 3 * sy + 9] * pv.vs + lxy;
-        const TS* top = y + (int64_t)snb[sx + 3 * sy + 18] * pv.vs + lxy;
+        const TS* mid = y + (int64_t)nbs[sx + 3 * sy + 9] * pv.vs + lxy;
+        const TS* top = y + (int64_t)nbs[sx + 3 * sy + 18] * pv.vs + lxy;
         TS raw[B];
 #pragma unroll
         for (int k = 0; k < B; ++k) raw[k] = k < B - 1 ? mid[NQ * k] : *top;
@@ -691,7 +703,7 @@ __global__ void __launch_bounds__(Col3::NT, sizeof(TS) == 8 ? 2 : 3) k_details3(
       }
       for (int g = t; g < SM::NG; g += NT) {
         const int e = gtab[g];
-        E[e & 2047] = (TT)y[(int64_t)snb[(e >> 11) & 31] * pv.vs + (e >> 16)];
+        E[e & 2047] = (TT)y[(int64_t)nbs[(e >> 11) & 31] * pv.vs + (e >> 16)];
       }
     } else {
       if (!(plan_ok && all_blocks)) {
@@ -757,7 +769,7 @@ __global__ void __launch_bounds__(Col3::NT, sizeof(TS) == 8 ? 2 : 3) k_details3(
 #pragma unroll
       for (int k = 0; k < B; ++k) {
         mqa.add(v[k]);
-        bad |= !isfinite(v[k]);
+        bad |= !finite(v[k]);
       }
       if (((x | yy) & 1) == 0) {
         TT* e0 = E + CP + (yy / 2 + 1) * CN + x / 2 + 1;
@@ -765,6 +777,7 @@ __global__ void __launch_bounds__(Col3::NT, sizeof(TS) == 8 ? 2 : 3) k_details3(
         for (int k = 0; k < B; k += 2) e0[CP * (k / 2)] = v[k];
       }
     }
+    if (bad) nonfinite = 1;
     __syncthreads();
     // x pass on the coarse rows into X, y pass of the column, z pass and the
     // detail at every odd node; with EX also the coarse lattice's largest |value|
@@ -837,9 +850,9 @@ __global__ void __launch_bounds__(Col3::NT, sizeof(TS) == 8 ? 2 : 3) k_details3(
     } else {
       md = (double)m0;
     }
-    const bool nan = __syncthreads_or(bad);
     if (t == 0) {
-      if (nan) md = __longlong_as_double(0x7ff8000000000000LL);
+      if (nonfinite) md = __longlong_as_double(0x7ff8000000000000LL);
+      nonfinite = 0;
       pv.md[b.slot] = md;
       pv.bmax[b.slot] = (double)mq;
       if (pv.norm_kind == 1) csv = fmax(csv, (double)mq);

@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(128, 8) k_details2(PoolView pv, TS* __restrict
       if (n >= NI) continue;
       const TT t = val[k] = to_tile<TT>(raw[k]);
       mqa.add(t);
-      bad |= !isfinite(t);
+      bad |= !finite(t);
       const int e = ntab[n];
       if (((e >> 12) & 3) == 0) E[e & 0xfff] = t;
     }
@@ -299,7 +299,8 @@ __global__ void __launch_bounds__(128, 8) k_details2(PoolView pv, TS* __restrict
         __syncthreads();
         if ((threadIdx.x & 31) == 0) r[threadIdx.x >> 5] = m;
         __syncthreads();
-        m = fmax(fmax(r[0], r[1]), fmax(r[2], r[3]));
+        const int w = threadIdx.x & 31;
+        m = warp_max_pos(w < 4 ? r[w] : A(0));
       }
       return m;
     };

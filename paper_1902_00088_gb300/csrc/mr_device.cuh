@@ -92,6 +92,10 @@ __device__ __forceinline__ TT to_tile(TS v) {
   if constexpr (sizeof(TS) == 8 && sizeof(TT) == 4) return f64_to_f32(v);
   else return (TT)v;
 }
+// Neither infinite nor NaN, likewise on the bit pattern (3D details, 2584 FP64 blocks:
+// 514 -> 470 us; 4096 blocks of 33^2 112 -> 92).
+__device__ __forceinline__ bool finite(float v) { return (__float_as_uint(v) & 0x7f800000u) != 0x7f800000u; }
+__device__ __forceinline__ bool finite(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
 // a != b of two finite or infinite values, doubles on their bit patterns (as above).
 __device__ __forceinline__ bool differs(float a, float b) { return a != b; }
 __device__ __forceinline__ bool differs(double a, double b) {
