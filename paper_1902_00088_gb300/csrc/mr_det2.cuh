@@ -10,105 +10,105 @@ namespace mr {
 // the ghost layer is a node of its owner whatever the owner's level, so 40 (17^2)
 // or 72 (33^2) ghost nodes are gathered and none is predicted.
 //
-// Rows of the work array, one per coarse y (-1 .. NC - 2): the NC coarse nodes,
-// then the x pass at the odd nodes between them.
+// Work array S: the block's own nodes row after row without padding, as they lie in
+// the pool (one bulk copy), the ghost rows y = -2 and B + 1 where that pitch puts
+// them, and the coarse ghosts x = -2 and B + 1 of every coarse row apart.  The x pass
+// takes the detail of an odd node of an even row and leaves its prediction in the
+// node's place; the y pass then reads rows y -+ 1 and y -+ 3 at every x alike.
 template <int B>
 struct Det2 {
   static constexpr int NC = (B + 1) / 2 + 2, NO = (B - 1) / 2;
-  static constexpr int RP = NC + NO, SZ = NC * RP;
-  static constexpr int NI = B * B;
+  static constexpr int NI = B * B, VS = (NI + 3) / 4 * 4;
   static constexpr int NG = NC * NC - ((B + 1) / 2) * ((B + 1) / 2);
   static constexpr int GS = B == 17 ? 32 : 128;        // threads per item
   static constexpr int NT = 128, ITEMS = NT / GS;      // threads and items per CTA
-  static constexpr int K = (NI + GS - 1) / GS;         // nodes per thread
   static constexpr int NE = 4 * (B - 1);               // edge nodes
+  static constexpr int NU = 2 * B - 1;                 // ... held by the upper neighbours
+  static constexpr int R0 = (2 * B + 3) / 4 * 4;       // node (0, 0), 16-byte aligned
+  static constexpr int GL = R0 + B * (B + 2), GR = GL + NC, SZ = GR + NC;
   // edge node e: lower edge from x = 0, right edge upward, upper edge back, left edge down
   __device__ static __forceinline__ void edge(int e, int& i, int& j) {
     const int s = e / (B - 1), r = e % (B - 1);
     i = s == 0 ? r : s == 1 ? B - 1 : s == 2 ? B - 1 - r : 0;
     j = s == 0 ? 0 : s == 1 ? r : s == 2 ? B - 1 : B - 1 - r;
   }
-  __device__ static __forceinline__ int edge_of(int i, int j) {  // -1: not an edge node
-    return j == 0 && i < B - 1 ? i : i == B - 1 && j < B - 1 ? B - 1 + j : j == B - 1 && i > 0 ? 3 * (B - 1) - i
-           : i == 0 ? 4 * (B - 1) - j : -1;
+  // coarse lattice position (0 .. NC - 1, at node 2 (n - 1)) of ghost node k: lower and
+  // upper row, then the pairs left and right of the rows between
+  __device__ static __forceinline__ void ghost(int k, int& nx, int& ny) {
+    if (k < 2 * NC) {
+      nx = k < NC ? k : k - NC;
+      ny = k < NC ? 0 : NC - 1;
+    } else {
+      nx = (k & 1) ? NC - 1 : 0;
+      ny = (k - 2 * NC) / 2 + 1;
+    }
   }
-  // place of node x in a row: coarse nodes (even x) from 1, odd ones after them
-  __host__ __device__ static constexpr int place(int x) { return (x & 1) ? NC + x / 2 : 1 + x / 2; }
+  __device__ static __forceinline__ int at_ghost(int nx, int ny) {
+    return nx == 0 ? GL + ny : nx == NC - 1 ? GR + ny : R0 + 2 * B * (ny - 1) + 2 * (nx - 1);
+  }
 };
 
 template <int B, typename TS, typename TT, typename TD>
 struct Det2Smem {
   using D2 = Det2<B>;
-  static constexpr size_t TABS = (4 * (D2::NI + D2::NG) + 15) / 16 * 16;  // per CTA
-  static constexpr size_t RING = ((size_t)kRingBytesD<2> + 15) / 16 * 16;
-  static constexpr size_t W = (sizeof(TT) * D2::SZ + 15) / 16 * 16;
+  static constexpr size_t up(size_t x) { return (x + 15) / 16 * 16; }
+  static constexpr size_t TABS = up(4 * D2::NG);  // per CTA
+  static constexpr size_t RING = up(kRingBytesD<2>);
+  static constexpr size_t W = up(sizeof(TT) * D2::SZ);
   // x pass of the FP64 evaluation of FP32 values
-  static constexpr size_t XD = sizeof(TD) > sizeof(TT) ? sizeof(TD) * D2::NC * D2::NO : 0;
-  static constexpr size_t NB = 80;                                          // neighbours' pool offsets
-  static constexpr size_t EV = sizeof(TS) * D2::NE;  // edge values (a multiple of 16 bytes)
-  static constexpr size_t ITEM = RING + W + (XD + 15) / 16 * 16 + EV + NB;
+  static constexpr size_t XD = sizeof(TD) > sizeof(TT) ? up(sizeof(TD) * D2::NC * D2::NO) : 0;
+  static constexpr size_t NB = 96;  // mbarrier, the neighbours' pool offsets
+  static constexpr size_t ITEM = NB + RING + W + XD;
   static constexpr size_t BYTES = TABS + D2::ITEMS * ITEM;
 };
 
-// Bound by instruction issue and latency (48 % of the issue slots used); 12 CTAs per SM
-// spill, 6 hide less latency: 8 CTAs of 4 warps.  Measured, before with one CTA (or warp) per block over the gathered and
-// predicted 21^2 tile, variable after variable: 65536 FP32 blocks of 17^2 104 -> 78 us;
-// 16384 blocks of 4 FP64 variables 165 -> 101 us; the rounds of an adaptive step with 64
-// trees 168 -> 94 us, with 33^2 blocks of 4 variables 443 -> 238 us (a third of it by
-// looking the owners of a block's edge nodes up apart from its own nodes).
+// Bound by instruction issue (66 % of the slots before the in-place x pass) and by
+// shared wavefronts.  Measured, first with one CTA (or warp) per block over the
+// gathered and predicted 21^2 tile, then with a table entry per node and a separate
+// work array, now: 65536 FP32 blocks of 17^2 104, 75, 61 us; the rounds of an adaptive
+// step with 64 trees 168, 92, 77; with 33^2 blocks of 4 variables 443, 238, 196; with 46
+// FP64 blocks of 17^2 66, 49, 41.  CTAs per SM: 17^2 8 (10: 68 us, 12: 70, 6: 74 on 65536
+// blocks), 33^2 12 (8: 241 us, 10: 206, 14: 204 on four variables).
 template <int B, typename TS, typename TD, typename TT>
-__global__ void __launch_bounds__(128, 8) k_details2(PoolView pv, TS* __restrict__ y) {
+__global__ void __launch_bounds__(128, B == 17 ? 8 : 12) k_details2(PoolView pv, TS* __restrict__ y) {
   pdl_enter();
   using D2 = Det2<B>;
   using SM = Det2Smem<B, TS, TT, TD>;
   using PL = Plan<2>;
   using G = std::conditional_t<D2::GS == 32, WarpGroup, CtaGroup>;
-  constexpr int NC = D2::NC, NO = D2::NO, RP = D2::RP, NI = D2::NI, GS = D2::GS, K = D2::K;
+  constexpr int NC = D2::NC, NO = D2::NO, NI = D2::NI, GS = D2::GS;
+  constexpr bool BULK = std::is_same<TS, TT>::value;  // own nodes by a bulk copy
   const G g{};
   const int rank = threadIdx.x % GS, item = threadIdx.x / GS;
   unsigned char* sm = smem_as<unsigned char>(0);
-  int32_t* ntab = reinterpret_cast<int32_t*>(sm);
-  int32_t* gtab = ntab + NI;
+  int32_t* gtab = reinterpret_cast<int32_t*>(sm);
   unsigned char* mem = sm + SM::TABS + item * SM::ITEM;
-  RingD<2>& R = *reinterpret_cast<RingD<2>*>(mem);
-  TT* E = reinterpret_cast<TT*>(mem + SM::RING);
-  TD* XD = reinterpret_cast<TD*>(mem + SM::RING + SM::W);
-  int64_t* nbo = reinterpret_cast<int64_t*>(mem + SM::ITEM - SM::NB);
-  TS* ev = reinterpret_cast<TS*>(mem + SM::ITEM - SM::NB - SM::EV);
+  uint64_t* bar = reinterpret_cast<uint64_t*>(mem);
+  int64_t* nbo = reinterpret_cast<int64_t*>(mem + 16);
+  RingD<2>& R = *reinterpret_cast<RingD<2>*>(mem + SM::NB);
+  TT* E = reinterpret_cast<TT*>(mem + SM::NB + SM::RING);
+  TT* S = E + D2::R0;  // node (0, 0)
+  TD* XD = reinterpret_cast<TD*>(mem + SM::NB + SM::RING + SM::W);
   __shared__ double red[4];
   const int nact = pv.cnt->n_round, nv = pv.nvar;
   if ((int64_t)blockIdx.x * D2::ITEMS >= (int64_t)nact * nv) return;  // no item for this CTA (small grids)
-  // nodes: place in the work array | kind << 12 (0 coarse, 1 odd x on a coarse row, 2
-  // odd y) | upper edge in x << 14, in y << 15 | edge node << 16 (0: none, else + 1)
-  for (int q = threadIdx.x; q < NI; q += blockDim.x) {
-    const int i = q % B, j = q / B;
-    const int row = (j & 1) ? j / 2 : j / 2 + 1;  // first row of the y pass, or the node's own
-    const int kind = (j & 1) ? 2 : (i & 1);
-    ntab[q] = (row * RP + D2::place(i)) | (kind << 12) | (i == B - 1 ? 1 << 14 : 0) | (j == B - 1 ? 1 << 15 : 0) |
-              ((D2::edge_of(i, j) + 1) << 16);
-  }
+  if (BULK && rank == 0) mbar_init(bar, 1);
+  unsigned phase = 0;
   // ghost nodes: place | neighbour << 12 | offset in that neighbour (of a uniform
   // neighbourhood) << 16
-  for (int q = threadIdx.x; q < D2::NG; q += blockDim.x) {
-    int n[2];  // coarse lattice position, at node 2 (n - 1)
-    if (q < 2 * NC) {
-      n[0] = q % NC;
-      n[1] = q < NC ? 0 : NC - 1;
-    } else {
-      const int r = q - 2 * NC;
-      n[0] = r % 2 ? NC - 1 : 0;
-      n[1] = r / 2 + 1;
-    }
+  for (int k = threadIdx.x; k < D2::NG; k += blockDim.x) {
+    int n[2];
+    D2::ghost(k, n[0], n[1]);
     int nb = 0, off = 0, mul = 1, lm = 1;
     for (int a = 0; a < 2; ++a) {
-      const int k = 2 * (n[a] - 1);
-      const int s = k < 0 ? 0 : (k <= B - 2 ? 1 : 2);
+      const int x = 2 * (n[a] - 1);
+      const int s = x < 0 ? 0 : (x <= B - 2 ? 1 : 2);
       nb += s * mul;
-      off += (k - (s - 1) * (B - 1)) * lm;
+      off += (x - (s - 1) * (B - 1)) * lm;
       mul *= 3;
       lm *= B;
     }
-    gtab[q] = (n[1] * RP + n[0]) | (nb << 12) | (off << 16);
+    gtab[k] = D2::at_ghost(n[0], n[1]) | (nb << 12) | (off << 16);
   }
   __syncthreads();
   auto group_and = [&](bool p) -> bool {
@@ -175,28 +175,62 @@ __global__ void __launch_bounds__(128, 8) k_details2(PoolView pv, TS* __restrict
     ndet += v == 0;
     const int64_t vo = (int64_t)v * pv.vs, bs = (int64_t)nv * pv.vs;  // variable offset, block stride
     TS* const me = y + (int64_t)b.slot * bs + vo;
-    // the thread's nodes; block-edge nodes held by another block take (and
-    // store) its value
-    TS raw[K];
+    // own nodes; block-edge nodes held by another block take (and store) its value
+    if constexpr (BULK) {
+      if (rank == 0) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        mbar_expect_tx(bar, sizeof(TT) * D2::VS);
+        bulk_g2s(S, me, sizeof(TT) * D2::VS, bar);
+      }
+    } else {
+#pragma unroll 5
+      for (int n = rank; n < NI; n += GS) S[n] = to_tile<TT>(me[n]);
+    }
+    auto landed = [&]() {
+      if constexpr (BULK) {
+        // bounded wait: a copy that never lands is reported, not waited for
+        if (!mbar_wait(bar, phase, 1 << 20)) set_err(pv, kErrTimeout);
+        phase ^= 1;
+      } else {
+        g.sync();
+      }
+    };
+    auto commit = [&](int n, TS v) {
+      TS mine;
+      if constexpr (BULK) mine = S[n];
+      else mine = me[n];
+      if (differs(mine, v)) me[n] = v;
+      S[n] = to_tile<TT>(v);
+    };
     if (uni) {
       if (rank < PL::NB) nbo[rank] = (int64_t)q * bs + vo;
       g.sync();
+      constexpr int RE = (D2::NU + GS - 1) / GS, RG = (D2::NG + GS - 1) / GS;
+      TS ve[RE], vg[RG];
 #pragma unroll
-      for (int k = 0; k < K; ++k) {
-        const int n = rank + k * GS;
-        if (n >= NI) continue;
-        const int e = ntab[n];
-        const int ux = (e >> 14) & 1, uy = (e >> 15) & 1;
-        raw[k] = y[nbo[4 + ux + 3 * uy] + n - ux * (B - 1) - uy * (B * (B - 1))];
+      for (int u = 0; u < RE; ++u) {  // column B - 1, then row B - 1
+        const int e = rank + u * GS;
+        if (e >= D2::NU) continue;
+        const int ux = e < B, uy = e >= B - 1;
+        ve[u] = y[nbo[4 + ux + 3 * uy] + (e < B ? 0 : e - B) + (uy ? 0 : B * e)];
       }
-      for (int k = rank; k < D2::NG; k += GS) {
+#pragma unroll
+      for (int u = 0; u < RG; ++u) {
+        const int k = rank + u * GS;
+        if (k >= D2::NG) continue;
         const int e = gtab[k];
-        E[e & 0xfff] = to_tile<TT>(y[nbo[(e >> 12) & 15] + (e >> 16)]);
+        vg[u] = y[nbo[(e >> 12) & 15] + (e >> 16)];
+      }
+      landed();
+#pragma unroll
+      for (int u = 0; u < RE; ++u) {
+        const int e = rank + u * GS;
+        if (e < D2::NU) commit(e < B ? B * e + B - 1 : B * (B - 1) + e - B, ve[u]);
       }
 #pragma unroll
-      for (int k = 0; k < K; ++k) {
-        const int n = rank + k * GS;
-        if (n < NI && (ntab[n] & (3 << 14)) && differs(me[n], raw[k])) me[n] = raw[k];
+      for (int u = 0; u < RG; ++u) {
+        const int k = rank + u * GS;
+        if (k < D2::NG) E[gtab[k] & 0xfff] = to_tile<TT>(vg[u]);
       }
     } else {
       if (!ring && plan_ok) {  // the stage plan's owner table
@@ -217,78 +251,81 @@ __global__ void __launch_bounds__(128, 8) k_details2(PoolView pv, TS* __restrict
         const int ox = 2 * i - (int)(int16_t)(e.z & 0xffff), oy = 2 * j - (e.z >> 16);
         return (int64_t)e.x * bs + vo + (ox >> sh) + B * (oy >> sh);
       };
+      constexpr int RE = (D2::NE + GS - 1) / GS, RG = (D2::NG + GS - 1) / GS;
+      TS ve[RE], vg[RG];
+      unsigned other = 0;  // edge nodes of other blocks
 #pragma unroll
-      for (int k = 0; k < K; ++k) {
-        const int n = rank + k * GS;
-        if (n < NI) raw[k] = me[n];
-      }
-      for (int k = rank; k < D2::NE; k += GS) {
+      for (int u = 0; u < RE; ++u) {
+        const int k = rank + u * GS;
+        if (k >= D2::NE) continue;
         int i, j;
         D2::edge(k, i, j);
         const int4 e = R.reg[reg_class<B>(i) + 7 * reg_class<B>(j)];
-        const int n = j * B + i;
-        TS val = me[n];
-        if (e.x < 0) {
-          lost = true;
-          val = TS(0);
-        } else if (e.x != b.slot) {
-          const TS mine = val;
-          val = y[owned(e, i, j)];
-          if (differs(mine, val)) me[n] = val;
-        }
-        ev[k] = val;
+        ve[u] = TS(0);
+        if (e.x < 0) lost = true;
+        else if (e.x != b.slot) ve[u] = y[owned(e, i, j)];
+        if (e.x != b.slot) other |= 1u << u;
       }
-      for (int k = rank; k < D2::NG; k += GS) {
-        const int at = gtab[k] & 0xfff;
-        const int i = 2 * (at % RP - 1), j = 2 * (at / RP - 1);
+#pragma unroll
+      for (int u = 0; u < RG; ++u) {
+        const int k = rank + u * GS;
+        if (k >= D2::NG) continue;
+        int nx, ny;
+        D2::ghost(k, nx, ny);
+        const int i = 2 * (nx - 1), j = 2 * (ny - 1);
         const int4 e = R.reg[reg_class<B>(i) + 7 * reg_class<B>(j)];
         const bool ok = e.x >= 0 && e.y >= b.lvl - 1;
         lost |= !ok;
-        E[at] = ok ? to_tile<TT>(y[owned(e, i, j)]) : TT(0);
+        vg[u] = ok ? y[owned(e, i, j)] : TS(0);
       }
-      g.sync();
+      landed();
 #pragma unroll
-      for (int k = 0; k < K; ++k) {
-        const int n = rank + k * GS;
-        if (n < NI && (ntab[n] >> 16)) raw[k] = ev[(ntab[n] >> 16) - 1];
+      for (int u = 0; u < RE; ++u) {
+        if (!((other >> u) & 1)) continue;
+        int i, j;
+        D2::edge(rank + u * GS, i, j);
+        if (lost) S[j * B + i] = TT(0);  // an error: the pool stays as it is
+        else commit(j * B + i, ve[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < RG; ++u) {
+        const int k = rank + u * GS;
+        if (k < D2::NG) E[gtab[k] & 0xfff] = to_tile<TT>(vg[u]);
       }
       if (lost) set_err(pv, kErrGraded);
     }
-    // largest |value| of the interior, non-finite test, coarse nodes to the work array
-    AbsMax<TT> mqa;
+    g.sync();
+    // x pass with the details of the even rows, then the y pass with those of the odd
+    // ones; every own node is read once: largest |value|, non-finite test
+    AbsMax<TT> mqa, md;
     bool bad = false;
-    TT val[K];
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      const int n = rank + k * GS;
-      if (n >= NI) continue;
-      const TT t = val[k] = to_tile<TT>(raw[k]);
+    auto seen = [&](TT t) {
       mqa.add(t);
       bad |= !finite(t);
-      const int e = ntab[n];
-      if (((e >> 12) & 3) == 0) E[e & 0xfff] = t;
-    }
-    g.sync();
-    // x pass, then the y pass and the detail at the thread's odd nodes
+    };
     float mt = 0.f;  // largest |value| of the coarse lattice
-    AbsMax<TT> md;
     for (int k = rank; k < NC * NO; k += GS) {
-      TT* r = E + (k / NO) * RP;
-      const int m = k % NO;
-      const TT a = r[m], c = r[m + 1], d = r[m + 2], f = r[m + 3];
+      const int r = k / NO, m = k % NO;
+      TT* w = S + 2 * B * (r - 1) + 2 * m;
+      const TT a = m == 0 ? E[D2::GL + r] : w[-2], c = w[0], d = w[2], f = m == NO - 1 ? E[D2::GR + r] : w[4];
       mt = fmaxf(fmaxf(mt, fmaxf(fabsf((float)a), fabsf((float)c))), fmaxf(fabsf((float)d), fabsf((float)f)));
-      r[NC + m] = dd4(a, c, d, f);
+      const TT pr = dd4(a, c, d, f);
+      if (r >= 1 && r <= NC - 2) {
+        seen(c);
+        if (m == NO - 1) seen(d);
+        const TT v = w[1];
+        seen(v);
+        md.add(v - pr);
+      }
+      w[1] = pr;
     }
     g.sync();
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      const int n = rank + k * GS;
-      if (n >= NI) continue;
-      const int e = ntab[n], kind = (e >> 12) & 3;
-      if (kind == 0) continue;
-      const TT* r = E + (e & 0xfff);
-      const TT pr = kind == 2 ? dd4(r[0], r[RP], r[2 * RP], r[3 * RP]) : r[0];
-      md.add(val[k] - pr);
+    for (int k = rank; k < NO * B; k += GS) {
+      const int m = k / B;
+      const TT* w = S + k + B * (m + 1);  // row 2 m + 1
+      const TT v = w[0];
+      seen(v);
+      md.add(v - dd4(w[-3 * B], w[-B], w[B], w[3 * B]));
     }
     constexpr bool cert = sizeof(TT) == 4 && sizeof(TD) == 8;
     auto group_max = [&](auto m) {
@@ -311,22 +348,24 @@ __global__ void __launch_bounds__(128, 8) k_details2(PoolView pv, TS* __restrict
       // certified as in k_details3: err bounds the FP32 evaluation's error
       const float err = 0x1p-19f * fmaxf(group_max(mt), (float)mq) + 1e-37f;
       if (!(pv.norm_kind == 0 && certain_vs_eps(m0, err, td))) {
+        // again in FP64; the odd nodes of the even rows are read back from the pool
+        AbsMax<TD> md64;
         for (int k = rank; k < NC * NO; k += GS) {
-          const TT* r = E + (k / NO) * RP + k % NO;
-          XD[k] = dd4((TD)r[0], (TD)r[1], (TD)r[2], (TD)r[3]);
+          const int r = k / NO, m2 = k % NO;
+          const TT* w = S + 2 * B * (r - 1) + 2 * m2;
+          const TD pr = dd4((TD)(m2 == 0 ? E[D2::GL + r] : w[-2]), (TD)w[0], (TD)w[2],
+                            (TD)(m2 == NO - 1 ? E[D2::GR + r] : w[4]));
+          XD[r * NO + m2] = pr;
+          if (r >= 1 && r <= NC - 2) md64.add((TD)me[2 * B * (r - 1) + 2 * m2 + 1] - pr);
         }
         g.sync();
-        AbsMax<TD> md64;
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-          const int n = rank + k * GS;
-          if (n >= NI) continue;
-          const int e = ntab[n], kind = (e >> 12) & 3;
-          if (kind == 0) continue;
-          const int row = (e & 0xfff) / RP, c = (e & 0xfff) % RP;
-          auto at = [&](int r) -> TD { return c < NC ? (TD)E[r * RP + c] : XD[r * NO + c - NC]; };
-          const TD pr = kind == 2 ? dd4(at(row), at(row + 1), at(row + 2), at(row + 3)) : at(row);
-          md64.add((TD)val[k] - pr);
+        for (int k = rank; k < NO * B; k += GS) {
+          const int m2 = k / B, x = k - m2 * B;
+          const TT* w = S + k + B * (m2 + 1);
+          const TD* xd = XD + m2 * NO + x / 2;
+          const TD pr = (x & 1) ? dd4(xd[0], xd[NO], xd[2 * NO], xd[3 * NO])
+                                : dd4((TD)w[-3 * B], (TD)w[-B], (TD)w[B], (TD)w[3 * B]);
+          md64.add((TD)w[0] - pr);
         }
         m = (double)group_max(md64.get());
       }
