@@ -114,7 +114,8 @@ TRAFFIC = {
 }
 
 
-DEVICE_SOURCES = ("mr_device.cuh", "mr_internal.h", "mr_kernels.cuh", "mr_launch.cuh")
+DEVICE_SOURCES = ("mr_adv2.cuh", "mr_adv3.cuh", "mr_det2.cuh", "mr_device.cuh", "mr_internal.h", "mr_kernels.cuh",
+                  "mr_launch.cuh")
 NS_SOURCES = DEVICE_SOURCES + ("mr_ns.cuh",)  # the skew-symmetric stage and the shock filter
 
 
@@ -833,12 +834,12 @@ def main():
     stage_ms = st["ms"]["stage"]
     kern["stage"] = dict(
         kernel="%s (RK stage incl. fused ghost gather)" % {"ns": "k_stage_ns", "ns_skew": "k_stage_nss"}.get(
-            w["rhs"], "k_stage_adv"),
+            w["rhs"], "k_stage%d" % w["dim"]),
         ms=stage_ms, launches=st["stage_launches"], blocks=st["stage_blocks"],
         bytes=st["stage_blocks"] * bytes_per_stage_block(w))
     det_s = 4 if w["precision"] == "fp32" else 8
     kern["details"] = dict(
-        kernel="k_details (ghost gather + wavelet details + block norms)", ms=st["ms"]["details"],
+        kernel="k_details%d (ghost gather + wavelet details + block norms)" % w["dim"], ms=st["ms"]["details"],
         launches=st["det_launches"], blocks=st["det_blocks"],
         bytes=st["det_blocks"] * (w["Bs"] ** w["dim"]) * w.get("nvar", 1) * det_s)
     if st["ms"].get("filter", 0.0) > 0:

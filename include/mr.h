@@ -327,9 +327,9 @@ mr_status mr_get_step_history(mr_ctx ctx, int64_t cap, int32_t* out, int64_t* n,
 mr_status mr_autotune(mr_ctx ctx, int32_t steps, int32_t* best);
 /* Fixes the launch configuration instead of the autotuner: ctas_per_sm
  * persistent CTAs per SM for the block kernels (0 = as many as occupancy
- * allows, at most 32) and the form of the 2D stage and details kernels on 17^2
- * advection blocks (stage_form 1 = one warp per block, 0 = one CTA per block,
- * -1 = by block count: warps once the grid holds 8 blocks per SM).  Results do
+ * allows, at most 32) and the form of the 2D stage kernel on 17^2 advection
+ * blocks (stage_form 1 = one warp per block, 0 = one CTA per block, -1 = by
+ * block count: warps once the grid holds 8 blocks per SM, 32 with FP64 states).  Results do
  * not depend on either choice.  MR_EINVAL for values out of range or the warp
  * form where it does not exist.  Drops the captured step. */
 mr_status mr_set_tuning(mr_ctx ctx, int32_t ctas_per_sm, int32_t stage_form);
