@@ -362,17 +362,17 @@ __global__ void __launch_bounds__(GT * NW, GT == 32 ? 20 / NW : 1024 / GT) k_sta
           u1 = -(ct * (fac[2 * (B + j)] * fac[2 * i + 1]));
         }
         const TC s = u0 * dxv + u1 * dyv;
-        const TS kk = (TS)(-s);
+        const TS kk = to_state<TS>(-s);
         const int64_t at = own + q;
         if (ST == 0) {
           TS y0;
           if constexpr (Y0) y0 = ys[q];
           else y0 = t0[0];
           acc[at] = y0 + cas * kk;
-          ynext[at] = (TY)(y0 + cys * kk);
+          ynext[at] = to_tile<TY>(y0 + cys * kk);
         } else if (NEEDY) {
           acc[at] = av[u] + cas * kk;
-          ynext[at] = (TY)(yv[u] + cys * kk);
+          ynext[at] = to_tile<TY>(yv[u] + cys * kk);
         } else {
           y[at] = av[u] + cas * kk;
         }

@@ -453,13 +453,13 @@ __global__ void __launch_bounds__(Stage3Smem<TY, TS>::NT, 2) k_stage3(PoolView p
       const TC dzv = d1_sum(zm2, zm1, zp1, zp2) * cd;
       TC s = u0 * dxv + u1 * dyv;
       s = s + u2 * dzv;
-      const TS kk = (TS)(-s);
+      const TS kk = to_state<TS>(-s);
       if (ST == 0) {
         acc[at] = yk + cas * kk;
-        ynext[at] = (TY)(yk + cys * kk);
+        ynext[at] = to_tile<TY>(yk + cys * kk);
       } else if (ST == 1 || ST == 2) {
         acc[at] = ak + cas * kk;
-        ynext[at] = (TY)(yk + cys * kk);
+        ynext[at] = to_tile<TY>(yk + cys * kk);
       } else {
         y[at] = ak + cas * kk;
       }
