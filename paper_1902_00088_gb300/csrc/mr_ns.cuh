@@ -109,7 +109,8 @@ struct NsUpdate {
     else return (TS)v;
   }
   __device__ __forceinline__ void load(const TS* y, const TS* acc, const TC* yn, int64_t at, int stage) {
-    yv = (stage == 0 || (!MIX && stage <= 2)) ? y[at] : TS(0);
+    // stage 0 of one type takes the committed state from the tile
+    yv = (MIX ? stage == 0 : stage == 1 || stage == 2) ? y[at] : TS(0);
     av = stage >= 1 ? acc[at] : TS(0);
     yf = TC(0);
     if (MIX && (stage == 1 || stage == 2)) yf = yn[at];
@@ -132,8 +133,8 @@ struct NsUpdate {
     } else {
       const TS kk = (TS)k;
       if (stage == 0) {
-        acc[at] = yv + cs.ca * kk;
-        ynext[at] = (TC)(yv + cs.cy * kk);
+        acc[at] = (TS)tile0 + cs.ca * kk;
+        ynext[at] = (TC)((TS)tile0 + cs.cy * kk);
       } else if (stage == 1 || stage == 2) {
         acc[at] = av + cs.ca * kk;
         ynext[at] = (TC)(yv + cs.cy * kk);
@@ -278,7 +279,8 @@ __global__ void __launch_bounds__(NsCfg<B, TY>::NT, NsCfg<B, TY>::MINB) k_stage_
     const StageCoef<TS> cs(pv, sa, b.tree, stage);  // RK weights in the state type
     const StageCoef<TC> cf(pv, sa, b.tree, stage);  // and in the stage type
     const int64_t base = (int64_t)b.slot * 4 * pv.vs;
-    const TS* yc = stage == 0 ? committed(y, src) : y;
+    const TS* yc = y;
+    if constexpr (sizeof(TS) != sizeof(TC)) yc = committed(y, src);
     for (int q = threadIdx.x; q < NI; q += blockDim.x) {
       const int i = q % B, j = q / B;
       NsUpdate<TS, TC, true> up[4];
@@ -426,7 +428,8 @@ __global__ void __launch_bounds__(NssCfg<B, TY>::NT, NssCfg<B, TY>::MINB) k_stag
     const StageCoef<TS> cs(pv, sa, b.tree, stage);
     const StageCoef<TC> cf(pv, sa, b.tree, stage);
     const int64_t base = (int64_t)b.slot * 4 * pv.vs;
-    const TS* yc = stage == 0 ? committed(y, src) : y;
+    const TS* yc = y;
+    if constexpr (sizeof(TS) != sizeof(TC)) yc = committed(y, src);
     for (int q = threadIdx.x; q < NI; q += blockDim.x) {
       const int i = q % B, j = q / B;
       const int o = I(i, j);
