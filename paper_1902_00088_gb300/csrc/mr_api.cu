@@ -135,6 +135,19 @@ struct TmpBuf {
   }
 };
 
+// Waits for the stream when a call returns with an error while its copies from or
+// to the caller's memory are queued: they must not run after the call.
+struct DrainOnError {
+  cudaStream_t st;
+  bool done = false;
+  explicit DrainOnError(cudaStream_t s) : st(s) {}
+  DrainOnError(const DrainOnError&) = delete;
+  DrainOnError& operator=(const DrainOnError&) = delete;
+  ~DrainOnError() {
+    if (!done) cudaStreamSynchronize(st);
+  }
+};
+
 template <typename T>
 cudaError_t dalloc(mr_ctx c, T** p, size_t n) {
   void* q = nullptr;
@@ -1608,6 +1621,7 @@ mr_status mr_cnn_eval(mr_ctx ctx, const float* params, const float* x, const flo
   TmpBuf<float> d;
   CK(d.alloc_on((nin + nout) * 4, ctx->st));
   float *dx = d.p, *dy = dx + n * fl, *dw = dy + n, *dg = dw + kCnnParams, *dl = dg + kCnnParams, *dp = dl + 1;
+  DrainOnError drain(ctx->st);
   CK(cudaMemcpyAsync(dx, x, n * fl * 4, cudaMemcpyHostToDevice, ctx->st));
   CK(cudaMemcpyAsync(dy, y, n * 4, cudaMemcpyHostToDevice, ctx->st));
   CK(cudaMemcpyAsync(dw, params, kCnnParams * 4, cudaMemcpyHostToDevice, ctx->st));
@@ -1618,6 +1632,7 @@ mr_status mr_cnn_eval(mr_ctx ctx, const float* params, const float* x, const flo
   if (grad) CK(cudaMemcpyAsync(grad, dg, kCnnParams * 4, cudaMemcpyDeviceToHost, ctx->st));
   if (loss) CK(cudaMemcpyAsync(loss, dl, 4, cudaMemcpyDeviceToHost, ctx->st));
   CK(cudaStreamSynchronize(ctx->st));
+  drain.done = true;
   return MR_OK;
 }
 
