@@ -244,8 +244,8 @@ __global__ void __launch_bounds__(GT * NW, GT == 32 ? 20 / NW : 1024 / GT) k_sta
         const int4 e = reg[reg_class<B>(i) + 7 * reg_class<B>(j)];
         if (h >= NG && e.x == b.slot) continue;
         if (e.x < 0) {
-          bad = true;
-          have |= 1u << u;  // zero
+          bad = true;  // zero; of an edge node in the tile only: the pool stays as it is
+          (h >= NG ? pred : have) |= 1u << u;
           continue;
         }
         const int sh = l1 - e.y, ox = 2 * i - (int)(int16_t)(e.z & 0xffff), oy = 2 * j - (e.z >> 16);
@@ -305,6 +305,7 @@ __global__ void __launch_bounds__(GT * NW, GT == 32 ? 20 / NW : 1024 / GT) k_sta
           i = s == 0 ? w : s == 1 ? B - 1 : s == 2 ? w + 1 : 0;
           j = s == 0 ? 0 : s == 1 ? w : s == 2 ? B - 1 : w + 1;
           if ((have >> u) & 1) commit(i, j, val[u]);
+          if ((pred >> u) & 1) tile[B * j + i] = TC(0);
           continue;
         }
         TC v = to_tile<TC>(val[u]);

@@ -252,13 +252,13 @@ __global__ void __launch_bounds__(Stage3Smem<TY, TS>::NT, 2) k_stage3(PoolView p
               for (int j = J0; j <= J1; ++j) raw[j] = mine[NQ * j];
               return;
             }
-            other |= C == 0 ? 1u : C == 1 ? 0xfeu : 0x100u;
-            if (e.x < 0) {
+            if (e.x < 0) {  // no owner: zero in the tile, the pool stays as it is
               bad = true;
 #pragma unroll
               for (int j = J0; j <= J1; ++j) raw[j] = TSRC(0);
               return;
             }
+            other |= C == 0 ? 1u : C == 1 ? 0xfeu : 0x100u;
             const ColOwn o(e, l1, x, yy, pv.vs);
 #pragma unroll
             for (int j = J0; j <= J1; ++j) raw[j] = src[o.at(z0 + j)];

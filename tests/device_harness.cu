@@ -1,0 +1,105 @@
+// Launches single kernels of the library on hand-made blocks, for states that the
+// public calls cannot reach (an owner table without owners).  Built and called by
+// tests/test_gpu_device_harness.py.
+#include <vector>
+
+#include "mr_adv2.cuh"
+#include "mr_adv3.cuh"
+
+using namespace mr;
+
+namespace {
+
+// One tree with one block (slot 0) at level `lvl`; its plan and owner table are the caller's.
+struct OneBlock {
+  std::vector<void*> mem;
+  PoolView pv{};
+  template <typename T>
+  T* put(const std::vector<T>& h) {
+    void* p = nullptr;
+    cudaMalloc(&p, h.size() * sizeof(T));
+    cudaMemcpy(p, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice);
+    mem.push_back(p);
+    return (T*)p;
+  }
+  OneBlock(int dim, int B, int lvl, const std::vector<int32_t>& plan, const std::vector<int4>& regs) {
+    int ni = 1;
+    for (int a = 0; a < dim; ++a) ni *= B;
+    pv.dim = dim; pv.Bs = B; pv.nvar = 1; pv.ntrees = 1; pv.cap = 1;
+    pv.vs = (ni + 3) / 4 * 4;
+    TreeDev td{};
+    td.Jmin = 0; td.Jmax = 4; td.eps = 1.0; td.N = (int64_t)(B - 1) << 4;
+    for (int l = 0; l <= kMaxLevel; ++l) td.cD[l] = td.cDf[l] = 1.0f;
+    for (int a = 0; a < 3; ++a) td.rhs[a] = td.rhsf[a] = 1.0f;
+    Counters c{};
+    c.n_act = c.n_round = 1;
+    c.first_round = 1;
+    pv.trees = put(std::vector<TreeDev>{td});
+    pv.cnt = put(std::vector<Counters>{c});
+    pv.plan = put(plan);
+    pv.regs = put(regs);
+  }
+  int err() {
+    Counters c{};
+    cudaMemcpy(&c, pv.cnt, sizeof(c), cudaMemcpyDeviceToHost);
+    return c.err;
+  }
+  ~OneBlock() {
+    for (void* p : mem) cudaFree(p);
+  }
+};
+
+template <typename K, typename... A>
+bool launch(K k, int threads, size_t smem, A... a) {
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k<<<1, threads, smem>>>(a...);
+  return cudaDeviceSynchronize() == cudaSuccess;
+}
+
+// Stage 0 of a block at level 2 whose ring no leaf covers: the owner table names no owner.
+template <int D, typename TS, typename TY, int GT, int NW>
+int ownerless(TS* y, int* err) {
+  using PL = Plan<D>;
+  std::vector<int32_t> plan(PL::INTS, -1);
+  plan[0] = 0;
+  plan[1] = 2;  // level 2, tree 0, not uniform
+  for (int a = 0; a < D; ++a) plan[2 + a] = a & 1;
+  OneBlock ob(D, 17, 2, plan, std::vector<int4>(reg_entries(D), make_int4(-1, -1, 0, 0)));
+  const int n = (int)ob.pv.vs;
+  TS* dy = ob.put(std::vector<TS>(y, y + n));
+  TS* acc = ob.put(std::vector<TS>(n, TS(0)));
+  TY* next = ob.put(std::vector<TY>(n, TY(0)));
+  StageArgs sa{};
+  bool ok;
+  if constexpr (D == 2) {
+    ok = launch(k_stage2<17, MR_RHS_ADV, TS, TY, TS, GT, NW, 0>, GT * NW, Stage2<17, TS, TY, GT, NW, 0>::BYTES, ob.pv,
+                (const TS*)dy, dy, acc, next, 1, sa);
+  } else {
+    using SM = Stage3Smem<TY, TS>;
+    ok = launch(k_stage3<TS, TY, TS, 0>, SM::NT, SM::BYTES, ob.pv, (const TS*)dy, dy, acc, next, sa);
+  }
+  cudaMemcpy(y, dy, n * sizeof(TS), cudaMemcpyDeviceToHost);
+  *err = ob.err();
+  return ok;
+}
+
+}  // namespace
+
+extern "C" {
+
+// form: 0 FP64, 1 FP32, 2 FP64 state with FP32 stages; warp: one warp per block (2D)
+int ownerless_stage(int dim, int form, int warp, void* y, int* err) {
+  double* d = (double*)y;
+  float* f = (float*)y;
+  if (dim == 2 && warp)
+    return form == 0 ? ownerless<2, double, double, 32, 4>(d, err) : form == 1 ? ownerless<2, float, float, 32, 4>(f, err)
+                                                                   : ownerless<2, double, float, 32, 4>(d, err);
+  if (dim == 2)
+    return form == 0   ? ownerless<2, double, double, 160, 1>(d, err)
+           : form == 1 ? ownerless<2, float, float, 160, 1>(f, err)
+                       : ownerless<2, double, float, 160, 1>(d, err);
+  return form == 0 ? ownerless<3, double, double, 0, 0>(d, err) : form == 1 ? ownerless<3, float, float, 0, 0>(f, err)
+                                                                : ownerless<3, double, float, 0, 0>(d, err);
+}
+
+}  // extern "C"
