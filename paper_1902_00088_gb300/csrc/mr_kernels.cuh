@@ -165,8 +165,23 @@ struct RefGeo {
 // and variable: with the four variables of a mother in one CTA, 376 mothers of 33^2
 // nodes were 1.2 waves of 304 CTAs (335 us); 216 us with 1504 items of a quarter of
 // the shared memory, 138 us with odd and even nodes apart (see below).
-template <int B, typename TS, int NT>
-__global__ void __launch_bounds__(NT, NT <= 128 ? 8 : 4) k_refine(PoolView pv, TS* __restrict__ y) {
+//
+// Launch shape of its own (not the stage's): a mother and variable keeps its CTA
+// waiting on the ring, the owners and the nodes in turn, so CTAs in flight count.
+// Refinement of a step, 17^2 blocks, 8 CTAs of 128 threads (64 registers) per SM against
+// 4 of 160: 64 trees 43 and 53 us, double shear layer 61 and 70, 736 blocks of 4
+// variables 41 and 48 (FP32), 49 and 56 (FP64); 5 of 192: 47, 63, 42, 47; 45 FP64
+// blocks, where a launch is one wave, 28 with any of them.  33^2 blocks: mixing layer
+// (FP64 state) 4 of 256 131, 3 of 288 135; 352 FP32 blocks 43 and 42.
+template <int B, typename TS>
+struct RefineCfg {
+  using Bx = Box<2, B, 1>;
+  static constexpr int NT = B == 17 ? 128 : 256, MINB = B == 17 ? 8 : 4;
+  static constexpr int SCR = Bx::SCR > RefGeo<B>::NX ? Bx::SCR : RefGeo<B>::NX;
+  static constexpr size_t BYTES = kRingBytesD<2> + sizeof(TS) * (Bx::TILE + Bx::CBOX + SCR);
+};
+template <int B, typename TS>
+__global__ void __launch_bounds__(RefineCfg<B, TS>::NT, RefineCfg<B, TS>::MINB) k_refine(PoolView pv, TS* __restrict__ y) {
   pdl_enter();
   constexpr int D = 2;
   using Gm = Geo<D, B>;

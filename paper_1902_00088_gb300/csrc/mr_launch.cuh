@@ -43,7 +43,7 @@ constexpr int64_t kFusedScanMax = 65536;
 // (FP32), 564 (FP64); 384 82 and 593; 256 70 and 572.  Small grids, where a launch
 // is one wave, do not depend on it (76 blocks of 17^2 FP64: 33 us with 160 to 256).
 template <int B>
-struct Threads { static constexpr int value = B == 17 ? 160 : 288; };
+struct StageThreads { static constexpr int value = B == 17 ? 160 : 288; };
 
 template <int B, int RHS, typename TS, typename TY>
 static void stage_impl(const PoolView& pv, const Fields& f, int stage, const StageArgs& sa,
@@ -82,7 +82,7 @@ static void stage_impl(const PoolView& pv, const Fields& f, int stage, const Sta
         return run(stc, C32{}, std::integral_constant<int, 4>{});
       }
     }
-    run(stc, std::integral_constant<int, Threads<B>::value>{}, std::integral_constant<int, 1>{});
+    run(stc, std::integral_constant<int, StageThreads<B>::value>{}, std::integral_constant<int, 1>{});
   };
   switch (stage) {
     case 0: go(std::integral_constant<int, 0>{}); break;
@@ -192,10 +192,8 @@ struct RefineRun {
     if constexpr (D == 3) {
       go(k_refine3<TS>, Col3::NT, Refine3Smem<TS>::BYTES);
     } else {
-      constexpr int threads = Threads<B>::value;
-      using Bx = Box<2, B, 1>;
-      constexpr int scr = Bx::SCR > RefGeo<B>::NX ? Bx::SCR : RefGeo<B>::NX;
-      go(k_refine<B, TS, threads>, threads, kRingBytesD<2> + sizeof(TS) * (Bx::TILE + Bx::CBOX + scr));
+      using RC = RefineCfg<B, TS>;
+      go(k_refine<B, TS>, RC::NT, RC::BYTES);
     }
   }
 };

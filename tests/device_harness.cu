@@ -1,5 +1,6 @@
 // Launches single kernels of the library on hand-made blocks, for states that the
-// public calls cannot reach (an owner table without owners).  Built and called by
+// public calls cannot reach (an owner table without owners), and asks for what a
+// kernel's launch shape leaves resident.  Built and called by
 // tests/test_gpu_device_harness.py.
 #include <vector>
 
@@ -83,6 +84,16 @@ int ownerless(TS* y, int* err) {
   return ok;
 }
 
+template <int B, typename TS>
+int refine_occupancy() {
+  using RC = RefineCfg<B, TS>;
+  auto k = k_refine<B, TS>;
+  cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RC::BYTES);
+  int n = 0;
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k, RC::NT, RC::BYTES);
+  return n * RC::NT;
+}
+
 }  // namespace
 
 extern "C" {
@@ -100,6 +111,12 @@ int ownerless_stage(int dim, int form, int warp, void* y, int* err) {
                        : ownerless<2, double, float, 160, 1>(d, err);
   return form == 0 ? ownerless<3, double, double, 0, 0>(d, err) : form == 1 ? ownerless<3, float, float, 0, 0>(f, err)
                                                                 : ownerless<3, double, float, 0, 0>(d, err);
+}
+
+// threads per SM of the 2D refinement kernel
+int refine_threads_per_sm(int Bs, int fp64) {
+  if (Bs == 17) return fp64 ? refine_occupancy<17, double>() : refine_occupancy<17, float>();
+  return fp64 ? refine_occupancy<33, double>() : refine_occupancy<33, float>();
 }
 
 }  // extern "C"

@@ -46,3 +46,10 @@ def test_stage_leaves_edge_nodes_without_an_owner(lib, dim, warp, form):
     assert lib.ownerless_stage(dim, form, warp, y.ctypes.data_as(ctypes.c_void_p), ctypes.byref(err))
     assert err.value == ERR_GRADED
     np.testing.assert_array_equal(y, want)
+
+
+@pytest.mark.parametrize("fp64", [0, 1])
+@pytest.mark.parametrize("Bs", [17, 33])
+def test_refinement_keeps_a_thousand_threads_per_sm(lib, Bs, fp64):
+    # its launch shape is its own: with the stage's 160 threads an SM held 640 of them
+    assert lib.refine_threads_per_sm(Bs, fp64) >= 1024
