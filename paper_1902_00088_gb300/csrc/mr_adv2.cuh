@@ -146,13 +146,11 @@ __global__ void __launch_bounds__(GT * NW, GT == 32 ? 20 / NW : 1024 / GT) k_sta
       }
       tile[q] = to_tile<TC>(v);
     };
-    auto landed = [&]() {
+    auto landed = [&]() -> bool {
       if (!BULK) g.sync();
-      // bounded wait: a copy that never lands is reported, not waited for
-      if (BULK || staged) {
-        if (!mbar_wait(bar, phase, 1 << 20)) set_err(pv, kErrTimeout);
-        phase ^= 1;
-      }
+      if (!BULK && !staged) return true;
+      phase ^= 1;
+      return bulk_landed(pv, bar, phase ^ 1);
     };
     // ghost h: rows -2, -1, B, B + 1, then the pairs left and right of each row
     auto ghost = [](int h, int& i, int& j) {
@@ -187,7 +185,7 @@ __global__ void __launch_bounds__(GT * NW, GT == 32 ? 20 / NW : 1024 / GT) k_sta
         const int ex = NE && h < NG && i == B - 1 ? 2 : sx, ey = NE && h < NG && j == B - 1 ? 2 : sy;
         val[u] = src[nb[ex + 3 * ey] + (i - (ex - 1) * (B - 1)) + B * (j - (ey - 1) * (B - 1))];
       }
-      landed();
+      if (!landed()) return;
 #pragma unroll
       for (int u = 0; u < RN; ++u) {
         const int h = r + u * GT;
@@ -293,7 +291,7 @@ __global__ void __launch_bounds__(GT * NW, GT == 32 ? 20 / NW : 1024 / GT) k_sta
         }
         g.sync();
       }
-      landed();
+      if (!landed()) return;
 #pragma unroll
       for (int u = 0; u < RN; ++u) {
         const int h = r + u * GT;

@@ -435,8 +435,7 @@ __global__ void __launch_bounds__(Stage3Smem<TY, TS>::NT, 2) k_stage3(PoolView p
     __syncthreads();
     if (!uni) stage_rows();
     if (ROWS) {
-      // bounded wait: a copy that never lands is reported, not waited for
-      if (!mbar_wait(&bar, phase, 1 << 20)) set_err(pv, kErrTimeout);
+      if (!bulk_landed(pv, &bar, phase)) return;
       phase ^= 1;
     }
     const TreeDev& td = pv.trees[b.tree];

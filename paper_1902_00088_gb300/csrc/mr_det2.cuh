@@ -188,13 +188,13 @@ __global__ void __launch_bounds__(128, B == 17 ? 8 : 12) k_details2(PoolView pv,
       // none for integer roundings (16384 blocks of 4 variables 89 us instead of 113)
       for (int n = rank; n < NI; n += GS) S[n] = (TT)(me[n]);
     }
-    auto landed = [&]() {
+    auto landed = [&]() -> bool {
       if constexpr (BULK) {
-        // bounded wait: a copy that never lands is reported, not waited for
-        if (!mbar_wait(bar, phase, 1 << 20)) set_err(pv, kErrTimeout);
         phase ^= 1;
+        return bulk_landed(pv, bar, phase ^ 1);
       } else {
         g.sync();
+        return true;
       }
     };
     auto commit = [&](int n, TS v) {
@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(128, B == 17 ? 8 : 12) k_details2(PoolView pv,
         const int e = gtab[k];
         vg[u] = y[nbo[(e >> 12) & 15] + (e >> 16)];
       }
-      landed();
+      if (!landed()) return;
 #pragma unroll
       for (int u = 0; u < RE; ++u) {
         const int e = rank + u * GS;
@@ -280,7 +280,7 @@ __global__ void __launch_bounds__(128, B == 17 ? 8 : 12) k_details2(PoolView pv,
         lost |= !ok;
         vg[u] = ok ? y[owned(e, i, j)] : TS(0);
       }
-      landed();
+      if (!landed()) return;
 #pragma unroll
       for (int u = 0; u < RE; ++u) {
         if (!((other >> u) & 1)) continue;

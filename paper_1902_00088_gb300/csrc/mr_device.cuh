@@ -309,6 +309,21 @@ __device__ __forceinline__ void set_err(const PoolView& pv, int bits) {
   atomicOr(&pv.cnt->err, bits);
 }
 
+// Polls after which a wait for a bulk copy is given up (a test sets 0).
+#ifndef MR_WAIT_POLLS
+#define MR_WAIT_POLLS (1 << 20)
+#endif
+// Waits for the bulk copies of the mbarrier's phase.  A copy that does not land is
+// reported, not waited for without end: false, and the caller leaves the kernel (the
+// barrier's phase is still open, and its block has no values), after a second bounded
+// wait, so that no copy is in flight to shared memory that another CTA may get.
+__device__ __forceinline__ bool bulk_landed(const PoolView& pv, uint64_t* bar, unsigned parity) {
+  if (mbar_wait(bar, parity, MR_WAIT_POLLS)) return true;
+  set_err(pv, kErrTimeout);
+  mbar_wait(bar, parity, 1 << 20);
+  return false;
+}
+
 // Ring map: for every level-(l+1) cell q in [-1,2]^d around the block (its own
 // 2^d child cells included) the leaf covering it, searched at l+1, l, l-1,
 // with the leaf's origin relative to the block origin in level-(l+1) node

@@ -1,11 +1,12 @@
 // Launches single kernels of the library on hand-made blocks, for states that the
-// public calls cannot reach (an owner table without owners), and asks for what a
-// kernel's launch shape leaves resident.  Built and called by
+// public calls cannot reach (an owner table without owners, a wait that runs out), and
+// asks for what a kernel's launch shape leaves resident.  Built and called by
 // tests/test_gpu_device_harness.py.
 #include <vector>
 
 #include "mr_adv2.cuh"
 #include "mr_adv3.cuh"
+#include "mr_det2.cuh"
 
 using namespace mr;
 
@@ -84,6 +85,41 @@ int ownerless(TS* y, int* err) {
   return ok;
 }
 
+// One block at level 0, its own neighbour on every side.
+template <int D>
+std::vector<int32_t> periodic_plan() {
+  using PL = Plan<D>;
+  std::vector<int32_t> plan(PL::INTS, 0);
+  plan[1] = 1 << 30;  // level 0, tree 0, uniform
+  return plan;
+}
+// Runs stage ST (2D or 3D) or, with ST = -1, the 2D details on it; the block's fields
+// in f: y, accumulator, the field read, the field written.
+template <int D, int B, typename T, int GT, int NW, int ST>
+int periodic(T* f, double* md, int* err) {
+  OneBlock ob(D, B, 0, periodic_plan<D>(), std::vector<int4>(reg_entries(D), make_int4(-1, -1, 0, 0)));
+  const int n = (int)ob.pv.vs;
+  T* dev = ob.put(std::vector<T>(f, f + 4 * n));
+  T *y = dev, *acc = dev + n, *src = dev + 2 * n, *next = dev + 3 * n;
+  ob.pv.md = ob.put(std::vector<double>{*md});
+  ob.pv.bmax = ob.put(std::vector<double>{*md});
+  StageArgs sa{};
+  bool ok;
+  if constexpr (ST < 0) {
+    ok = launch(k_details2<B, T, T, T>, Det2<B>::NT, Det2Smem<B, T, T, T>::BYTES, ob.pv, y);
+  } else if constexpr (D == 2) {
+    ok = launch(k_stage2<B, MR_RHS_ADV, T, T, T, GT, NW, ST>, GT * NW, Stage2<B, T, T, GT, NW, ST>::BYTES, ob.pv,
+                (const T*)src, y, acc, next, 1, sa);
+  } else {
+    using SM = Stage3Smem<T, T>;
+    ok = launch(k_stage3<T, T, T, ST>, SM::NT, SM::BYTES, ob.pv, (const T*)src, y, acc, next, sa);
+  }
+  cudaMemcpy(f, dev, 4 * n * sizeof(T), cudaMemcpyDeviceToHost);
+  cudaMemcpy(md, ob.pv.md, sizeof(double), cudaMemcpyDeviceToHost);
+  *err = ob.err();
+  return ok;
+}
+
 template <int B, typename TS>
 int refine_occupancy() {
   using RC = RefineCfg<B, TS>;
@@ -111,6 +147,20 @@ int ownerless_stage(int dim, int form, int warp, void* y, int* err) {
                        : ownerless<2, double, float, 160, 1>(d, err);
   return form == 0 ? ownerless<3, double, double, 0, 0>(d, err) : form == 1 ? ownerless<3, float, float, 0, 0>(f, err)
                                                                 : ownerless<3, double, float, 0, 0>(d, err);
+}
+
+// kernels that wait for bulk copies; f: four fields of a block (see periodic)
+int periodic_block(int kernel, void* f, double* md, int* err) {
+  float* s = (float*)f;
+  double* d = (double*)f;
+  switch (kernel) {
+    case 0: return periodic<2, 17, float, 32, 4, 0>(s, md, err);
+    case 1: return periodic<2, 17, float, 160, 1, 1>(s, md, err);
+    case 2: return periodic<2, 33, double, 288, 1, 2>(d, md, err);
+    case 3: return periodic<3, 17, float, 0, 0, 1>(s, md, err);
+    case 4: return periodic<2, 17, float, 0, 0, -1>(s, md, err);
+    default: return periodic<2, 33, double, 0, 0, -1>(d, md, err);
+  }
 }
 
 // threads per SM of the 2D refinement kernel

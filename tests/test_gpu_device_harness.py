@@ -10,7 +10,7 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-ERR_GRADED = 2
+ERR_GRADED, ERR_TIMEOUT = 2, 16
 
 
 def build(path, *defines):
@@ -27,6 +27,14 @@ def lib(tmp_path_factory):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     return build(tmp_path_factory.mktemp("harness"))
+
+
+@pytest.fixture(scope="module")
+def lib_impatient(tmp_path_factory):
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return build(tmp_path_factory.mktemp("harness0"), "-DMR_WAIT_POLLS=0")
 
 
 def block(dim, form, seed):
@@ -53,3 +61,34 @@ def test_stage_leaves_edge_nodes_without_an_owner(lib, dim, warp, form):
 def test_refinement_keeps_a_thousand_threads_per_sm(lib, Bs, fp64):
     # its launch shape is its own: with the stage's 160 threads an SM held 640 of them
     assert lib.refine_threads_per_sm(Bs, fp64) >= 1024
+
+
+# kernel: dimension, block size, type; 4 and 5 are the details, the others stages
+PERIODIC = {0: (2, 17, np.float32), 1: (2, 17, np.float32), 2: (2, 33, np.float64), 3: (3, 17, np.float32),
+            4: (2, 17, np.float32), 5: (2, 33, np.float64)}
+
+
+def run_periodic(lib, kernel):
+    dim, B, dt = PERIODIC[kernel]
+    f = np.random.default_rng(4).standard_normal((4, (B ** dim + 3) // 4 * 4)).astype(dt)
+    before = f.copy()
+    md, err = ctypes.c_double(-1.0), ctypes.c_int(0)
+    assert lib.periodic_block(kernel, f.ctypes.data_as(ctypes.c_void_p), ctypes.byref(md), ctypes.byref(err))
+    return before, f, md.value, err.value
+
+
+@pytest.mark.parametrize("kernel", sorted(PERIODIC))
+def test_wait_that_runs_out(lib, lib_impatient, kernel):
+    # built to give up at once, the first wait for a block's bulk copies runs out (the
+    # copies land in the second one): the kernel reports it and leaves, and it stores
+    # nothing of the block whose values it does not have
+    before, after, md, err = run_periodic(lib_impatient, kernel)
+    assert err == ERR_TIMEOUT and md == -1.0
+    np.testing.assert_array_equal(before, after)
+    # the same launch with the library's limit
+    before, after, md, err = run_periodic(lib, kernel)
+    assert err == 0
+    if kernel >= 4:
+        assert md > 0.0
+    else:
+        assert not np.array_equal(before, after)
