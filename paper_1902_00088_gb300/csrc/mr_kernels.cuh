@@ -891,7 +891,9 @@ __global__ void __launch_bounds__(256) k_flags(PoolView pv) {
       const unsigned nans = __ballot_sync(0xffffffffu, nan);
       nan = (nans >> (4 * sis)) & 15u;
       if (nan) mb = 0x7ff8000000000000LL;
-      bool ok = sis >= NS || (t >= 0 && !nan && mb < __double_as_longlong(td.eps));
+      // on bit patterns, as eps > 0; nothing is below a threshold that is NaN
+      const long long eb = __double_as_longlong(td.eps);
+      bool ok = sis >= NS || (t >= 0 && !nan && mb < eb && eb <= 0x7ff0000000000000LL);
       const double m = __longlong_as_double(__shfl_sync(0xffffffffu, mb, 4 * own));
       // no finer leaf around the family: cells of [-1, 4]^d outside [0, 3]^d
       // (looked up only for a family whose members are all candidates)
