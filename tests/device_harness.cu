@@ -1,6 +1,7 @@
 // Launches single kernels of the library on hand-made blocks, for states that the
-// public calls cannot reach (an owner table without owners, a wait that runs out), and
-// asks for what a kernel's launch shape leaves resident.  Built and called by
+// public calls cannot reach (an owner table without owners, a wait that runs out), rounds
+// chosen values with the library's helpers, and asks for what a kernel's launch shape
+// leaves resident.  Built and called by
 // tests/test_gpu_device_harness.py.
 #include <vector>
 
@@ -120,6 +121,17 @@ int periodic(T* f, double* md, int* err) {
   return ok;
 }
 
+__global__ void k_round(const double* d, float* f, double* w, double* q, int n) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x) {
+    f[i] = f64_to_f32(d[i]);
+    w[i] = f32_to_f64(f[i]);
+    q[i] = sixteenth(d[i]);
+  }
+}
+__global__ void k_widen(const float* f, double* d, int n) {
+  for (int i = threadIdx.x; i < n; i += blockDim.x) d[i] = f32_to_f64(f[i]);
+}
+
 template <int B, typename TS>
 int refine_occupancy() {
   using RC = RefineCfg<B, TS>;
@@ -161,6 +173,27 @@ int periodic_block(int kernel, void* f, double* md, int* err) {
     case 4: return periodic<2, 17, float, 0, 0, -1>(s, md, err);
     default: return periodic<2, 33, double, 0, 0, -1>(d, md, err);
   }
+}
+
+// FP64 values d (n) rounded to FP32, widened again and divided by 16; FP32 values widened
+int round_values(int n, const double* d, float* f, double* w, double* q) {
+  OneBlock ob(2, 17, 0, {0}, {make_int4(0, 0, 0, 0)});
+  double* dd = ob.put(std::vector<double>(d, d + n));
+  float* df = ob.put(std::vector<float>(n));
+  double *dw = ob.put(std::vector<double>(n)), *dq = ob.put(std::vector<double>(n));
+  const bool ok = launch(k_round, 512, 0, (const double*)dd, df, dw, dq, n);
+  cudaMemcpy(f, df, n * 4, cudaMemcpyDeviceToHost);
+  cudaMemcpy(w, dw, n * 8, cudaMemcpyDeviceToHost);
+  cudaMemcpy(q, dq, n * 8, cudaMemcpyDeviceToHost);
+  return ok;
+}
+int widen_values(int n, const float* f, double* d) {
+  OneBlock ob(2, 17, 0, {0}, {make_int4(0, 0, 0, 0)});
+  float* df = ob.put(std::vector<float>(f, f + n));
+  double* dd = ob.put(std::vector<double>(n));
+  const bool ok = launch(k_widen, 512, 0, (const float*)df, dd, n);
+  cudaMemcpy(d, dd, n * 8, cudaMemcpyDeviceToHost);
+  return ok;
 }
 
 // threads per SM of the 2D refinement kernel

@@ -1,4 +1,5 @@
-"""Sums of the proposal network's gradients over many samples of one CTA."""
+"""The proposal network's training kernel with many samples per CTA: the error of the
+gradients' summation, and calls of every shape against the FP64 network."""
 import ctypes
 import math
 
@@ -64,3 +65,28 @@ def test_summation_error_over_the_samples_of_a_cta(mr, Bs, ctas):  # noqa: F811
     for a, b in zip(cnn.unpack(got), cnn.unpack(want)):
         if a.ndim == 4:
             assert np.linalg.norm(a - b) <= tol * np.linalg.norm(b), (a.shape, np.linalg.norm(a - b) / np.linalg.norm(b))
+
+
+@pytest.mark.parametrize("n", [1, 7, "several"])
+@pytest.mark.parametrize("Bs", [17, 33])
+def test_calls_of_every_shape_match_fp64_reference(mr, Bs, n):  # noqa: F811
+    # one sample (a CTA of a cluster has none), fewer than CTAs, and three or more for
+    # every CTA with an odd rest; five tiled samples, so that the reference is their
+    # weighted mean.  Bounds as for six samples of 25^2: FP32 arithmetic against FP64,
+    # probabilities to 1e-5, loss and gradient to 1e-4 of the gradient's scale
+    import torch
+    if n == "several":
+        n = 2 * 3 * torch.cuda.get_device_properties(0).multi_processor_count + 3
+    g = mr.Forest(dim=2, Bs=Bs, trees=[dict(Jmin=2, Jmax=4, ic="none")], capacity=1000)
+    theta, rng, T = weights(9), np.random.default_rng(4), Bs + 8
+    m = min(n, 5)
+    base, label = rng.standard_normal((m, 2, T, T)), np.array([1, 0, 1, 1, 0], np.float64)[:m]
+    of = np.arange(n) % m
+    share = np.bincount(of) / n
+    p, gr, loss = g.cnn_eval(theta, base[of], label[of], w_pos=W_POS)
+    pref = np.array([cnn.forward(theta, x)[0] for x in base])
+    ref = [cnn.loss_and_grad(theta, [x], [y], W_POS) for x, y in zip(base, label)]
+    L, gref = sum(a * r[0] for a, r in zip(share, ref)), sum(a * r[1] for a, r in zip(share, ref))
+    np.testing.assert_allclose(p, pref[of], rtol=0, atol=1e-5)
+    assert abs(loss - L) <= 1e-4 * max(1.0, abs(L))
+    assert np.abs(gr - gref).max() <= 1e-4 * np.abs(gref).max(), np.abs(gr - gref).max()

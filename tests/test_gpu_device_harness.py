@@ -1,5 +1,6 @@
 """Single kernels of the library on hand-made blocks (tests/device_harness.cu, built
-here): what a kernel does in states that no sequence of public calls reaches."""
+here): what a kernel does in states that no sequence of public calls reaches, and what
+the kernels' roundings on the integer pipes give at the ends of their formats."""
 import ctypes
 import os
 import subprocess
@@ -92,3 +93,44 @@ def test_wait_that_runs_out(lib, lib_impatient, kernel):
         assert md > 0.0
     else:
         assert not np.array_equal(before, after)
+
+
+def same(a, b):
+    # equal bits, or both NaN
+    u = np.uint32 if a.dtype == np.float32 else np.uint64
+    return (a.view(u) == b.view(u)) | (np.isnan(a) & np.isnan(b))
+
+
+def ptr(a):
+    return a.ctypes.data_as(ctypes.c_void_p)
+
+
+def fp64_patterns():
+    # every exponent with the mantissas next to every rounding boundary of FP32 results,
+    # normal (the low 29 bits) and subnormal (up to the whole mantissa), and random ones
+    m = {0, 1, (1 << 52) - 1}
+    for s in range(29, 53):
+        for k in (0, 1, 2, 3):
+            for d in (-1, 0, 1):
+                m.add(((k << s) + (1 << (s - 1)) + d) & ((1 << 52) - 1))
+    m = np.array(sorted(m) + list(np.random.default_rng(1).integers(0, 1 << 52, 64)), np.uint64)
+    e = np.arange(2048, dtype=np.uint64) << np.uint64(52)
+    u = (e[:, None] | m[None, :]).ravel()
+    return np.concatenate([u, u | np.uint64(1 << 63)]).view(np.float64)
+
+
+def test_roundings_are_the_conversions(lib):
+    d = fp64_patterns()
+    f, w, q = np.empty(len(d), np.float32), np.empty(len(d)), np.empty(len(d))
+    assert lib.round_values(len(d), ptr(d), ptr(f), ptr(w), ptr(q))
+    with np.errstate(all="ignore"):
+        assert same(f, d.astype(np.float32)).all()
+        assert same(w, f.astype(np.float64)).all()
+        assert same(q, d / 16.0).all()
+    m = np.concatenate([[0, 1, 2, 3, (1 << 23) - 1], 1 << np.arange(23), np.random.default_rng(2).integers(0, 1 << 23, 200)])
+    u = ((np.arange(512) << 23)[:, None] | m[None, :]).ravel().astype(np.uint32)
+    f = u.view(np.float32)
+    d = np.empty(len(f))
+    assert lib.widen_values(len(f), ptr(f), ptr(d))
+    with np.errstate(all="ignore"):
+        assert same(d, f.astype(np.float64)).all()
