@@ -321,8 +321,9 @@ mr_status mr_get_step_history(mr_ctx ctx, int64_t cap, int32_t* out, int64_t* n,
  * accumulator rows staged by bulk copies or loaded (steps steps each; the
  * solution advances during tuning) and keeps the fastest; *best = CTAs per SM
  * (0 = occupancy) + 100 x form + 1000 x blocks per CTA + 10000 x staging.
- * Without tuning the 2D stage on 17^2 blocks uses one warp per block once the
- * grid holds at least 8 blocks per SM, 4 blocks per CTA, rows staged.
+ * Without tuning the 2D stage on 17^2 advection blocks uses one warp per block once
+ * the grid holds at least 8 blocks per SM (32 with FP64 states), 4 blocks per CTA,
+ * rows staged.
  * Synchronises. */
 mr_status mr_autotune(mr_ctx ctx, int32_t steps, int32_t* best);
 /* Fixes the launch configuration instead of the autotuner: ctas_per_sm
@@ -333,10 +334,10 @@ mr_status mr_autotune(mr_ctx ctx, int32_t steps, int32_t* best);
  * not depend on either choice.  MR_EINVAL for values out of range or the warp
  * form where it does not exist.  Drops the captured step. */
 mr_status mr_set_tuning(mr_ctx ctx, int32_t ctas_per_sm, int32_t stage_form);
-/* Warp-per-block form of the 2D stage on FP32 fields: blocks_per_cta (2, 4 or
- * 8 warps per CTA, one block each) and staging (1: the state and accumulator
- * rows of a block are copied to shared memory by the bulk-copy engine while
- * its ghost layer is gathered; 0: loaded by the threads).  Results do not
+/* 2D advection stage on FP32 fields: blocks_per_cta of the warp-per-block form (2, 4
+ * or 8 warps per CTA, one block each) and, in either form, staging (1: the state and
+ * accumulator rows of a block are copied to shared memory by the bulk-copy engine
+ * while its ghost layer is gathered; 0: loaded by the threads).  Results do not
  * depend on either.  MR_EINVAL for other values.  Drops the captured step. */
 mr_status mr_set_warp_form(mr_ctx ctx, int32_t blocks_per_cta, int32_t staging);
 /* Synchronises; accumulates pending timers into *out. */

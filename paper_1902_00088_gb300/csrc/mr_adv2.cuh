@@ -56,8 +56,10 @@ struct Stage2 {
 // 62 us per launch on 65536 blocks of 17^2 (FP32, one warp per block), where the
 // five arrays of stages 1 and 2 alone take 58; 89 with the whole tile of width 2
 // gathered node by node.  7472 blocks of an adapted forest: 19 us, 36 before.
-// Warps per SM for one warp per block: 20 (96 registers, nothing spilled) 62 us,
-// 16 65, 24 64, 28 70, 32 (64 registers, 150 bytes spilled) 73.
+// Warps per SM for one warp per block, FP32 advection: 20 (96 registers, nothing
+// spilled) 62 us, 16 65, 24 64, 28 70, 32 (64 registers, 150 bytes spilled) 73.  At 20
+// the FP32 swirl spills 8 to 16 bytes and the FP64 states, bound by the FP64 pipe, up
+// to 100.
 template <int B, int RHS, typename TS, typename TY, typename TSRC, int GT, int NW, int ST>
 __global__ void __launch_bounds__(GT * NW, GT == 32 ? 20 / NW : 1024 / GT) k_stage2(PoolView pv, const TSRC* __restrict__ src,
                                                                      TS* __restrict__ y, TS* __restrict__ acc,

@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(Stage3Smem<TY, TS>::NT, 2) k_stage3(PoolView p
       const int fm = sface;
       if (fm) {
         // Prediction of the face layers: x first, then y, then z (the order of
-        // coarse_passes), each face from a patch of 4 coarse nodes across it
+        // predict_box), each face from a patch of 4 coarse nodes across it
         // and 11 x 11 along it.  n0: first coarse node across the face.  The
         // passes take the odd nodes (4 products and sums) before the even ones
         // (copies), so that their warps hold one kind.
@@ -997,7 +997,7 @@ __global__ void __launch_bounds__(Col3::NT, sizeof(TS) == 8 ? 2 : 3) k_refine3(P
         }
         cp_async_wait_all();
         __syncthreads();
-        // x, then y (then z at the node): the order of coarse_passes
+        // x, then y (then z at the node): the order of predict_box
         const int ex = hi[0] - lo[0] + 1, ey = nhi[1] - nlo[1] + 1, ez = nhi[2] - nlo[2] + 1, fyn = hi[1] - lo[1] + 1;
         for (int q = t; q < ex * ey * ez; q += NT) {
           const int xx = q % ex + lo[0], ny = (q / ex) % ey + nlo[1] - ky0, nz = q / (ex * ey) + nlo[2] + 2;

@@ -148,13 +148,11 @@ __device__ __forceinline__ const T* committed(const T* y, const void* src) {
 
 // Thread groups that cooperate on one block: the whole CTA, or one warp.
 struct CtaGroup {
-  static constexpr int kSize = 0;  // size known at run time only
   __device__ __forceinline__ int rank() const { return threadIdx.x; }
   __device__ __forceinline__ int size() const { return blockDim.x; }
   __device__ __forceinline__ void sync() const { __syncthreads(); }
 };
 struct WarpGroup {
-  static constexpr int kSize = 32;
   __device__ __forceinline__ int rank() const { return threadIdx.x & 31; }
   __device__ __forceinline__ int size() const { return 32; }
   __device__ __forceinline__ void sync() const { __syncwarp(); }
@@ -275,14 +273,8 @@ struct Box {
   static constexpr int CLO = -((W + 1) / 2) - 1;
   static constexpr int CB = (B - 1) / 2 + 2 * ((W + 1) / 2) + 3;
   static constexpr int CBOX = CB * CB * (D == 3 ? CB : 1);
-  // scratch of the separable prediction, per variable: X[nz][ny][x] (coarse
-  // y, z; fine x) and, in 3D, Y[nz][y][x] (coarse z; fine x, y).  In 3D X is
-  // kept in the variable's tile, which is written only after the y pass, so
-  // the scratch holds Y alone.
-  static constexpr int NXP = (D == 3 ? CB : 1) * CB * S;
-  static constexpr int NYP = D == 3 ? CB * S * S : 0;
-  static constexpr int SCR = D == 3 ? NYP : NXP;
-  static_assert(D == 2 || NXP <= TILE, "the x pass fits in the tile");
+  // scratch of the separable prediction (2D), per variable: X[ny][x] (coarse y, fine x)
+  static constexpr int SCR = CB * S;
   __device__ static __forceinline__ int cix(int i, int j, int k) {
     return ((D == 3 ? k - CLO : 0) * CB + (j - CLO)) * CB + (i - CLO);
   }
@@ -532,13 +524,6 @@ __device__ __forceinline__ T dd4(T fm1, T f0, T f1, T f2) {
   return sixteenth(T(9) * (f0 + f1) - (fm1 + f2));
 }
 
-// Value of node `li` (local index at the owner's level) of variable v.
-template <int D, int B, typename TF>
-__device__ __forceinline__ TF pool_at(const PoolView& pv, const TF* F, int slot, int v,
-                                      const int li[3]) {
-  return F[((int64_t)slot * pv.nvar + v) * pv.vs + Geo<D, B>::lin(li[0], li[1], D == 3 ? li[2] : 0)];
-}
-
 // Coarse-lattice prediction at half-coarse position o (relative to the block
 // origin) from the staged coarse box: x first, then y, then z.
 template <int D, int B, int W, typename TT>
@@ -662,49 +647,26 @@ struct PredBox {
   }
 };
 
-// Separable prediction over the coarse box (values of nv variables in cbox),
-// x first, then y (then z at the point): the same operations in the same order
-// as predict_box, evaluated only where the predicted nodes of pb need them.
-// 2D: the x pass goes to scr (y per point from it); 3D: the x pass is kept in
-// the variable's tile (overwritten later by the gather) and the y pass goes to
-// scr (z per point).  Ends with a group barrier.
-template <int D, int B, int W, typename TT, typename G>
-__device__ void coarse_passes(int nv, const TT* cbox, TT* tile, TT* scr, const PredBox<B, W>& pb) {
+// Separable prediction over the 2D coarse box (values of nv variables in cbox), x
+// first, then y: the same operations in the same order as predict_box, evaluated only
+// where the predicted nodes of pb need them.  The x pass goes to scr (y per point from
+// it).  Ends with a group barrier.
+template <int B, int W, typename TT, typename G>
+__device__ void coarse_passes(int nv, const TT* cbox, TT* scr, const PredBox<B, W>& pb) {
   const G g{};
-  using Bx = Box<D, B, W>;
-  // x pass: x in [lo0, hi0], coarse rows ny in [nlo1, nhi1], nz in [nlo2, nhi2]
+  using Bx = Box<2, B, W>;
+  // x in [lo0, hi0], coarse rows ny in [nlo1, nhi1]
   const int ex = pb.hi[0] - pb.lo[0] + 1, ey = pb.nhi[1] - pb.nlo[1] + 1;
-  const int nxp = ex * ey * (D == 3 ? pb.nhi[2] - pb.nlo[2] + 1 : 1);
   for (int v = 0; v < nv; ++v) {
     const TT* cb = cbox + v * Bx::CBOX;
-    TT* X = D == 3 ? tile + v * Bx::TILE : scr + v * Bx::SCR;
-    for (int q = g.rank(); q < nxp; q += g.size()) {
+    TT* X = scr + v * Bx::SCR;
+    for (int q = g.rank(); q < ex * ey; q += g.size()) {
       const int x = q % ex + pb.lo[0], ny = (q / ex) % ey + pb.nlo[1];
-      const int nz = D == 3 ? q / (ex * ey) + pb.nlo[2] : 0;
       const int fl = x >> 1;
-      const int at = ((D == 3 ? nz - Bx::CLO : 0) * Bx::CB + (ny - Bx::CLO)) * Bx::S + (x + W);
-      X[at] = (x & 1) ? dd4(cb[Bx::cix(fl - 1, ny, nz)], cb[Bx::cix(fl, ny, nz)], cb[Bx::cix(fl + 1, ny, nz)],
-                            cb[Bx::cix(fl + 2, ny, nz)])
-                      : cb[Bx::cix(fl, ny, nz)];
-    }
-  }
-  if (D == 3) {
-    g.sync();
-    // y pass: x in [lo0, hi0], y in [lo1, hi1], coarse nz in [nlo2, nhi2]
-    const int fy = pb.hi[1] - pb.lo[1] + 1;
-    const int nyp = ex * fy * (pb.nhi[2] - pb.nlo[2] + 1);
-    for (int v = 0; v < nv; ++v) {
-      const TT* X = tile + v * Bx::TILE;
-      TT* Y = scr + v * Bx::SCR;
-      for (int q = g.rank(); q < nyp; q += g.size()) {
-        const int x = q % ex + pb.lo[0] + W, y = (q / ex) % fy + pb.lo[1];
-        const int nzi = q / (ex * fy) + pb.nlo[2] - Bx::CLO;
-        const int fl = y >> 1;
-        const TT* c = X + nzi * Bx::CB * Bx::S + x;
-        Y[(nzi * Bx::S + (y + W)) * Bx::S + x] = (y & 1) ? dd4(c[(fl - 1 - Bx::CLO) * Bx::S], c[(fl - Bx::CLO) * Bx::S],
-                                                               c[(fl + 1 - Bx::CLO) * Bx::S], c[(fl + 2 - Bx::CLO) * Bx::S])
-                                                         : c[(fl - Bx::CLO) * Bx::S];
-      }
+      const int at = (ny - Bx::CLO) * Bx::S + (x + W);
+      X[at] = (x & 1) ? dd4(cb[Bx::cix(fl - 1, ny, 0)], cb[Bx::cix(fl, ny, 0)], cb[Bx::cix(fl + 1, ny, 0)],
+                            cb[Bx::cix(fl + 2, ny, 0)])
+                      : cb[Bx::cix(fl, ny, 0)];
     }
   }
   g.sync();
@@ -717,7 +679,8 @@ __device__ void coarse_passes(int nv, const TT* cbox, TT* tile, TT* scr, const P
 // they are also written back into F when they differ.  cbox: scratch
 // of nvar x CBOX values for the coarse lattice (used when a coarser leaf
 // touches the block): every coarse node takes its owner's value, and ghost
-// nodes between coarse nodes are predicted from it.
+// nodes between coarse nodes are predicted from it, in 2D in separable passes over
+// scr (nvar x SCR values) if given, else node by node.
 // ES: tile layout, 1 = variable after variable, 4 = the four variables of a node
 // side by side.
 template <int D, int B, typename TF, typename TT, int W = kG, typename G = CtaGroup, int ES = 1>
@@ -839,7 +802,9 @@ __device__ void fill_tile(const PoolView& pv, const BlockInfo& b, const TF* F, T
       }
     }
     g.sync();
-    if (scr) coarse_passes<D, B, W, TT, G>(nv, cbox, tile, scr, pb);
+    if constexpr (D == 2) {
+      if (scr) coarse_passes<B, W, TT, G>(nv, cbox, scr, pb);
+    }
   }
   // kinds of tile points: 0 own node, 1 block-edge node of another owner,
   // 2 ghost node that is a node of its owner, 3 ghost predicted from the coarse
@@ -911,12 +876,11 @@ __device__ void fill_tile(const PoolView& pv, const BlockInfo& b, const TF* F, T
         if (kind[u] == 5) continue;
         TT* t = tile + at_tile(v, idx[u]);
         if (kind[u] == 3) {
-          if (scr) {
-            // last axis from the scratch: z in 3D (Y), y in 2D (X)
-            const TT* c = scr + v * Bx::SCR + (ijk[u][0] + W) +
-                          (D == 3 ? (ijk[u][1] + W) * Bx::S : 0);
-            const int st = D == 3 ? Bx::S * Bx::S : Bx::S;
-            const int e = ijk[u][D - 1], fl = e >> 1;
+          if (D == 2 && scr) {
+            // y from the scratch (X)
+            const TT* c = scr + v * Bx::SCR + (ijk[u][0] + W);
+            constexpr int st = Bx::S;
+            const int e = ijk[u][1], fl = e >> 1;
             *t = (e & 1) ? dd4(c[(fl - 1 - Bx::CLO) * st], c[(fl - Bx::CLO) * st], c[(fl + 1 - Bx::CLO) * st],
                                c[(fl + 2 - Bx::CLO) * st])
                          : c[(fl - Bx::CLO) * st];

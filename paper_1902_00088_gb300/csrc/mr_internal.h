@@ -174,7 +174,7 @@ struct LaunchCfg {
   int n_hint;      // block count last read by the host (chooses the form when -1)
   int pdl;         // step kernels use programmatic dependent launch (launch_k)
   int warp_blocks; // 2D warp-per-block stage on FP32 fields: blocks (warps) per CTA, 2, 4 or 8
-  int staging;     // ... and whether its state/accumulator rows are staged by bulk copies (1) or loaded (0)
+  int staging;     // 2D stage on FP32 fields, either form: state/accumulator rows by bulk copies (1) or loads (0)
 };
 
 #ifdef __CUDACC__

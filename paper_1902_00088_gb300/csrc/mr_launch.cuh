@@ -201,7 +201,6 @@ struct RefineRun {
 template <int D>
 void launch_refine(const PoolView& pv, const Fields& f, int mode, const int8_t* mask,
                    const LaunchCfg& lc, cudaStream_t st) {
-  const int nch = 1 << D;
   // short lists: the counting kernel's last CTA scans them (no scan launch)
   if (2 * (int64_t)lc.n_hint <= kFusedScanMax) {
     const int grid = std::min(flat_grid(pv, 256), std::max(lc.num_sms, (2 * lc.n_hint + 255) / 256));
@@ -216,7 +215,6 @@ void launch_refine(const PoolView& pv, const Fields& f, int mode, const int8_t* 
   dispatch_bs<D, RefineRun>(pv, f, lc, st);
   launch_k(lc.pdl, k_refine_commit<D>, flat_grid(pv, 256), 256, 0, st, pv);
   count_launch(1);
-  (void)nch;
 }
 
 // ------------------------------------------------------------------- IC ------
@@ -305,7 +303,6 @@ void launch_round_merge(const PoolView& pv, const Fields& f, bool merge, const R
                  4 * (int64_t)lc.n_hint / 8, lc.pdl != 0, 3);
   }
   dispatch_bs<D, CoarsenRun>(pv, f, rc, lc, st);
-  (void)nch;
 }
 
 template <int D>
