@@ -101,16 +101,19 @@ WORKLOADS = {
 
 # DRAM traffic per launch (dram__bytes_read.sum + dram__bytes_write.sum), averaged
 # over the launches of one step (the four RK stages; the details of the
-# coarsening rounds; the filter), from an ncu capture per workload (profiles/),
-# valid only for the device sources it was taken on (the digest in each entry);
-# otherwise reported as null.
+# coarsening rounds; the filter), from an ncu capture per workload
+# (profiles/traffic.md), valid only for the device sources it was taken on (the
+# digest in each entry) and a grid of its size (blocks per stage launch, within
+# 5 %); otherwise reported as null.
 TRAFFIC = {
     # workload: {kernel: DRAM bytes per launch}, plus the digest of the device sources it was taken on
-    "adv3d": {"digest": ("DEVICE", "1001c46c9ab0dc4b"), "stage": (36.01e6 + 99.01e6 + 98.98e6 + 60.53e6) / 4,
-              "details": (32.93e6 + 6.51e6 + 7.59e6 + 2.80e6) / 4},
-    "dsl": {"digest": ("NS", "2a19634679daf7a6"), "stage": (279.74e6 + 336.89e6 + 336.16e6 + 289.24e6) / 4,
-            "details": (113.75e6 + 11.25e6 + 4.95e6 + 2.66e6) / 4,
-            "filter": 71.71e6},
+    "adv3d": {"digest": ("DEVICE", "efbcf082809e55a9"), "blocks": 1408,
+              "stage": (39.51e6 + 100.23e6 + 100.21e6 + 62.30e6) / 4,
+              "details": (32.89e6 + 5.81e6 + 6.83e6 + 2.69e6) / 4},
+    "dsl": {"digest": ("NS", "4d600f034aabd6ef"), "blocks": 11776,
+            "stage": (285.56e6 + 340.05e6 + 339.94e6 + 292.11e6) / 4,
+            "details": (112.10e6 + 10.02e6 + 4.54e6 + 2.52e6) / 4,
+            "filter": 72.05e6},
 }
 
 
@@ -863,7 +866,9 @@ def main():
     twl = TRAFFIC.get(args.workload, {})
     tr = twl.get(dom)
     dig_ok = bool(twl) and source_digest(NS_SOURCES if twl["digest"][0] == "NS" else DEVICE_SOURCES) == twl["digest"][1]
-    if tr and dig_ok and not args.precision and not args.learned:
+    per_launch = kern["stage"]["blocks"] / max(1, kern["stage"]["launches"])
+    same_grid = abs(per_launch - twl.get("blocks", 0)) <= 0.05 * per_launch
+    if tr and dig_ok and same_grid and not args.precision and not args.learned:
         traffic = tr
         traffic_note = {"kernel": kern[dom]["kernel"],
                         "algorithmic_bytes_per_launch": kern[dom]["bytes"] / max(1, kern[dom]["launches"]),
